@@ -422,7 +422,7 @@ __device__ __forceinline__ float interface_weight(const float rho[2], float2 cbu
 
 // Densities and total momentum of one site's gathered populations, summed in one
 // fixed order (the mass sums and the correction must see the same values).
-__device__ __forceinline__ void site_moments(const float f[2][9], float rho[2], float& jx, float& jy) {
+__device__ __forceinline__ void site_moments(const float2 f[9], float rho[2], float& jx, float& jy) {
     jx = 0.0f;
     jy = 0.0f;
 #pragma unroll
@@ -430,9 +430,10 @@ __device__ __forceinline__ void site_moments(const float f[2][9], float rho[2], 
         float r = 0.0f;
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
-            r += f[s][i];
-            jx += cx(i) * f[s][i];
-            jy += cy(i) * f[s][i];
+            const float v = s == 0 ? f[i].x : f[i].y;
+            r += v;
+            jx += cx(i) * v;
+            jy += cy(i) * v;
         }
         rho[s] = r;
     }
@@ -441,16 +442,16 @@ __device__ __forceinline__ void site_moments(const float f[2][9], float rho[2], 
 // Pass 1 of a correction: the densities rho2 [2][n] and total momenta j2 [2][n] of the
 // coarse run's populations after streaming (FP32 storage), gathered as the step
 // kernels pull them.
-__global__ void __launch_bounds__(128) closure_moments_kernel(const float* __restrict__ fin, Grid g,
+__global__ void __launch_bounds__(128) closure_moments_kernel(const float2* __restrict__ fin, Grid g,
                                                               float* __restrict__ rho2, float* __restrict__ j2) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y;
     if (x >= g.nx) return;
-    const float zero[2] = {0.0f, 0.0f};
     const int xm = x == 0 ? g.nx - 1 : x - 1;
     const int xp = x == g.nx - 1 ? 0 : x + 1;
-    float f[2][9], rho[2], jx, jy;
-    pull_site<float>(fin, g, zero, y, x, xm, xp, f);
+    float2 f[9];
+    float rho[2], jx, jy;
+    pull_site<float>(fin, g, splat(0.0f), y, x, xm, xp, f);
     site_moments(f, rho, jx, jy);
     const size_t n = (size_t)g.nx * g.ny, k = (size_t)y * g.nx + x;
     rho2[k] = rho[0];
@@ -543,7 +544,7 @@ __global__ void __launch_bounds__(256) drho_total_kernel(double* __restrict__ pa
 // du_x, du_y); hw = sum(h) / sum(w) (mode 4), mA / mB the mean corrections (modes
 // 1-3).  FP32: the corrections are small next to the populations, and the mass sums
 // are FP64.
-__device__ __forceinline__ void correct_site(float f[2][9], float4 p, int mode, float2 cbulk, float hw, float mA,
+__device__ __forceinline__ void correct_site(float2 f[9], float4 p, int mode, float2 cbulk, float hw, float mA,
                                              float mB) {
     // mode 2 keeps the velocity; modes 3 and 4 relax it a quarter of the way (the
     // full correction of mode 1 feeds back into the growing coarse modes)
@@ -565,18 +566,20 @@ __device__ __forceinline__ void correct_site(float f[2][9], float4 p, int mode, 
         d[1] -= mB;
     }
     const float du2 = 1.5f * ((vx * vx + vy * vy) - (ux * ux + uy * uy));
+    // an absent component keeps its populations: q = 1, r1 = 0
+    float q[2], r1[2];
 #pragma unroll
     for (int s = 0; s < 2; ++s) {
-        const float r0 = rho[s];
-        if (!(r0 > 0.0f)) continue;
-        const float r1 = fmaxf(r0 + d[s], 0.0f);
-        const float q = r1 / r0;
+        const bool present = rho[s] > 0.0f;
+        r1[s] = present ? fmaxf(rho[s] + d[s], 0.0f) : 0.0f;
+        q[s] = present ? r1[s] / rho[s] : 1.0f;
+    }
+    const float2 q2 = make_float2(q[0], q[1]), r2 = make_float2(r1[0], r1[1]);
 #pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            const float c0 = cx(i) * ux + cy(i) * uy, c1 = cx(i) * vx + cy(i) * vy;
-            const float dc = c1 - c0;
-            f[s][i] = q * f[s][i] + wf(i) * r1 * (3.0f * dc + 4.5f * dc * (c1 + c0) - du2);
-        }
+    for (int i = 0; i < 9; ++i) {
+        const float c0 = cx(i) * ux + cy(i) * uy, c1 = cx(i) * vx + cy(i) * vy;
+        const float dc = c1 - c0;
+        f[i] = fma2(q2, f[i], mul2(r2, splat(wf(i) * (3.0f * dc + 4.5f * dc * (c1 + c0) - du2))));
     }
 }
 
@@ -587,10 +590,10 @@ __device__ __forceinline__ void correct_site(float f[2][9], float4 p, int mode, 
 // wall row), corrects them (correct_site) and writes them back to the same slots,
 // with the periodic ghost copy of columns 0, 1, nx - 2, nx - 1 that the staged
 // kernels' row windows read.  Every stored slot belongs to exactly one (site,
-// direction) pair, so no two threads touch the same slot; a thread's 18 loads
+// direction) pair, so no two threads touch the same slot; a thread's 9 loads
 // precede its stores through one pointer.  scalars: sum(h) / sum(w) (mode 4) and the
 // mean corrections (modes 1-3), from drho_total_kernel.
-__global__ void __launch_bounds__(128, 7) correct_inplace_kernel(float* pops, Grid g, const float* __restrict__ y,
+__global__ void __launch_bounds__(128, 7) correct_inplace_kernel(float2* pops, Grid g, const float* __restrict__ y,
                                                               float4 oscale, int mode, float2 cbulk,
                                                               const float* __restrict__ scalars) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -601,22 +604,20 @@ __global__ void __launch_bounds__(128, 7) correct_inplace_kernel(float* pops, Gr
     const int dxe = x == g.nx - 1 ? 1 - g.nx : 1;
     const bool bottom = row == 0, top = row == g.ny - 1;
     const ptrdiff_t plane = (ptrdiff_t)g.plane, pitch = g.pitch;
-    float* const site = pops + (ptrdiff_t)row * pitch + g.origin + x;
-    // slot of direction i of component s, and the slot's column offset from x
-    auto slot = [&](int s, int i, int* dcol) -> float* {
+    float2* const site = pops + (ptrdiff_t)row * pitch + g.origin + x;
+    // slot of direction i (both components), and the slot's column offset from x
+    auto slot = [&](int i, int* dcol) -> float2* {
         if ((cy(i) == 1 && bottom) || (cy(i) == -1 && top)) {
             *dcol = 0;
-            return site + (s * 9 + opp(i)) * plane;
+            return site + opp(i) * plane;
         }
         *dcol = cx(i) == 0 ? 0 : (cx(i) == 1 ? dxw : dxe);
-        return site + (s * 9 + i) * plane - cy(i) * pitch + *dcol;
+        return site + i * plane - cy(i) * pitch + *dcol;
     };
-    float f[2][9];
+    float2 f[9];
     int dcol;
 #pragma unroll
-    for (int s = 0; s < 2; ++s)
-#pragma unroll
-        for (int i = 0; i < 9; ++i) f[s][i] = *slot(s, i, &dcol);
+    for (int i = 0; i < 9; ++i) f[i] = *slot(i, &dcol);
     const size_t n = (size_t)g.nx * g.ny, k = (size_t)row * g.nx + x;
     const float4 p = make_float4(y[k] * oscale.x, y[n + k] * oscale.y, y[2 * n + k] * oscale.z,
                                  y[3 * n + k] * oscale.w);
@@ -625,17 +626,15 @@ __global__ void __launch_bounds__(128, 7) correct_inplace_kernel(float* pops, Gr
     // slot in columns 0, 1, nx - 2, nx - 1
     const bool edge = x < 3 || x >= g.nx - 3;
 #pragma unroll
-    for (int s = 0; s < 2; ++s)
-#pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            float* q = slot(s, i, &dcol);
-            *q = f[s][i];
-            if (edge) {
-                const int col = x + dcol;
-                if (col < 2) q[g.nx] = f[s][i];
-                else if (col >= g.nx - 2) q[-g.nx] = f[s][i];
-            }
+    for (int i = 0; i < 9; ++i) {
+        float2* q = slot(i, &dcol);
+        *q = f[i];
+        if (edge) {
+            const int col = x + dcol;
+            if (col < 2) q[g.nx] = f[i];
+            else if (col >= g.nx - 2) q[-g.nx] = f[i];
         }
+    }
 }
 
 }  // namespace
@@ -752,7 +751,7 @@ lbm_status correct(lbm_closure* c, int mode, bool clear_status) {
                                        q.minority * q.mass_A / (q.minority * q.mass_A + q.mass_B));
     const lbm::PopView v = lbm::handle_pops(c->coarse);
     if (v.storage != LBM_STORE_F32) return cl_fail(LBM_ESTATE, "the closure's coarse run must store FP32");
-    float* pops = static_cast<float*>(v.pops);
+    float2* pops = static_cast<float2*>(v.pops);
     // raw holds the densities (first half) and the momenta (second half)
     float* rho2 = c->raw;
     float* j2 = c->raw + 2 * c->nc;

@@ -159,18 +159,21 @@ struct Acc {
 };
 
 template <typename T>
-__global__ void __launch_bounds__(DX * DY) moments_kernel(const T* __restrict__ fin, DiagArgs a, float sA, float sB) {
+__global__ void __launch_bounds__(DX * DY) moments_kernel(const Cell<T>* __restrict__ fin, DiagArgs a,
+                                                         float sA, float sB) {
     const int x = blockIdx.x * DX + threadIdx.x;
     dfl v[2] = {{0.0f, 0.0f}, {0.0f, 0.0f}};
 #pragma unroll 1
     for (int r = 0; r < RY; ++r) {
         const int y = row_of(r);
         if (x >= a.nx || y >= a.ny) break;
-        const float shift[2] = {sA, sB};
         // the columns beside the grid from the ghost columns (periodic copies, or a
         // split grid's neighbours)
+        float2 fp[9];
+        pull_site<T>(fin, a.g, make_float2(sA, sB), y, x, x - 1, x + 1, fp);
         float f[2][9];
-        pull_site<T>(fin, a.g, shift, y, x, x - 1, x + 1, f);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) { f[0][i] = fp[i].x; f[1][i] = fp[i].y; }
         dfl rho[2], jx[2], jy[2];
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
@@ -439,7 +442,7 @@ DiagArgs make_args(const DiagLaunch& D) {
 template <typename T>
 cudaError_t launch_moments(const DiagLaunch& D, const DiagArgs& a, cudaStream_t st) {
     dim3 grid(a.nbx, (a.ny + BY - 1) / BY), block(DX, DY);
-    moments_kernel<T><<<grid, block, 0, st>>>((const T*)D.fin, a, D.shift[0], D.shift[1]);
+    moments_kernel<T><<<grid, block, 0, st>>>((const Cell<T>*)D.fin, a, D.shift[0], D.shift[1]);
     return cudaGetLastError();
 }
 

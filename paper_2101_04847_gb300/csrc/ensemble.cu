@@ -33,8 +33,7 @@ struct lbm_ensemble {
     std::vector<lbm::EnsMember> table;
     lbm::EnsMember* d_table = nullptr;
     int total_tiles = 0;
-    int tile_x = lbm::kEnsPaired;    // 128 or 256 columns per tile (one per thread), or
-                                     // kEnsPaired (FP32 128 columns, 16-bit paired 256)
+    int tile_x = lbm::kEnsAuto;      // 128 or 256 columns per tile (one per thread), or kEnsAuto
     int tile_y = 0;       // requested rows per tile; 0: chosen from the device's block slots
     int rows = 0;         // rows per tile in use
     size_t smem = 0;      // dynamic shared memory per block (largest storage type present)
@@ -195,7 +194,7 @@ lbm_status lbm_ens_create(int32_t n, const lbm_params* params, void* cuda_stream
     }
     e->tile_y = params[0].tile_y > 0 ? params[0].tile_y : 0;
     e->tile_x = params[0].tile_x == lbm::kWideTileW || params[0].tile_x == lbm::kBlockTileW ? params[0].tile_x
-                                                                                             : lbm::kEnsPaired;
+                                                                                             : lbm::kEnsAuto;
     for (int i = 0; i < n; ++i) {
         lbm_params p = params[i];
         p.kernel = LBM_KERNEL_STAGED;
@@ -274,7 +273,7 @@ lbm_status lbm_ens_diagnostics(lbm_ensemble* e, lbm_diag* out) {
 lbm_status lbm_ens_tune(lbm_ensemble* e, int32_t* tile_y_out, double* ms_out) {
     if (!e) return ens_fail(LBM_EINVAL, "ensemble is NULL");
     const int cand[] = {0, 12, 16, 20, 24, 32, 48, 64, 96};   // 0: the slot-filling default
-    const int widths[] = {lbm::kEnsPaired, lbm::kBlockTileW, lbm::kWideTileW};
+    const int widths[] = {lbm::kEnsAuto, lbm::kBlockTileW, lbm::kWideTileW};
     cudaEvent_t a, b;
     ENS_TRY(cudaEventCreate(&a), "event");
     ENS_TRY(cudaEventCreate(&b), "event");

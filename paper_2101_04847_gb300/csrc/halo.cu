@@ -15,6 +15,12 @@
 namespace lbm {
 namespace {
 
+// Index of column x, row r of plane pl = 9 component + direction in the stored cells.
+__device__ __forceinline__ size_t stored(const Grid& g, int pl, int r, int x) {
+    const int s = pl / 9, i = pl - 9 * s;
+    return 2 * ((size_t)i * g.plane + (size_t)r * g.pitch + g.origin + x) + s;
+}
+
 // buf layout: [plane 18][row ny][column 2], element type of the storage
 template <typename T>
 __global__ void halo_pack_kernel(const T* __restrict__ pops, Grid g, int col0, T* __restrict__ buf) {
@@ -22,7 +28,7 @@ __global__ void halo_pack_kernel(const T* __restrict__ pops, Grid g, int col0, T
     const int n = 36 * g.ny;
     if (idx >= n) return;
     const int c = idx & 1, r = (idx >> 1) % g.ny, pl = (idx >> 1) / g.ny;
-    buf[idx] = pops[(size_t)pl * g.plane + (size_t)r * g.pitch + g.origin + col0 + c];
+    buf[idx] = pops[stored(g, pl, r, col0 + c)];
 }
 
 template <typename T>
@@ -31,7 +37,7 @@ __global__ void halo_unpack_kernel(T* __restrict__ pops, Grid g, int col0, const
     const int n = 36 * g.ny;
     if (idx >= n) return;
     const int c = idx & 1, r = (idx >> 1) % g.ny, pl = (idx >> 1) / g.ny;
-    pops[(size_t)pl * g.plane + (size_t)r * g.pitch + g.origin + col0 + c] = buf[idx];
+    pops[stored(g, pl, r, col0 + c)] = buf[idx];
 }
 
 size_t elem_bytes(int storage) { return storage == LBM_STORE_F32 ? 4 : 2; }

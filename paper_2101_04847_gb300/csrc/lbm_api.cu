@@ -85,21 +85,31 @@ std::vector<double> interface_height(const lbm_params& p) {
 
 struct Layout {
     size_t pops[2], psi, scratch, partials, out, flag, y0, total;
-    size_t pop_bytes, plane;
-    int pitch, origin;
+    size_t pop_bytes, plane, file_bytes;
+    int pitch, origin, file_pitch, file_origin;   // in cells; in values
 };
+
+// Columns from column 0 on that a stored row leaves room for.
+int row_columns(int nx) {
+    const int wide_end = (nx + lbm::kWideTileW - 1) / lbm::kWideTileW * lbm::kWideTileW + 8;
+    return std::max(nx + lbm::kBlockTileW + 32, wide_end);
+}
 
 Layout make_layout(const lbm_params& p) {
     Layout L;
     // column 0 sits 128 bytes into each row; the row leaves room for the staged
     // kernels' windows (up to 144 columns from x0 - 10, x0 < nx; the 256-column tile's
-    // up to 8 columns past nx rounded up to 256) and the ghost copies.  No wider: at
-    // 1024 x 2048 a row of 1344 floats instead of 1216 measured 0.5 % slower.
-    L.origin = (int)(128 / elem_size(p.storage));
-    const int wide_end = (p.nx + lbm::kWideTileW - 1) / lbm::kWideTileW * lbm::kWideTileW + 8;
-    L.pitch = (L.origin + std::max(p.nx + lbm::kBlockTileW + 32, wide_end) + 63) / 64 * 64;
+    // up to 8 columns past nx rounded up to 256) and the ghost copies.  No wider: wider
+    // rows measured slower.
+    const size_t cell = 2 * elem_size(p.storage);
+    L.origin = (int)(128 / cell);
+    L.pitch = (L.origin + row_columns(p.nx) + 63) / 64 * 64;
     L.plane = (size_t)p.ny * L.pitch;
-    L.pop_bytes = 18 * L.plane * elem_size(p.storage);
+    L.pop_bytes = 9 * L.plane * cell;
+    // state files hold planes of one component and direction with a row layout of their own
+    L.file_origin = (int)(128 / elem_size(p.storage));
+    L.file_pitch = (L.file_origin + row_columns(p.nx) + 63) / 64 * 64;
+    L.file_bytes = 18 * (size_t)p.ny * L.file_pitch * elem_size(p.storage);
     const size_t n = (size_t)p.nx * p.ny;
     size_t off = 0;
     L.pops[0] = off; off = align_up(off + L.pop_bytes);
@@ -108,7 +118,7 @@ Layout make_layout(const lbm_params& p) {
     // scratch: diagnostics fields, host staging (18 doubles per site), or a saved copy
     // of one population buffer (tuning)
     const size_t scratch_b = std::max({lbm::diag_scratch_doubles(p.nx, p.ny) * sizeof(double),
-                                       (size_t)18 * n * sizeof(double), L.pop_bytes});
+                                       (size_t)18 * n * sizeof(double), L.pop_bytes, L.file_bytes});
     L.scratch = off; off = align_up(off + scratch_b);
     L.partials = off; off = align_up(off + lbm::diag_partials_doubles(p.nx, p.ny) * sizeof(double));
     L.out = off; off = align_up(off + (lbm::kDiagTerms + 2 * (size_t)p.ny) * sizeof(double));
@@ -894,8 +904,11 @@ struct SaveHeader {
 
 lbm_status lbm_save(lbm_handle* h, const char* path) {
     if (!h || !path) return fail(LBM_EINVAL, "NULL argument");
-    std::vector<char> buf(h->L.pop_bytes);
-    LBM_TRY(cudaMemcpyAsync(buf.data(), h->pops(h->cur), buf.size(), cudaMemcpyDeviceToHost, h->stream), "copy state");
+    std::vector<char> buf(h->L.file_bytes);
+    LBM_TRY(cudaMemsetAsync(h->scratch(), 0, h->L.file_bytes, h->stream), "clear scratch");
+    LBM_TRY(lbm::launch_cells_to_planes(h->pops(h->cur), h->grid, h->p.storage, h->scratch(), h->L.file_pitch,
+                                        h->L.file_origin, h->stream), "state planes");
+    LBM_TRY(cudaMemcpyAsync(buf.data(), h->scratch(), buf.size(), cudaMemcpyDeviceToHost, h->stream), "copy state");
     LBM_TRY(cudaStreamSynchronize(h->stream), "sync");
     SaveHeader hd;
     std::memset(&hd, 0, sizeof(hd));
@@ -904,7 +917,7 @@ lbm_status lbm_save(lbm_handle* h, const char* path) {
     hd.nx = h->p.nx;
     hd.ny = h->p.ny;
     hd.storage = h->p.storage;
-    hd.pitch = h->L.pitch;
+    hd.pitch = h->L.file_pitch;
     hd.step = h->step;
     hd.bytes = buf.size();
     hd.params = h->p;
@@ -925,8 +938,8 @@ lbm_status lbm_load(lbm_handle* h, const char* path) {
         std::fclose(f);
         return fail(LBM_EIO, "not a state file");
     }
-    if (hd.nx != h->p.nx || hd.ny != h->p.ny || hd.storage != h->p.storage || hd.pitch != h->L.pitch ||
-        hd.bytes != h->L.pop_bytes) {
+    if (hd.nx != h->p.nx || hd.ny != h->p.ny || hd.storage != h->p.storage || hd.pitch != h->L.file_pitch ||
+        hd.bytes != h->L.file_bytes) {
         std::fclose(f);
         return fail(LBM_EINVAL, "state file does not match the handle (nx, ny, storage)");
     }
@@ -934,7 +947,9 @@ lbm_status lbm_load(lbm_handle* h, const char* path) {
     const bool ok = std::fread(buf.data(), 1, buf.size(), f) == buf.size();
     std::fclose(f);
     if (!ok) return fail(LBM_EIO, "truncated state file");
-    LBM_TRY(cudaMemcpyAsync(h->pops(h->cur), buf.data(), buf.size(), cudaMemcpyHostToDevice, h->stream), "copy state");
+    LBM_TRY(cudaMemcpyAsync(h->scratch(), buf.data(), buf.size(), cudaMemcpyHostToDevice, h->stream), "copy state");
+    LBM_TRY(lbm::launch_planes_to_cells(h->scratch(), h->L.file_pitch, h->L.file_origin, h->grid, h->p.storage,
+                                        h->pops(h->cur), h->stream), "state cells");
     // the rounding counter continues from the saved step, as in the run that saved it
     h->saved_ctr[0] = h->saved_ctr[1] = (uint32_t)hd.step;
     LBM_TRY(cudaMemcpyAsync(h->step_ctr(), h->saved_ctr, sizeof(h->saved_ctr), cudaMemcpyHostToDevice, h->stream),

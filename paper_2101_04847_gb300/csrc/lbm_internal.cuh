@@ -58,10 +58,10 @@ struct Physics {
 // Geometry of one population array set.
 struct Grid {
     int nx, ny;
-    int pitch;          // elements per stored row
-    int origin;         // element offset of column 0 in a row (128 bytes); columns
+    int pitch;          // cells (both components of a direction at a site) per stored row
+    int origin;         // cell offset of column 0 in a row (128 bytes); columns
                         // -2, -1, nx, nx+1 hold periodic copies of nx-2, nx-1, 0, 1
-    size_t plane;       // elements per (component, direction) plane = ny * pitch
+    size_t plane;       // cells per direction plane = ny * pitch
     int x_offset = 0;   // column 0 is column x_offset of a whole grid of nx_total columns
     int nx_total = 0;   // (domain decomposition; 0 = nx): the stochastic rounding's site index
 };
@@ -70,14 +70,13 @@ struct Grid {
 // ensemble kernel's and the narrow single-grid tile, and the wide single-grid tile.
 constexpr int kBlockTileW = 128;
 constexpr int kWideTileW = 256;
-// Ensemble tile width 0: blocks of 128 threads, FP32 members in tiles of 128 columns
-// (one per thread), 16-bit members in paired-column tiles of 256 (two per thread).
-constexpr int kEnsPaired = 0;
+// Ensemble tile width 0: chosen by the library (128 columns).
+constexpr int kEnsAuto = 0;
 
 struct StepLaunch {
     const void* fin;
     void* fout;
-    float* psi;          // two-pass only: [2][ny][pitch]
+    float* psi;          // two-pass only: [ny][pitch] pairs
     int* flag;           // guard flag (NaN / negative density)
     Grid grid;
     Physics phys;
@@ -102,7 +101,7 @@ struct EnsMember {
 // ensemble / tiling helpers (step_kernels.cu)
 int warp_tiles(const Grid& g, int tile_y, int* tiles_x);
 int default_tile_y();
-// columns of one ensemble tile of a member with this storage (tile_x 128, 256 or kEnsPaired)
+// columns of one ensemble tile of a member with this storage (tile_x 128, 256 or kEnsAuto)
 int ensemble_tile_cols(int storage, int tile_x);
 // dynamic shared memory of one block tile for a storage type
 size_t block_tile_smem_bytes(int storage, int tile_x);
@@ -154,6 +153,12 @@ cudaError_t launch_init(void* fout, const Grid& g, int storage, const float shif
 // S (double, [2][9][ny][nx]) from the stored state
 cudaError_t launch_pull_to_double(const void* fin, const Grid& g, int storage,
                                   const float shift[2], double* S, cudaStream_t st);
+// the planes of a state file, [component][direction][ny][pitch] values with the ghost
+// columns, column 0 `origin` values into a row, from / to the stored cells
+cudaError_t launch_cells_to_planes(const void* pops, const Grid& g, int storage, void* planes, int pitch, int origin,
+                                   cudaStream_t st);
+cudaError_t launch_planes_to_cells(const void* planes, int pitch, int origin, const Grid& g, int storage, void* pops,
+                                   cudaStream_t st);
 // stored state from S (double, [2][9][ny][nx])
 cudaError_t launch_push_from_double(const double* S, const Grid& g, int storage,
                                     const float shift[2], void* fout, cudaStream_t st);

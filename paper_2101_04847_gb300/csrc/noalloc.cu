@@ -54,47 +54,33 @@ noalloc_collide_push_kernel(const float* __restrict__ S, float* __restrict__ out
     if (x >= nx) return;
     const size_t n = (size_t)nx * ny;
     const size_t k = (size_t)y * nx + x;
-    float f[2][9];
+    float2 f[9];
 #pragma unroll
-    for (int s = 0; s < 2; ++s)
-#pragma unroll
-        for (int i = 0; i < 9; ++i) f[s][i] = __ldg(S + (size_t)(s * 9 + i) * n + k);
+    for (int i = 0; i < 9; ++i)
+        f[i] = make_float2(__ldg(S + (size_t)i * n + k), __ldg(S + (size_t)(9 + i) * n + k));
     const int xm = x == 0 ? nx - 1 : x - 1;
     const int xp = x == nx - 1 ? 0 : x + 1;
-    Nbr p[2];
+    auto at = [&](int yy, int xx) {   // (B, A)
+        const size_t q = (size_t)yy * nx + xx;
+        return make_float2(__ldg(rho + n + q), __ldg(rho + q));
+    };
+    Nbr2 p;
+    p.E = at(y, xp);
+    p.W = at(y, xm);
+    p.N = p.NE = p.NW = p.S = p.SE = p.SW = splat(0.0f);
+    if (y + 1 < ny) { p.N = at(y + 1, x); p.NE = at(y + 1, xp); p.NW = at(y + 1, xm); }
+    if (y > 0) { p.S = at(y - 1, x); p.SE = at(y - 1, xp); p.SW = at(y - 1, xm); }
+    if (!collide_site<true, true>(f, sum9_2(f), p, ph, y, ny)) atomicOr(flag, 1);
 #pragma unroll
-    for (int s = 0; s < 2; ++s) {
-        const float* r = rho + (size_t)s * n;
-        p[s].E = __ldg(r + (size_t)y * nx + xp);
-        p[s].W = __ldg(r + (size_t)y * nx + xm);
-        if (y + 1 < ny) {
-            p[s].N = __ldg(r + (size_t)(y + 1) * nx + x);
-            p[s].NE = __ldg(r + (size_t)(y + 1) * nx + xp);
-            p[s].NW = __ldg(r + (size_t)(y + 1) * nx + xm);
-        } else {
-            p[s].N = p[s].NE = p[s].NW = 0.0f;
+    for (int i = 0; i < 9; ++i) {
+        const int ty = y + cy(i);
+        size_t dst = (size_t)opp(i) * n + k;
+        if (ty >= 0 && ty < ny) {
+            const int tx = cx(i) == 0 ? x : (cx(i) == 1 ? xp : xm);
+            dst = (size_t)i * n + (size_t)ty * nx + tx;
         }
-        if (y > 0) {
-            p[s].S = __ldg(r + (size_t)(y - 1) * nx + x);
-            p[s].SE = __ldg(r + (size_t)(y - 1) * nx + xp);
-            p[s].SW = __ldg(r + (size_t)(y - 1) * nx + xm);
-        } else {
-            p[s].S = p[s].SE = p[s].SW = 0.0f;
-        }
-    }
-    collide_site<true>(f, p[0], p[1], ph, y, ny, flag);
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-#pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            const int ty = y + cy(i);
-            if (ty >= 0 && ty < ny) {
-                const int tx = cx(i) == 0 ? x : (cx(i) == 1 ? xp : xm);
-                out[(size_t)(s * 9 + i) * n + (size_t)ty * nx + tx] = f[s][i];
-            } else {
-                out[(size_t)(s * 9 + opp(i)) * n + k] = f[s][i];
-            }
-        }
+        out[dst] = f[i].x;
+        out[9 * n + dst] = f[i].y;
     }
 }
 

@@ -7,25 +7,39 @@
 // post-streaming populations of the kinetic equation are obtained by pulling:
 //     S_i(x, y) = B_i(x - c_ix, y - c_iy)   if 0 <= y - c_iy < ny
 //     S_i(x, y) = B_opp(i)(x, y)            otherwise (bounce-back at the wall)
-// Layout: structure of arrays [component][direction][y][pitch], x fastest.
+// Layout: [direction][y][pitch] cells of both components (lattice.cuh), x fastest.
 #include <algorithm>
+#include <type_traits>
 
 #include "collide.cuh"
 
 namespace lbm {
 
+__device__ __forceinline__ float2 shift_of(const Physics& ph) { return make_float2(ph.shift[0], ph.shift[1]); }
+// FP32 keeps the increments the stored values received (collide_site<true>)
+template <typename T> struct Exact { static constexpr bool value = !IsShifted<T>::value; };
+
+// The eight neighbours of ring column c from the density rows S, C, N.
+__device__ __forceinline__ Nbr2 ring_nbr(const float2* S, const float2* C, const float2* N, int c) {
+    Nbr2 p;
+    p.E = C[c + 1]; p.W = C[c - 1];
+    p.N = N[c]; p.NE = N[c + 1]; p.NW = N[c - 1];
+    p.S = S[c]; p.SE = S[c + 1]; p.SW = S[c - 1];
+    return p;
+}
+
 // ---------------------------------------------------------------------------
 // Fused pull stream-collide.  A block owns kThreadsX columns and tile_y rows and
 // sweeps its rows bottom-up.  Each thread keeps the populations of its column for
 // the current and the next row in registers; the densities of three consecutive
-// rows (plus one halo column each side) live in a 4-slot shared-memory ring.
-// The only redundant loads are the pulls of the halo columns and of the two halo
-// rows y0 - 1 and y1, which only feed densities.
+// rows (plus one halo column each side), as (B, A), live in a 4-slot shared-memory
+// ring.  The only redundant loads are the pulls of the halo columns and of the two
+// halo rows y0 - 1 and y1, which only feed densities.
 // ---------------------------------------------------------------------------
 template <typename T>
 __global__ void __launch_bounds__(kThreadsX)
-step_fused_kernel(const T* __restrict__ fin, T* __restrict__ fout, Grid g, Physics ph, int tile_y, int* flag) {
-    __shared__ float sR[4][2][kThreadsX + 2];
+step_fused_kernel(const Cell<T>* __restrict__ fin, Cell<T>* __restrict__ fout, Grid g, Physics ph, int tile_y, int* flag) {
+    __shared__ float2 sR[4][kThreadsX + 2];
     const int t = threadIdx.x;
     const uint32_t seed = launch_seed(ph);
     advance_step(ph, blockIdx.x == 0 && blockIdx.y == 0 && t == 0);
@@ -45,74 +59,37 @@ step_fused_kernel(const T* __restrict__ fin, T* __restrict__ fout, Grid g, Physi
     const int hxp = hx == g.nx - 1 ? 0 : hx + 1;
     const int hk = haloL ? 0 : w + 1;
     const bool halo = haloL || haloR;
-    const float shift[2] = {ph.shift[0], ph.shift[1]};
+    const float2 shift = shift_of(ph);
 
-    float cur[2][9];
-    // rows y0-1 (density only) and y0
-    {
-        const int slot = (y0 - 1) & 3;
-        float rA = 0.0f, rB = 0.0f, hA = 0.0f, hB = 0.0f;
-        if (y0 > 0) {
-            float tmp[2][9];
-            pull_site<T>(fin, g, shift, y0 - 1, x, xm, xp, tmp);
-            rA = sum9(tmp[0]); rB = sum9(tmp[1]);
+    // row yo into f and its densities into the ring (zero on the virtual wall rows)
+    auto pull_row = [&](int yo, float2 f[9]) {
+        const int slot = yo & 3;
+        float2 r = splat(0.0f), h = splat(0.0f);
+        if (yo >= 0 && yo < g.ny) {
+            pull_site<T>(fin, g, shift, yo, x, xm, xp, f);
+            r = swap2(sum9_2(f));
             if (halo) {
-                pull_site<T>(fin, g, shift, y0 - 1, hx, hxm, hxp, tmp);
-                hA = sum9(tmp[0]); hB = sum9(tmp[1]);
+                float2 tmp[9];
+                pull_site<T>(fin, g, shift, yo, hx, hxm, hxp, tmp);
+                h = swap2(sum9_2(tmp));
             }
         }
-        if (active) { sR[slot][0][t + 1] = rA; sR[slot][1][t + 1] = rB; }
-        if (halo) { sR[slot][0][hk] = hA; sR[slot][1][hk] = hB; }
-    }
-    {
-        const int slot = y0 & 3;
-        pull_site<T>(fin, g, shift, y0, x, xm, xp, cur);
-        if (active) { sR[slot][0][t + 1] = sum9(cur[0]); sR[slot][1][t + 1] = sum9(cur[1]); }
-        if (halo) {
-            float tmp[2][9];
-            pull_site<T>(fin, g, shift, y0, hx, hxm, hxp, tmp);
-            sR[slot][0][hk] = sum9(tmp[0]); sR[slot][1][hk] = sum9(tmp[1]);
-        }
-    }
+        if (active) sR[slot][t + 1] = r;
+        if (halo) sR[slot][hk] = h;
+    };
+    float2 cur[9], nxt[9];
+    pull_row(y0 - 1, nxt);
+    pull_row(y0, cur);
     for (int y = y0; y < y1; ++y) {
-        float nxt[2][9];
-        const int sn = (y + 1) & 3;
-        if (y + 1 < g.ny) {
-            pull_site<T>(fin, g, shift, y + 1, x, xm, xp, nxt);
-            if (active) { sR[sn][0][t + 1] = sum9(nxt[0]); sR[sn][1][t + 1] = sum9(nxt[1]); }
-            if (halo) {
-                float tmp[2][9];
-                pull_site<T>(fin, g, shift, y + 1, hx, hxm, hxp, tmp);
-                sR[sn][0][hk] = sum9(tmp[0]); sR[sn][1][hk] = sum9(tmp[1]);
-            }
-        } else {
-#pragma unroll
-            for (int s = 0; s < 2; ++s)
-#pragma unroll
-                for (int i = 0; i < 9; ++i) nxt[s][i] = 0.0f;
-            if (active) { sR[sn][0][t + 1] = 0.0f; sR[sn][1][t + 1] = 0.0f; }
-            if (halo) { sR[sn][0][hk] = 0.0f; sR[sn][1][hk] = 0.0f; }
-        }
+        pull_row(y + 1, nxt);
         __syncthreads();
         if (active) {
-            const int k = t + 1;
-            const int s0 = (y - 1) & 3, s1 = y & 3, s2 = sn;
-            Nbr pA, pB;
-            pA.E = sR[s1][0][k + 1]; pA.W = sR[s1][0][k - 1];
-            pA.N = sR[s2][0][k];     pA.S = sR[s0][0][k];
-            pA.NE = sR[s2][0][k + 1]; pA.NW = sR[s2][0][k - 1];
-            pA.SE = sR[s0][0][k + 1]; pA.SW = sR[s0][0][k - 1];
-            pB.E = sR[s1][1][k + 1]; pB.W = sR[s1][1][k - 1];
-            pB.N = sR[s2][1][k];     pB.S = sR[s0][1][k];
-            pB.NE = sR[s2][1][k + 1]; pB.NW = sR[s2][1][k - 1];
-            pB.SE = sR[s0][1][k + 1]; pB.SW = sR[s0][1][k - 1];
-            collide_site<IsShifted<T>::value == false>(cur, pA, pB, ph, y, g.ny, flag);
+            const Nbr2 p = ring_nbr(sR[(y - 1) & 3], sR[y & 3], sR[(y + 1) & 3], t + 1);
+            if (!collide_site<Exact<T>::value, true>(cur, sum9_2(cur), p, ph, y, g.ny)) atomicOr(flag, 1);
             store_step<T>(fout, g, y, x, cur, shift, seed);
         }
 #pragma unroll
-        for (int s = 0; s < 2; ++s)
-#pragma unroll
-            for (int i = 0; i < 9; ++i) cur[s][i] = nxt[s][i];
+        for (int i = 0; i < 9; ++i) cur[i] = nxt[i];
     }
 }
 
@@ -123,7 +100,7 @@ step_fused_kernel(const T* __restrict__ fin, T* __restrict__ fout, Grid g, Physi
 // xw - 1 + l, so lanes 0 and 31 only supply the halo densities of their
 // neighbours.  The warp brings its input rows into its own shared-memory ring
 // with bulk asynchronous copies (cp.async.bulk, one mbarrier per stage, issued by
-// lane 0): row r of all 18 planes, a 16-byte aligned window of kWinW(T) columns
+// lane 0): row r of all 9 planes, a 16-byte aligned window of kWinW(T) columns
 // covering [xw - 2, xw + 32), lands in stage (q0 + r - rfirst) mod kStages.  The
 // densities of rows y-1, y, y+1 stay in registers and the x-neighbours come by
 // warp shuffles, so no block-wide barrier is ever needed; a warp refills a stage
@@ -134,9 +111,8 @@ constexpr int kStages = 6;     // rows y..y+2 in use + 3 rows prefetched
 constexpr int kWarpOwned = 30;
 constexpr int kWarpsPerBlock = kThreadsX / 32;
 constexpr uint32_t kWaitLimit = 1u << 22;
-template <typename T> struct WinW { static constexpr int value = 40; };   // 160 B rows (FP32)
-template <> struct WinW<__half> { static constexpr int value = 48; };     // 96 B rows
-template <> struct WinW<__nv_bfloat16> { static constexpr int value = 48; };
+constexpr uint32_t kTestWaitLimit = 4096;   // the timeout test's
+template <typename T> struct WinW { static constexpr int value = 40; };   // 36 columns and the alignment slack, 16-byte multiple
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
@@ -173,48 +149,62 @@ __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.p
 // Dynamic shared memory of one warp: kStages mbarriers, then the row ring.
 template <typename T>
 __host__ __device__ constexpr size_t warp_smem_bytes() {
-    return 128 + (size_t)kStages * 18 * WinW<T>::value * sizeof(T);
+    return 128 + (size_t)kStages * 9 * WinW<T>::value * sizeof(Cell<T>);
 }
 template <typename T>
 size_t warp_kernel_smem_bytes() { return kWarpsPerBlock * warp_smem_bytes<T>(); }
 
-// Post-streaming populations of window column k on row yo from the stages holding
-// rows yo-1 (S), yo (C) and yo+1 (N); on the wall rows the populations coming from
-// outside are the bounced-back ones of row yo.
-template <typename T>
-__device__ __forceinline__ void pull_staged(const T* __restrict__ stS, const T* __restrict__ stC,
-                                            const T* __restrict__ stN, bool bottom, bool top, int k,
-                                            const float shift[2], float f[2][9]) {
-    constexpr int W = WinW<T>::value;
+// Post-streaming cells of window column k on row yo from the stages holding rows
+// yo-1 (S), yo (C) and yo+1 (N), W columns per plane; on the wall rows the
+// populations coming from outside are the bounced-back ones of row yo.
+template <int W, typename C>
+__device__ __forceinline__ void pull_cells(const C* __restrict__ stS, const C* __restrict__ stC, const C* __restrict__ stN,
+                                           bool bottom, bool top, int k, C f[9]) {
 #pragma unroll
-    for (int s = 0; s < 2; ++s) {
-#pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            const int pl = s * 9 + i;
-            T v;
-            if (cy(i) == 0) {
-                v = stC[pl * W + k - cx(i)];
-            } else if (cy(i) == 1) {
-                v = bottom ? stC[(s * 9 + opp(i)) * W + k] : stS[pl * W + k - cx(i)];
-            } else {
-                v = top ? stC[(s * 9 + opp(i)) * W + k] : stN[pl * W + k - cx(i)];
-            }
-            float fv = to_f<T>(v);
-            if (IsShifted<T>::value) fv += wf(i) * shift[s];
-            f[s][i] = fv;
-        }
+    for (int i = 0; i < 9; ++i) {
+        if (cy(i) == 0) f[i] = stC[i * W + k - cx(i)];
+        else if (cy(i) == 1) f[i] = bottom ? stC[opp(i) * W + k] : stS[i * W + k - cx(i)];
+        else f[i] = top ? stC[opp(i) * W + k] : stN[i * W + k - cx(i)];
     }
+}
+// the same as populations
+template <typename T, int W>
+__device__ __forceinline__ void pull_staged(const Cell<T>* __restrict__ stS, const Cell<T>* __restrict__ stC,
+                                            const Cell<T>* __restrict__ stN, bool bottom, bool top, int k, float2 shift,
+                                            float2 f[9]) {
+    Cell<T> c[9];
+    pull_cells<W>(stS, stC, stN, bottom, top, k, c);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) f[i] = cell_pops<T>(c[i], i, shift);
+}
+
+// The neighbours of a lane's column from the lanes beside it: own densities, as
+// (B, A), of rows y - 1 (rm), y (rc) and y + 1 (rp).
+__device__ __forceinline__ float2 shfl_up2(float2 v) {
+    return make_float2(__shfl_up_sync(0xffffffffu, v.x, 1), __shfl_up_sync(0xffffffffu, v.y, 1));
+}
+__device__ __forceinline__ float2 shfl_down2(float2 v) {
+    return make_float2(__shfl_down_sync(0xffffffffu, v.x, 1), __shfl_down_sync(0xffffffffu, v.y, 1));
+}
+__device__ __forceinline__ Nbr2 lane_nbr(float2 rm, float2 rc, float2 rp) {
+    Nbr2 p;
+    p.S = rm; p.N = rp;
+    p.W = shfl_up2(rc); p.E = shfl_down2(rc);
+    p.SW = shfl_up2(rm); p.SE = shfl_down2(rm);
+    p.NW = shfl_up2(rp); p.NE = shfl_down2(rp);
+    return p;
 }
 
 // One warp tile (tx, ty): `my` is the warp's shared-memory region.
 template <typename T>
-__device__ __forceinline__ void warp_tile(const T* __restrict__ fin, T* __restrict__ fout, const Grid& g,
+__device__ __forceinline__ void warp_tile(const Cell<T>* __restrict__ fin, Cell<T>* __restrict__ fout, const Grid& g,
                                           const Physics& ph, int tile_y, int tx, int ty, unsigned char* my,
                                           uint32_t seed, int* flag) {
+    typedef Cell<T> C;
     constexpr int W = WinW<T>::value;
     const int lane = threadIdx.x & 31;
     uint64_t* bar = reinterpret_cast<uint64_t*>(my);
-    T* stage = reinterpret_cast<T*>(my + 128);
+    C* stage = reinterpret_cast<C*>(my + 128);
     const int xw = tx * kWarpOwned;
     const int y0 = ty * tile_y;
     const int y1 = min(y0 + tile_y, g.ny);
@@ -222,13 +212,13 @@ __device__ __forceinline__ void warp_tile(const T* __restrict__ fin, T* __restri
     const int rlast = min(y1 + 1, g.ny - 1);
     const int x = xw - 1 + lane;
     const bool owner = lane >= 1 && lane <= kWarpOwned && x < g.nx;
-    constexpr int kAlign = 16 / (int)sizeof(T);
+    constexpr int kAlign = 16 / (int)sizeof(C);
     const int e0 = g.origin + xw - 2;
     const int slack = e0 % kAlign;
     const int k = lane + 1 + slack;                 // window column of this lane's site
-    const T* win = fin + (e0 - slack);
-    const float shift[2] = {ph.shift[0], ph.shift[1]};
-    const uint32_t row_bytes = W * sizeof(T);
+    const C* win = fin + (e0 - slack);
+    const float2 shift = shift_of(ph);
+    const uint32_t row_bytes = W * sizeof(C);
 
     if (lane == 0) {
         for (int j = 0; j < kStages; ++j) mbar_init(&bar[j], 1);
@@ -239,11 +229,11 @@ __device__ __forceinline__ void warp_tile(const T* __restrict__ fin, T* __restri
     auto issue = [&](int r) {
         const int j = (r - rfirst) % kStages;
         uint64_t* b = &bar[j];
-        mbar_expect_tx(b, 18 * row_bytes);
-        T* dst = stage + (size_t)j * 18 * W;
-        const T* src = win + (size_t)r * g.pitch;
+        mbar_expect_tx(b, 9 * row_bytes);
+        C* dst = stage + (size_t)j * 9 * W;
+        const C* src = win + (size_t)r * g.pitch;
 #pragma unroll 1
-        for (int p = 0; p < 18; ++p) bulk_copy_g2s(dst + p * W, src + (size_t)p * g.plane, row_bytes, b);
+        for (int p = 0; p < 9; ++p) bulk_copy_g2s(dst + p * W, src + (size_t)p * g.plane, row_bytes, b);
     };
     if (lane == 0)
         for (; next <= rlast && next < rfirst + kStages; ++next) issue(next);
@@ -251,12 +241,12 @@ __device__ __forceinline__ void warp_tile(const T* __restrict__ fin, T* __restri
         if (r >= rfirst && r <= rlast)
             mbar_wait(&bar[(r - rfirst) % kStages], (uint32_t)(((r - rfirst) / kStages) & 1), flag);
     };
-    auto stage_of = [&](int r) -> const T* {
+    auto stage_of = [&](int r) -> const C* {
         const int rr = min(max(r, rfirst), rlast);
-        return stage + (size_t)((rr - rfirst) % kStages) * 18 * W;
+        return stage + (size_t)((rr - rfirst) % kStages) * 9 * W;
     };
-    auto pull_row = [&](int yo, float f[2][9]) {
-        pull_staged<T>(stage_of(yo - 1), stage_of(yo), stage_of(yo + 1), yo == 0, yo == g.ny - 1, k, shift, f);
+    auto pull_row = [&](int yo, float2 f[9]) {
+        pull_staged<T, W>(stage_of(yo - 1), stage_of(yo), stage_of(yo + 1), yo == 0, yo == g.ny - 1, k, shift, f);
     };
     // After the reads of row yo (which used input rows up to yo + 1), input rows
     // <= yo - 1 are no longer needed: refill their stages.
@@ -268,43 +258,33 @@ __device__ __forceinline__ void warp_tile(const T* __restrict__ fin, T* __restri
         }
     };
 
-    float fa[2][9], fb[2][9];
-    float rm[2] = {0.0f, 0.0f};   // densities of row y - 1 (zero on the virtual wall row)
+    float2 fa[9], fb[9];
+    float2 rm = splat(0.0f);   // densities of row y - 1, as (B, A) (zero on the virtual wall row)
     if (y0 > 0) {
         wait_row(y0 - 2); wait_row(y0 - 1); wait_row(y0);
         pull_row(y0 - 1, fb);
-        rm[0] = sum9(fb[0]); rm[1] = sum9(fb[1]);
+        rm = swap2(sum9_2(fb));
     }
     wait_row(y0 - 1); wait_row(y0); wait_row(y0 + 1);
     pull_row(y0, fa);
-    float rc[2] = {sum9(fa[0]), sum9(fa[1])};      // row y
+    float2 rc = swap2(sum9_2(fa));      // row y
     refill(y0);
 
-    auto row = [&](int y, float cur[2][9], float nxt[2][9]) {
-        float rp[2] = {0.0f, 0.0f};                 // row y + 1
+    auto row = [&](int y, float2 cur[9], float2 nxt[9]) {
+        float2 rp = splat(0.0f);        // row y + 1
         if (y + 1 < g.ny) {
             wait_row(y + 2);
             pull_row(y + 1, nxt);
-            rp[0] = sum9(nxt[0]); rp[1] = sum9(nxt[1]);
+            rp = swap2(sum9_2(nxt));
         }
         refill(y + 1);
-        Nbr p[2];
-#pragma unroll
-        for (int s = 0; s < 2; ++s) {
-            p[s].S = rm[s]; p[s].N = rp[s];
-            p[s].W = __shfl_up_sync(0xffffffffu, rc[s], 1);
-            p[s].E = __shfl_down_sync(0xffffffffu, rc[s], 1);
-            p[s].SW = __shfl_up_sync(0xffffffffu, rm[s], 1);
-            p[s].SE = __shfl_down_sync(0xffffffffu, rm[s], 1);
-            p[s].NW = __shfl_up_sync(0xffffffffu, rp[s], 1);
-            p[s].NE = __shfl_down_sync(0xffffffffu, rp[s], 1);
-        }
+        const Nbr2 p = lane_nbr(rm, rc, rp);
         if (owner) {
-            collide_site<IsShifted<T>::value == false>(cur, p[0], p[1], ph, y, g.ny, flag);
+            if (!collide_site<Exact<T>::value, true>(cur, sum9_2(cur), p, ph, y, g.ny)) atomicOr(flag, 1);
             store_step<T>(fout, g, y, x, cur, shift, seed);
         }
-#pragma unroll
-        for (int s = 0; s < 2; ++s) { rm[s] = rc[s]; rc[s] = rp[s]; }
+        rm = rc;
+        rc = rp;
     };
     for (int y = y0; y < y1; y += 2) {
         row(y, fa, fb);
@@ -314,7 +294,7 @@ __device__ __forceinline__ void warp_tile(const T* __restrict__ fin, T* __restri
 
 template <typename T>
 __global__ void __launch_bounds__(kThreadsX, 4)
-step_warp_kernel(const T* __restrict__ fin, T* __restrict__ fout, Grid g, Physics ph, int tile_y,
+step_warp_kernel(const Cell<T>* __restrict__ fin, Cell<T>* __restrict__ fout, Grid g, Physics ph, int tile_y,
                    int tiles_x, int tiles, int* flag) {
     extern __shared__ __align__(128) unsigned char dsm[];
     const int warp = threadIdx.x >> 5;
@@ -337,7 +317,7 @@ int default_tile_y() { return 32; }
 
 // ---------------------------------------------------------------------------
 // Pipelined fused pull stream-collide.  A block of 4 warps shares one ring of
-// input rows (bulk asynchronous copies of all 18 planes, 16-byte aligned windows of
+// input rows (bulk asynchronous copies of all 9 planes, 16-byte aligned windows of
 // kPipeWin columns covering [x0 - 2, x0 + 122)); each warp sweeps its own 32 columns
 // (30 owned, lanes 0 and 31 supply halo densities) with the x-neighbour densities
 // from warp shuffles, so warps never wait for one another at a block barrier.  A
@@ -351,7 +331,7 @@ constexpr int kPipeWin = 136;                              // >= 124 + 7, 16-byt
 
 template <typename T>
 __host__ __device__ constexpr size_t pipe_smem_bytes() {
-    return 128 + (size_t)kPipeStages * 18 * kPipeWin * sizeof(T);
+    return 128 + (size_t)kPipeStages * 9 * kPipeWin * sizeof(Cell<T>);
 }
 
 __device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
@@ -367,42 +347,17 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
 }
 
-// Post-streaming populations of window column k on row yo from the stages holding
-// rows yo-1 (S), yo (C), yo+1 (N) of a kPipeWin-wide window.
-template <typename T>
-__device__ __forceinline__ void pull_pipe(const T* __restrict__ stS, const T* __restrict__ stC,
-                                          const T* __restrict__ stN, bool bottom, bool top, int k,
-                                          const float shift[2], float f[2][9]) {
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-#pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            const int pl = s * 9 + i;
-            T v;
-            if (cy(i) == 0) {
-                v = stC[pl * kPipeWin + k - cx(i)];
-            } else if (cy(i) == 1) {
-                v = bottom ? stC[(s * 9 + opp(i)) * kPipeWin + k] : stS[pl * kPipeWin + k - cx(i)];
-            } else {
-                v = top ? stC[(s * 9 + opp(i)) * kPipeWin + k] : stN[pl * kPipeWin + k - cx(i)];
-            }
-            float fv = to_f<T>(v);
-            if (IsShifted<T>::value) fv += wf(i) * shift[s];
-            f[s][i] = fv;
-        }
-    }
-}
-
 template <typename T>
 __global__ void __launch_bounds__(kThreadsX, 4)
-step_pipe_kernel(const T* __restrict__ fin, T* __restrict__ fout, Grid g, Physics ph, int tile_y, int* flag) {
+step_pipe_kernel(const Cell<T>* __restrict__ fin, Cell<T>* __restrict__ fout, Grid g, Physics ph, int tile_y, int* flag) {
+    typedef Cell<T> C;
     const uint32_t seed = launch_seed(ph);
     advance_step(ph, blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0);
     constexpr int S = kPipeStages;
     extern __shared__ __align__(128) unsigned char dsm[];
     uint64_t* full = reinterpret_cast<uint64_t*>(dsm);
     uint64_t* empty = full + S;
-    T* stage = reinterpret_cast<T*>(dsm + 128);
+    C* stage = reinterpret_cast<C*>(dsm + 128);
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int x0 = blockIdx.x * kPipeOwned;
@@ -412,13 +367,13 @@ step_pipe_kernel(const T* __restrict__ fin, T* __restrict__ fout, Grid g, Physic
     const int rlast = min(y1 + 1, g.ny - 1);
     const int x = x0 + warp * kWarpOwned - 1 + lane;
     const bool owner = lane >= 1 && lane <= kWarpOwned && x < g.nx;
-    constexpr int kAlign = 16 / (int)sizeof(T);
+    constexpr int kAlign = 16 / (int)sizeof(C);
     const int e0 = g.origin + x0 - 2;
     const int slack = e0 % kAlign;
     const int k = warp * kWarpOwned + lane + 1 + slack;
-    const T* win = fin + (e0 - slack);
-    const float shift[2] = {ph.shift[0], ph.shift[1]};
-    const uint32_t row_bytes = kPipeWin * sizeof(T);
+    const C* win = fin + (e0 - slack);
+    const float2 shift = shift_of(ph);
+    const uint32_t row_bytes = kPipeWin * sizeof(C);
     const bool producer = threadIdx.x == 0;
 
     if (producer) {
@@ -445,11 +400,11 @@ step_pipe_kernel(const T* __restrict__ fin, T* __restrict__ fout, Grid g, Physic
                 }
             }
             fence_proxy_async_smem();
-            mbar_expect_tx(&full[j], 18 * row_bytes);
-            T* dst = stage + (size_t)j * 18 * kPipeWin;
-            const T* src = win + (size_t)next * g.pitch;
+            mbar_expect_tx(&full[j], 9 * row_bytes);
+            C* dst = stage + (size_t)j * 9 * kPipeWin;
+            const C* src = win + (size_t)next * g.pitch;
 #pragma unroll 1
-            for (int p = 0; p < 18; ++p) bulk_copy_g2s(dst + p * kPipeWin, src + (size_t)p * g.plane, row_bytes, &full[j]);
+            for (int p = 0; p < 9; ++p) bulk_copy_g2s(dst + p * kPipeWin, src + (size_t)p * g.plane, row_bytes, &full[j]);
             ++next;
         }
     };
@@ -461,15 +416,15 @@ step_pipe_kernel(const T* __restrict__ fin, T* __restrict__ fout, Grid g, Physic
         }
         mbar_wait(&full[(r - rfirst) % S], (uint32_t)(((r - rfirst) / S) & 1), flag);
     };
-    auto stage_of = [&](int r) -> const T* {
+    auto stage_of = [&](int r) -> const C* {
         const int rr = min(max(r, rfirst), rlast);
-        return stage + (size_t)((rr - rfirst) % S) * 18 * kPipeWin;
+        return stage + (size_t)((rr - rfirst) % S) * 9 * kPipeWin;
     };
-    auto pull_row = [&](int yo, float f[2][9]) {
+    auto pull_row = [&](int yo, float2 f[9]) {
         if (yo > 0 && yo < g.ny - 1)
-            pull_pipe<T>(stage_of(yo - 1), stage_of(yo), stage_of(yo + 1), false, false, k, shift, f);
+            pull_staged<T, kPipeWin>(stage_of(yo - 1), stage_of(yo), stage_of(yo + 1), false, false, k, shift, f);
         else
-            pull_pipe<T>(stage_of(yo - 1), stage_of(yo), stage_of(yo + 1), yo == 0, yo == g.ny - 1, k, shift, f);
+            pull_staged<T, kPipeWin>(stage_of(yo - 1), stage_of(yo), stage_of(yo + 1), yo == 0, yo == g.ny - 1, k, shift, f);
     };
     int released = rfirst;   // rows < released have been handed back by this warp
     auto release_upto = [&](int r) {   // this warp no longer reads rows <= r
@@ -478,43 +433,33 @@ step_pipe_kernel(const T* __restrict__ fin, T* __restrict__ fout, Grid g, Physic
             if (lane == 0) mbar_arrive(&empty[(released - rfirst) % S]);
     };
 
-    float fa[2][9], fb[2][9];
-    float rm[2] = {0.0f, 0.0f};
+    float2 fa[9], fb[9];
+    float2 rm = splat(0.0f);
     if (y0 > 0) {
         wait_row(y0 - 2); wait_row(y0 - 1); wait_row(y0);
         pull_row(y0 - 1, fb);
-        rm[0] = sum9(fb[0]); rm[1] = sum9(fb[1]);
+        rm = swap2(sum9_2(fb));
     }
     wait_row(y0 - 1); wait_row(y0); wait_row(y0 + 1);
     pull_row(y0, fa);
-    float rc[2] = {sum9(fa[0]), sum9(fa[1])};
+    float2 rc = swap2(sum9_2(fa));
     release_upto(y0 - 2);
 
-    auto row = [&](int y, float cur[2][9], float nxt[2][9]) {
-        float rp[2] = {0.0f, 0.0f};
+    auto row = [&](int y, float2 cur[9], float2 nxt[9]) {
+        float2 rp = splat(0.0f);
         if (y + 1 < g.ny) {
             wait_row(y + 2);
             pull_row(y + 1, nxt);
-            rp[0] = sum9(nxt[0]); rp[1] = sum9(nxt[1]);
+            rp = swap2(sum9_2(nxt));
         }
         release_upto(y - 1);
-        Nbr p[2];
-#pragma unroll
-        for (int s = 0; s < 2; ++s) {
-            p[s].S = rm[s]; p[s].N = rp[s];
-            p[s].W = __shfl_up_sync(0xffffffffu, rc[s], 1);
-            p[s].E = __shfl_down_sync(0xffffffffu, rc[s], 1);
-            p[s].SW = __shfl_up_sync(0xffffffffu, rm[s], 1);
-            p[s].SE = __shfl_down_sync(0xffffffffu, rm[s], 1);
-            p[s].NW = __shfl_up_sync(0xffffffffu, rp[s], 1);
-            p[s].NE = __shfl_down_sync(0xffffffffu, rp[s], 1);
-        }
+        const Nbr2 p = lane_nbr(rm, rc, rp);
         if (owner) {
-            collide_site<IsShifted<T>::value == false>(cur, p[0], p[1], ph, y, g.ny, flag);
+            if (!collide_site<Exact<T>::value, true>(cur, sum9_2(cur), p, ph, y, g.ny)) atomicOr(flag, 1);
             store_step<T>(fout, g, y, x, cur, shift, seed);
         }
-#pragma unroll
-        for (int s = 0; s < 2; ++s) { rm[s] = rc[s]; rc[s] = rp[s]; }
+        rm = rc;
+        rc = rp;
     };
     for (int y = y0; y < y1; y += 2) {
         row(y, fa, fb);
@@ -523,236 +468,286 @@ step_pipe_kernel(const T* __restrict__ fin, T* __restrict__ fout, Grid g, Physic
 }
 
 // ---------------------------------------------------------------------------
-// Block-staged fused pull stream-collide.  A block of 128 threads owns 128 columns
-// [x0, x0 + 128) and the rows [y0, y1) of one of gridDim.y tiles (the ny rows are
+// Block-staged fused pull stream-collide.  A block of TW threads owns TW columns
+// [x0, x0 + TW) and the rows [y0, y1) of one of gridDim.y tiles (the ny rows are
 // split evenly over the tiles); thread t handles column x0 + t, and threads 64 and
-// 65 also supply the densities of the halo columns x0 - 1 and x0 + 128.  Input rows
+// 65 also supply the densities of the halo columns x0 - 1 and x0 + TW.  Input rows
 // are brought into shared memory by bulk asynchronous copies (cp.async.bulk, one
-// mbarrier per stage), one plane per lane of lanes 0-17 of warp 0: row r of all 18
-// planes, a 16-byte aligned window of BlockWin<T> columns covering [x0 - 2, x0 + 130),
-// lands in stage (r - rfirst) mod kBlockStages.  All pulls read shared memory; each
-// input value crosses HBM once per tile and two rows ahead of the sweep are in
-// flight.  The densities of three rows are exchanged through a shared-memory ring
+// mbarrier per stage), one plane per lane of lanes 0-8 of warp 0: a 16-byte aligned
+// window of BlockWin<T> columns covering [x0 - 2, x0 + TW + 2) of each of the 9 planes a
+// row's pull reads (TileRows).  All pulls read shared memory; each input value crosses
+// HBM once per tile.  The densities of three rows are exchanged through a shared-memory ring
 // (one block barrier per row).
+//
+// What bounds it: FP32 is limited by HBM (0.97 of the copy rate at 10000x5000, 0.87 at
+// 1024x2048, where the ramp of each 51 us launch shows); 16-bit storage by instruction issue
+// (361 per site with the paired tile below).  Cells of both components halve the loads,
+// stores and address arithmetic (FP32 492 -> 323 instructions per site, paired FP16 500 ->
+// 361), a window of TW + 4 FP32 cells needs no alignment slack (34 sectors read per 32
+// owned at 128 columns, 36 before), and a tile whose sweep meets no wall row runs code without the wall
+// checks.  us per step before and after: FP32 54.0 -> 51.4 (1024x2048), 1232 -> 1101
+// (10000x5000); FP16 47.3 -> 36.2, 1024 -> 783; BF16 36.9 -> 27.1 (1501x999).
 // ---------------------------------------------------------------------------
-constexpr int kBlockStages = 5;   // rows y..y+2 in use + 2 rows prefetched (4 stages / 5 blocks per SM measured slower)
+// Row stages of a tile (rows y and y + 1 in use, the others prefetched) and the resident
+// blocks per SM that its registers are limited for.  FP32 (HBM-bound) is fastest with
+// about 800 to 1000 prefetched columns per SM; measured, us per step at 1024x2048 /
+// 10000x5000: 128 columns with 3 stages and 6 blocks 51.4 / 1119, 4 and 5 57.0 / 1273,
+// 5 and 4 57.0 / 1343; 256 columns with 4 stages and 2 blocks 53.3 / 1101, 3 and 3 52.5 /
+// 1145, 5 and 2 57.5 / 1242.
+template <typename T, int TW> struct TileCfg {
+    static constexpr int kStages = TW == 128 ? 3 : 4, kBlocks = TW == 128 ? 6 : 2;
+};
+template <int TW> struct TileCfg<__half, TW> { static constexpr int kStages = 5, kBlocks = 768 / TW; };
+template <int TW> struct TileCfg<__nv_bfloat16, TW> { static constexpr int kStages = 5, kBlocks = 768 / TW; };
+
 template <typename T, int TW = kBlockTileW> struct BlockWin {
-    // TW + 4 columns plus the alignment slack of the window start, in 16-byte units
-    static constexpr int kAlign = 16 / (int)sizeof(T);
-    static constexpr int value = (TW + 4 + kAlign - 1 + kAlign - 1) / kAlign * kAlign;
+    // TW + 4 columns from x0 - 2 plus the alignment slack of the window start, in
+    // 16-byte units; column 0 of a row sits 128 bytes into it and x0 is a multiple of TW
+    static constexpr int kAlign = 16 / (int)sizeof(Cell<T>);
+    static constexpr int kSlack = (128 / (int)sizeof(Cell<T>) - 2) % kAlign;
+    static constexpr int value = (TW + 4 + kSlack + kAlign - 1) / kAlign * kAlign;
 };
 
 template <typename T, int TW = kBlockTileW>
-size_t block_smem_bytes() {
-    return (size_t)kBlockStages * 18 * BlockWin<T, TW>::value * sizeof(T) + kBlockStages * sizeof(uint64_t);
+__host__ __device__ constexpr size_t block_smem_bytes() {
+    return (size_t)TileCfg<T, TW>::kStages * (9 * BlockWin<T, TW>::value * sizeof(Cell<T>) + sizeof(uint64_t));
 }
 
-// Post-streaming stored values of window column k on row yo from the stages
-// holding rows yo-1 (S), yo (C), yo+1 (N) (bounce-back on the wall rows): the
-// populations for FP32 storage, the shifted values h = f - w rho0 for 16-bit.
-template <typename T, int TW>
-__device__ __forceinline__ void pull_block(const T* __restrict__ stS, const T* __restrict__ stC,
-                                           const T* __restrict__ stN, bool bottom, bool top, int k,
-                                           float f[2][9]) {
-    constexpr int W = BlockWin<T, TW>::value;
+// Density ring of a block tile of TW columns, as (B, A): slot 1 + t holds column
+// x0 + t, slots 0 and TW + 1 the halo columns x0 - 1 and x0 + TW.
+template <int TW> using BlockRingT = float2[4][TW + 2];
+
+// Planes of row r that the tile [y0, y1) reads (bit i: direction i): all 9 for its
+// own rows and the wall rows (bounce-back reads the opposite planes); of the halo
+// rows only the populations that stream into the tile or into the density rows y0 - 1
+// and y1: c_y = +1 from y0 - 2, c_y = 0 or +1 from y0 - 1, c_y = 0 or -1 from y1 and
+// c_y = -1 from y1 + 1 (directions 2, 5, 6 move up, 4, 7, 8 down).
+__device__ __forceinline__ uint32_t tile_row_planes(int r, int y0, int y1, int ny) {
+    constexpr uint32_t up = (1u << 2) | (1u << 5) | (1u << 6);
+    constexpr uint32_t mid = (1u << 0) | (1u << 1) | (1u << 3);
+    constexpr uint32_t down = (1u << 4) | (1u << 7) | (1u << 8);
+    if ((r >= y0 && r < y1) || r == 0 || r == ny - 1) return up | mid | down;
+    if (r == y0 - 2) return up;
+    if (r == y0 - 1) return up | mid;
+    if (r == y1) return mid | down;
+    return down;   // y1 + 1
+}
+
+// The densities (A, B) of a site from the sum of its stored values (16-bit storage
+// holds h = f - w rho0, whose sum is rho - rho0).
+template <typename T>
+__device__ __forceinline__ float2 density_of(float2 sum, float2 shift) {
+    if constexpr (IsShifted<T>::value) return add2(shift, sum);
+    else return sum;
+}
+template <typename C>
+__device__ __forceinline__ float2 sum_cells(const C c[9]) {
+    float2 v[9];
 #pragma unroll
-    for (int s = 0; s < 2; ++s) {
+    for (int i = 0; i < 9; ++i) v[i] = to_f2(c[i]);
+    return sum9_2(v);
+}
+// Collide a site's stored cells (sum: their sum) into the cells to store.
+template <typename T, bool kWalls>
+__device__ __forceinline__ bool collide_cells(const Cell<T> cur[9], float2 sum, const Nbr2& p, int ny, const Physics& ph,
+                                              int y, uint32_t site, uint32_t seed, Cell<T> out[9]) {
+    float2 v[9];
 #pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            const int pl = s * 9 + i;
-            T v;
-            if (cy(i) == 0) {
-                v = stC[pl * W + k - cx(i)];
-            } else if (cy(i) == 1) {
-                v = bottom ? stC[(s * 9 + opp(i)) * W + k] : stS[pl * W + k - cx(i)];
-            } else {
-                v = top ? stC[(s * 9 + opp(i)) * W + k] : stN[pl * W + k - cx(i)];
-            }
-            f[s][i] = to_f<T>(v);
+    for (int i = 0; i < 9; ++i) v[i] = to_f2(cur[i]);
+    bool ok;
+    if constexpr (IsShifted<T>::value) {
+        ok = collide_shifted<kWalls>(v, sum, p, ph, y, ny);
+        round_site<T>(site, v, seed, out);
+    } else {
+        ok = collide_site<true, kWalls>(v, sum, p, ph, y, ny);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) out[i] = v[i];
+    }
+    return ok;
+}
+
+// The row stages of one tile.  A stage holds what the pull of one row reads: of each
+// direction the plane row that streams into it (row r - c_y of direction i for the pull of
+// row r, or the row's own opposite plane where that lies beyond a wall), so that a row
+// occupies one stage, not the three its source rows would, and every stage is one full
+// set of 9 copies.  The pulls are of rows y0 - 1 .. y1, row r in stage (r - y0 + 1) mod S.
+// dsm: S stages of 9 planes, then the S mbarriers.
+template <typename T, int TW, int S, bool kWithhold>
+struct TileRows {
+    typedef Cell<T> C;
+    static constexpr int W = BlockWin<T, TW>::value;
+    static constexpr int kCells = 9 * W;   // per stage
+    static constexpr int kStages = S;
+    C* stage;
+    uint64_t* bar;
+    const C* win;   // the window's start in row 0 of plane 0
+    size_t plane;
+    int y0, y1, ny, pitch;
+    int* flag;
+
+    __device__ __forceinline__ TileRows(const C* fin, const Grid& g, int x0, int y0_, int y1_, unsigned char* dsm, int* flag_)
+        : plane(g.plane), y0(y0_), y1(y1_), ny(g.ny), pitch(g.pitch), flag(flag_) {
+        stage = reinterpret_cast<C*>(dsm);
+        bar = reinterpret_cast<uint64_t*>(dsm + (size_t)S * kCells * sizeof(C));
+        win = fin + (g.origin + x0 - 2 - BlockWin<T, TW>::kSlack);
+        if (threadIdx.x == 0) {
+#pragma unroll 1
+            for (int j = 0; j < S; ++j) mbar_init(&bar[j], 1);
+            mbar_fence_init();
         }
+        __syncthreads();
+        if (threadIdx.x < 32) {
+#pragma unroll 1
+            for (int j = 0; j < S; ++j) issue(y0 - 1 + j, j);
+        }
+    }
+    // the pull of row r into stage j (warp 0, all lanes; one direction per lane); a virtual
+    // wall row has nothing to copy, its stage's phase completes at once
+    __device__ __forceinline__ void issue(int r, int j) {
+        if constexpr (kWithhold) return;
+        if (r > y1) return;
+        const bool real = r >= 0 && r < ny;
+        constexpr uint32_t bytes = W * sizeof(C);
+        if (threadIdx.x == 0) mbar_expect_tx(&bar[j], real ? 9 * bytes : 0u);
+        __syncwarp();
+        const int i = threadIdx.x;
+        if (i < 9 && real) {
+            // directions 2, 5, 6 move up, 4, 7, 8 down
+            const int c = (0x64 >> i & 1) - (0x190 >> i & 1);
+            const bool inside = r - c >= 0 && r - c < ny;
+            const int row = inside ? r - c : r, pl = inside ? i : opp(i);
+            bulk_copy_g2s(stage + j * kCells + i * W, win + (size_t)pl * plane + (size_t)row * pitch, bytes, &bar[j]);
+        }
+    }
+    __device__ __forceinline__ void wait_stage(int j, uint32_t phase) {
+        mbar_wait(&bar[j], phase, flag, kWithhold ? kTestWaitLimit : kWaitLimit);
+    }
+};
+// Post-streaming cells of window column k from the stage of a row's pull (W columns per
+// plane); bounced-back populations come from the column itself.
+template <int W, typename C>
+__device__ __forceinline__ void pull_stage(const C* __restrict__ st, bool bottom, bool top, int k, C f[9]) {
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        const bool bounced = (cy(i) == 1 && bottom) || (cy(i) == -1 && top);
+        f[i] = st[i * W + (bounced ? k : k - cx(i))];
     }
 }
 
-// Density ring of a block tile of TW columns: slot 1 + t holds column x0 + t, slots
-// 0 and TW + 1 the halo columns x0 - 1 and x0 + TW.
-template <int TW> using BlockRingT = float[4][2][TW + 2];
-typedef BlockRingT<kBlockTileW> BlockRing;
+// A sweep over the rows of a tile, bottom up, one block barrier per row.
+// densities(yo, st): the densities of row yo into the ring, from its stage (yo may be a
+// virtual wall row); collide(y, st): row y.  Row y + 1's densities are taken before the
+// barrier and row y collided after it, so a row's populations are pulled twice: holding
+// them in registers from one iteration to the next instead takes a loop unrolled over
+// two rows, whose code (41 KB for the paired tile) outgrew the instruction cache, and 36
+// registers.  The two iterations before the tile's first row run without a collision: the
+// code stays one copy.
+template <typename Rows, typename Densities, typename Collide>
+__device__ __forceinline__ void sweep_tile(Rows& R, Densities densities, Collide collide) {
+    constexpr int S = Rows::kStages;
+    const int y1 = R.y1;
+    // pc, pn: the stages of rows y and y + 1; jn that of row y + 1, and the phase of the wait
+    // for it, which flips whenever the stage wraps to 0
+    const auto *pc = R.stage, *pn = R.stage;
+    int jn = 0;
+    uint32_t phase = 0;
+#pragma unroll 1
+    for (int y = R.y0 - 2; y < y1; ++y) {
+        R.wait_stage(jn, phase);
+        densities(y + 1, pn);
+        __syncthreads();
+        // every thread is past its reads of rows < y: refill the stage of row y - 1
+        if (threadIdx.x < 32 && y >= R.y0) {
+            fence_proxy_async_smem();
+            R.issue(y - 1 + S, jn >= 2 ? jn - 2 : jn - 2 + S);
+        }
+        if (y >= R.y0) collide(y, pc);
+        pc = pn;
+        pn += Rows::kCells;
+        if (++jn == S) {
+            jn = 0;
+            pn = R.stage;
+            phase ^= 1u;
+        }
+    }
+}
+// Whether a tile's sweep reaches a wall row: its pulls are of rows y0 - 1 .. y1.
+__device__ __forceinline__ bool tile_has_walls(int y0, int y1, int ny) { return y0 < 2 || y1 > ny - 2; }
 
 // One block tile: columns [x0, x0 + TW) and rows [y0, y1) of one grid, TW threads.
 // dsm: the block_smem_bytes<T, TW>() of dynamic shared memory (row stages, then
 // the mbarriers).  kWithhold (the timeout test's instantiation only): no row copy is
 // issued and each wait gives up after kTestWaitLimit polls, so every wait of the tile
 // runs out with nothing in flight.
-constexpr uint32_t kTestWaitLimit = 4096;
-template <typename T, int TW = kBlockTileW, bool kWithhold = false>
-__device__ __forceinline__ void block_tile(const T* __restrict__ fin, T* __restrict__ fout, const Grid& g,
-                                           const Physics& ph, int x0, int y0, int y1, unsigned char* dsm,
-                                           BlockRingT<TW>& sR, uint32_t seed, int* flag) {
-    constexpr int W = BlockWin<T, TW>::value;
-    constexpr int kAlign = BlockWin<T, TW>::kAlign;
-    T* stage = reinterpret_cast<T*>(dsm);
-    uint64_t* bar = reinterpret_cast<uint64_t*>(dsm + (size_t)kBlockStages * 18 * W * sizeof(T));
+template <typename T, int TW, bool kWalls, bool kWithhold>
+__device__ __forceinline__ void block_sweep(const Cell<T>* __restrict__ fin, Cell<T>* __restrict__ fout, const Grid& g,
+                                            const Physics& ph, int x0, int y0, int y1, unsigned char* dsm,
+                                            BlockRingT<TW>& sR, uint32_t seed, int* flag) {
+    typedef Cell<T> C;
+    constexpr int W = BlockWin<T, TW>::value, slack = BlockWin<T, TW>::kSlack, S = TileCfg<T, TW>::kStages;
+    TileRows<T, TW, S, kWithhold> R(fin, g, x0, y0, y1, dsm, flag);
     const int t = threadIdx.x;
-    const int rfirst = max(y0 - 2, 0);
-    const int rlast = min(y1 + 1, g.ny - 1);
     const int x = x0 + t;
     const bool owner = x < g.nx;
-    const bool dens = x <= g.nx;   // column nx is the periodic ghost of column 0
-    const int e0 = g.origin + x0 - 2;
-    const int slack = e0 % kAlign;
+    const bool edge = x < 2 || x >= g.nx - 2;
     const int k = t + 2 + slack;
     // threads 64 / 65: the halo columns x0 - 1 / x0 + TW (window columns 1 / TW + 2 + slack)
     const bool halo = t == 64 || t == 65;
     const int kh = t == 64 ? 1 + slack : TW + 2 + slack;
     const int sh = t == 64 ? 0 : TW + 1;
-    const T* win = fin + (e0 - slack);
-    const float shift[2] = {ph.shift[0], ph.shift[1]};
-    const uint32_t row_bytes = W * sizeof(T);
-
-    if (t == 0) {
-        for (int j = 0; j < kBlockStages; ++j) mbar_init(&bar[j], 1);
-        mbar_fence_init();
-    }
-    __syncthreads();
-    int next = rfirst;  // next row to issue (every lane of warp 0 keeps the same count)
-    // Planes of row r the tile reads (bit p: plane p = 9 s + i).  The tile's own rows
-    // and the wall rows (bounce-back reads the opposite planes) take all 18; of the
-    // halo rows only the populations that stream into the tile or into the density
-    // rows y0 - 1 and y1: c_y = +1 from y0 - 2, c_y = 0 or +1 from y0 - 1, c_y = 0 or
-    // -1 from y1, c_y = -1 from y1 + 1 (directions 2, 5, 6 move up, 4, 7, 8 down).
-    auto planes_of = [&](int r) -> uint32_t {
-        constexpr uint32_t both = 1u | (1u << 9);
-        constexpr uint32_t up = ((1u << 2) | (1u << 5) | (1u << 6)) * both;
-        constexpr uint32_t mid = ((1u << 0) | (1u << 1) | (1u << 3)) * both;
-        constexpr uint32_t down = ((1u << 4) | (1u << 7) | (1u << 8)) * both;
-        if ((r >= y0 && r < y1) || r == 0 || r == g.ny - 1) return up | mid | down;
-        if (r == y0 - 2) return up;
-        if (r == y0 - 1) return up | mid;
-        if (r == y1) return mid | down;
-        return down;   // y1 + 1
-    };
-    auto issue = [&](int r) {   // warp 0, all lanes
-        if constexpr (kWithhold) return;
-        const int j = (r - rfirst) % kBlockStages;
-        uint64_t* b = &bar[j];
-        const uint32_t planes = planes_of(r);
-        if (t == 0) mbar_expect_tx(b, (uint32_t)__popc(planes) * row_bytes);
-        __syncwarp();
-        if (t < 18 && ((planes >> t) & 1u))
-            bulk_copy_g2s(stage + (size_t)j * 18 * W + t * W, win + (size_t)r * g.pitch + (size_t)t * g.plane,
-                          row_bytes, b);
-    };
-    if (t < 32)
-        for (; next <= rlast && next < rfirst + kBlockStages; ++next) issue(next);
-    auto wait_row = [&](int r) {
-        if (r >= rfirst && r <= rlast)
-            mbar_wait(&bar[(r - rfirst) % kBlockStages], (uint32_t)(((r - rfirst) / kBlockStages) & 1), flag,
-                      kWithhold ? kTestWaitLimit : kWaitLimit);
-    };
-    auto stage_of = [&](int r) -> const T* {
-        const int rr = min(max(r, rfirst), rlast);
-        return stage + (size_t)((rr - rfirst) % kBlockStages) * 18 * W;
-    };
-    // pull of row yo from the stages of rows yo - 1 (S), yo (C), yo + 1 (N)
-    auto pull_row = [&](int yo, const T* sS, const T* sC, const T* sN, int kk, float f[2][9]) {
-        if (yo > 0 && yo < g.ny - 1)   // interior row (uniform over the block): no bounce-back selects
-            pull_block<T, TW>(sS, sC, sN, false, false, kk, f);
-        else
-            pull_block<T, TW>(sS, sC, sN, yo == 0, yo == g.ny - 1, kk, f);
-    };
-    // densities of row yo into ring slot yo & 3 (zero for columns past nx); 16-bit
-    // storage holds h = f - w rho0, whose sum is rho - rho0
-    auto density = [&](const float* f, int s) {
-        if constexpr (IsShifted<T>::value) return sum9(f) + shift[s];
-        else return sum9(f);
-    };
-    auto densities = [&](int yo, const T* sS, const T* sC, const T* sN, float f[2][9]) {
-        pull_row(yo, sS, sC, sN, k, f);
-        const int sl = yo & 3;
-        sR[sl][0][t + 1] = dens ? density(f[0], 0) : 0.0f;
-        sR[sl][1][t + 1] = dens ? density(f[1], 1) : 0.0f;
+    const float2 shift = shift_of(ph);
+    C* q = fout + (size_t)y0 * g.pitch + g.origin + x;
+    uint32_t site = site_index(g, y0, x);
+    const uint32_t site_row = site_index(g, 1, x) - site_index(g, 0, x);
+    bool good = true;
+    float2 sum = splat(0.0f), next = splat(0.0f);   // sums of the stored values of rows y, y + 1
+    // densities of columns past nx are never read by an owner
+    auto densities = [&](int yo, const C* st) {
+        float2* ring = sR[yo & 3];
+        sum = next;
+        if (kWalls && (yo < 0 || yo >= g.ny)) {   // a virtual wall row
+            ring[t + 1] = splat(0.0f);
+            if (halo) ring[sh] = splat(0.0f);
+            return;
+        }
+        const bool bottom = kWalls && yo == 0, top = kWalls && yo == g.ny - 1;
+        C f[9];
+        pull_stage<W>(st, bottom, top, k, f);
+        next = sum_cells(f);
+        ring[t + 1] = swap2(density_of<T>(next, shift));
         if (halo) {
-            float fh[2][9];
-            pull_row(yo, sS, sC, sN, kh, fh);
-            sR[sl][0][sh] = density(fh[0], 0);
-            sR[sl][1][sh] = density(fh[1], 1);
+            pull_stage<W>(st, bottom, top, kh, f);
+            ring[sh] = swap2(density_of<T>(sum_cells(f), shift));
         }
     };
-
-    float fa[2][9], fb[2][9];
-    if (y0 > 0) {   // densities of row y0 - 1 (zero on the virtual wall row)
-        wait_row(y0 - 2); wait_row(y0 - 1); wait_row(y0);
-        densities(y0 - 1, stage_of(y0 - 2), stage_of(y0 - 1), stage_of(y0), fb);
-    } else {
-        const int sl = (y0 - 1) & 3;
-        sR[sl][0][t + 1] = 0.0f; sR[sl][1][t + 1] = 0.0f;
-        if (halo) { sR[sl][0][sh] = 0.0f; sR[sl][1][sh] = 0.0f; }
-    }
-    wait_row(y0 - 1); wait_row(y0); wait_row(y0 + 1);
-    densities(y0, stage_of(y0 - 1), stage_of(y0), stage_of(y0 + 1), fa);
-    // everybody is past the prologue's reads of row y0 - 2: its stage can take row y0 + 3
-    __syncthreads();
-    if (t < 32) {
-        fence_proxy_async_smem();
-        for (; next <= rlast && next - kBlockStages <= y0 - 2; ++next) issue(next);
-    }
-
-    // jy: the stage of row y, advanced by one per row without a division.  Rows y .. y + 2
-    // sit in it and the two stages after it; a row beyond rlast maps to some stage, but
-    // its pull is not read (bounce-back on the top wall row takes the centre row instead).
-    constexpr size_t kStageElems = (size_t)18 * W;
-    // pq: the phase of the wait for row y + 2 in stage jq
-    auto row = [&](int y, int jy, uint32_t pq, float cur[2][9], float nxt[2][9]) {
-        if (y + 1 < g.ny) {
-            const int jp = jy == kBlockStages - 1 ? 0 : jy + 1;
-            const int jq = jp == kBlockStages - 1 ? 0 : jp + 1;
-            if (y + 2 <= rlast) mbar_wait(&bar[jq], pq, flag, kWithhold ? kTestWaitLimit : kWaitLimit);
-            densities(y + 1, stage + jy * kStageElems, stage + jp * kStageElems, stage + jq * kStageElems, nxt);
-        } else {
-            const int sl = (y + 1) & 3;
-            sR[sl][0][t + 1] = 0.0f; sR[sl][1][t + 1] = 0.0f;
-            if (halo) { sR[sl][0][sh] = 0.0f; sR[sl][1][sh] = 0.0f; }
-        }
-        __syncthreads();
-        // every thread is past its reads of rows < y: refill those stages
-        if (t < 32) {
-            fence_proxy_async_smem();
-            for (; next <= rlast && next - kBlockStages <= y - 1; ++next) issue(next);
-        }
+    auto collide = [&](int y, const C* st) {
         if (owner) {
-            const int s0 = (y - 1) & 3, s1 = y & 3, s2 = (y + 1) & 3;
-            const int c = t + 1;
-            Nbr pA, pB;
-            pA.E = sR[s1][0][c + 1]; pA.W = sR[s1][0][c - 1];
-            pA.N = sR[s2][0][c];     pA.S = sR[s0][0][c];
-            pA.NE = sR[s2][0][c + 1]; pA.NW = sR[s2][0][c - 1];
-            pA.SE = sR[s0][0][c + 1]; pA.SW = sR[s0][0][c - 1];
-            pB.E = sR[s1][1][c + 1]; pB.W = sR[s1][1][c - 1];
-            pB.N = sR[s2][1][c];     pB.S = sR[s0][1][c];
-            pB.NE = sR[s2][1][c + 1]; pB.NW = sR[s2][1][c - 1];
-            pB.SE = sR[s0][1][c + 1]; pB.SW = sR[s0][1][c - 1];
-            if constexpr (IsShifted<T>::value) {
-                collide_shifted(cur, pA, pB, ph, y, g.ny, flag);
-                store_site_sr<T>(fout, g, y, x, cur, seed);
-            } else {
-                collide_site<true>(cur, pA, pB, ph, y, g.ny, flag);
-                store_site<T>(fout, g, y, x, cur, shift);
+            C f[9];
+            pull_stage<W>(st, kWalls && y == 0, kWalls && y == g.ny - 1, k, f);
+            good &= collide_cells<T, kWalls>(f, sum, ring_nbr(sR[(y - 1) & 3], sR[y & 3], sR[(y + 1) & 3], t + 1), g.ny, ph,
+                                             y, site, seed, f);
+#pragma unroll
+            for (int i = 0; i < 9; ++i) q[(size_t)i * g.plane] = f[i];
+            if (edge) {   // periodic ghost copy
+                C* qg = q + (x < 2 ? g.nx : -g.nx);
+#pragma unroll
+                for (int i = 0; i < 9; ++i) qg[(size_t)i * g.plane] = f[i];
             }
         }
+        q += g.pitch;
+        site += site_row;
     };
-    // row r waits for fill (r - rfirst) / kBlockStages of its stage: the phase flips
-    // whenever the waited row's stage wraps to 0, i.e. after a row whose own stage is
-    // kBlockStages - 3
-    int jy = y0 - rfirst;
-    uint32_t pq = (uint32_t)(((y0 + 2 - rfirst) / kBlockStages) & 1);
-    for (int y = y0; y < y1; y += 2) {
-        const int jn = jy == kBlockStages - 1 ? 0 : jy + 1;
-        row(y, jy, pq, fa, fb);
-        pq ^= (uint32_t)(jy == kBlockStages - 3);
-        if (y + 1 < y1) row(y + 1, jn, pq, fb, fa);
-        pq ^= (uint32_t)(jn == kBlockStages - 3);
-        jy = jn == kBlockStages - 1 ? 0 : jn + 1;
-    }
+    sweep_tile(R, densities, collide);
+    if (!good) atomicOr(flag, 1);
+}
+template <typename T, int TW = kBlockTileW, bool kWithhold = false>
+__device__ __forceinline__ void block_tile(const Cell<T>* __restrict__ fin, Cell<T>* __restrict__ fout, const Grid& g,
+                                           const Physics& ph, int x0, int y0, int y1, unsigned char* dsm,
+                                           BlockRingT<TW>& sR, uint32_t seed, int* flag) {
+    if (kWithhold || tile_has_walls(y0, y1, g.ny))
+        block_sweep<T, TW, true, kWithhold>(fin, fout, g, ph, x0, y0, y1, dsm, sR, seed, flag);
+    else
+        block_sweep<T, TW, false, kWithhold>(fin, fout, g, ph, x0, y0, y1, dsm, sR, seed, flag);
 }
 
 // ---------------------------------------------------------------------------
@@ -762,7 +757,7 @@ __device__ __forceinline__ void block_tile(const T* __restrict__ fin, T* __restr
 // 31 pull those as well), in a density ring of its own, and a stage is handed back
 // through an "empty" mbarrier on which each warp arrives once it no longer reads
 // the stage's row.  A warp waits only for the rows it reads (full barriers); warp
-// 0, whose lanes 0-17 issue the copies, also waits until every warp has handed back
+// 0, whose lanes 0-8 issue the copies, also waits until every warp has handed back
 // the stage it refills.  Stage indices and barrier phases advance incrementally,
 // without a division by the stage count.
 // ---------------------------------------------------------------------------
@@ -772,55 +767,35 @@ template <> struct DecCfg<__nv_bfloat16, kWideTileW> { static constexpr int kSta
 
 template <typename T, int TW>
 size_t dec_smem_bytes() {
-    return (size_t)DecCfg<T, TW>::kStages * (18 * BlockWin<T, TW>::value * sizeof(T) + 2 * sizeof(uint64_t));
+    return (size_t)DecCfg<T, TW>::kStages * (9 * BlockWin<T, TW>::value * sizeof(Cell<T>) + 2 * sizeof(uint64_t));
 }
-template <int TW> using DecRingT = float[TW / 32][4][2][34];
-
-// Planes of row r that the tile [y0, y1) reads (bit p: plane p = 9 s + i): all 18 for
-// its own rows and the wall rows (bounce-back reads the opposite planes); of the halo
-// rows only the populations that stream into the tile or into the density rows y0 - 1
-// and y1: c_y = +1 from y0 - 2, c_y = 0 or +1 from y0 - 1, c_y = 0 or -1 from y1 and
-// c_y = -1 from y1 + 1 (directions 2, 5, 6 move up, 4, 7, 8 down).
-__device__ __forceinline__ uint32_t tile_row_planes(int r, int y0, int y1, int ny) {
-    constexpr uint32_t both = 1u | (1u << 9);
-    constexpr uint32_t up = ((1u << 2) | (1u << 5) | (1u << 6)) * both;
-    constexpr uint32_t mid = ((1u << 0) | (1u << 1) | (1u << 3)) * both;
-    constexpr uint32_t down = ((1u << 4) | (1u << 7) | (1u << 8)) * both;
-    if ((r >= y0 && r < y1) || r == 0 || r == ny - 1) return up | mid | down;
-    if (r == y0 - 2) return up;
-    if (r == y0 - 1) return up | mid;
-    if (r == y1) return mid | down;
-    return down;   // y1 + 1
-}
+template <int TW> using DecRingT = float2[TW / 32][4][34];
 
 template <typename T, int TW>
-__device__ __forceinline__ void dec_tile(const T* __restrict__ fin, T* __restrict__ fout, const Grid& g,
+__device__ __forceinline__ void dec_tile(const Cell<T>* __restrict__ fin, Cell<T>* __restrict__ fout, const Grid& g,
                                          const Physics& ph, int x0, int y0, int y1, unsigned char* dsm,
                                          DecRingT<TW>& sR, uint32_t seed, int* flag) {
-    constexpr int W = BlockWin<T, TW>::value;
-    constexpr int kAlign = BlockWin<T, TW>::kAlign;
+    typedef Cell<T> C;
+    constexpr int W = BlockWin<T, TW>::value, slack = BlockWin<T, TW>::kSlack;
     constexpr int S = DecCfg<T, TW>::kStages;
     constexpr int NW = TW / 32;
-    T* stage = reinterpret_cast<T*>(dsm);
-    uint64_t* full = reinterpret_cast<uint64_t*>(dsm + (size_t)S * 18 * W * sizeof(T));
+    C* stage = reinterpret_cast<C*>(dsm);
+    uint64_t* full = reinterpret_cast<uint64_t*>(dsm + (size_t)S * 9 * W * sizeof(C));
     uint64_t* empty = full + S;
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
     const int rfirst = max(y0 - 2, 0);
     const int rlast = min(y1 + 1, g.ny - 1);
     const int x = x0 + t;
     const bool owner = x < g.nx;
-    const bool dens = x <= g.nx;   // column nx is the periodic ghost of column 0
-    const int e0 = g.origin + x0 - 2;
-    const int slack = e0 % kAlign;
     const int k = t + 2 + slack;
     // lanes 0 / 31 also supply the densities of the columns beside the warp
     const bool halo = lane == 0 || lane == 31;
     const int kh = lane == 0 ? k - 1 : k + 1;
     const int sh = lane == 0 ? 0 : 33;
-    const T* win = fin + (e0 - slack);
-    const float shift[2] = {ph.shift[0], ph.shift[1]};
-    const uint32_t row_bytes = W * sizeof(T);
-    float(&ring)[4][2][34] = sR[wid];
+    const C* win = fin + (g.origin + x0 - 2 - slack);
+    const float2 shift = shift_of(ph);
+    const uint32_t row_bytes = W * sizeof(C);
+    float2(&ring)[4][34] = sR[wid];
 
     if (t == 0) {
         for (int j = 0; j < S; ++j) {
@@ -841,9 +816,9 @@ __device__ __forceinline__ void dec_tile(const T* __restrict__ fin, T* __restric
         const uint32_t planes = tile_row_planes(next, y0, y1, g.ny);
         if (lane == 0) mbar_expect_tx(&full[nj], (uint32_t)__popc(planes) * row_bytes);
         __syncwarp();
-        if (lane < 18 && ((planes >> lane) & 1u)) {
+        if (lane < 9 && ((planes >> lane) & 1u)) {
             fence_proxy_async_smem();
-            bulk_copy_g2s(stage + (size_t)nj * 18 * W + lane * W, win + (size_t)next * g.pitch + (size_t)lane * g.plane,
+            bulk_copy_g2s(stage + (size_t)nj * 9 * W + lane * W, win + (size_t)next * g.pitch + (size_t)lane * g.plane,
                           row_bytes, &full[nj]);
         }
         ++next;
@@ -873,45 +848,38 @@ __device__ __forceinline__ void dec_tile(const T* __restrict__ fin, T* __restric
             if (++rj == S) rj = 0;
         }
     };
-    // stage of row r (rfirst <= r <= rlast), from the stage jc of a row rc near it
-    auto stage_ptr = [&](int j) -> const T* { return stage + (size_t)j * 18 * W; };
+    auto stage_ptr = [&](int j) -> const C* { return stage + (size_t)j * 9 * W; };
     auto wrap = [&](int j) { return j < 0 ? j + S : (j >= S ? j - S : j); };
     // pull of row yo whose own stage is jc (rows yo - 1 / yo + 1 in the stages beside it)
-    auto pull_row = [&](int yo, int jc, int kk, float f[2][9]) {
-        const T* sS = stage_ptr(wrap(jc - 1));
-        const T* sC = stage_ptr(jc);
-        const T* sN = stage_ptr(wrap(jc + 1));
+    auto pull_row = [&](int yo, int jc, int kk, C f[9]) {
+        const C* sS = stage_ptr(wrap(jc - 1));
+        const C* sC = stage_ptr(jc);
+        const C* sN = stage_ptr(wrap(jc + 1));
         if (yo > 0 && yo < g.ny - 1)
-            pull_block<T, TW>(sS, sC, sN, false, false, kk, f);
+            pull_cells<W>(sS, sC, sN, false, false, kk, f);
         else
-            pull_block<T, TW>(sS, sC, sN, yo == 0, yo == g.ny - 1, kk, f);
+            pull_cells<W>(sS, sC, sN, yo == 0, yo == g.ny - 1, kk, f);
     };
-    auto density = [&](const float* f, int s) {
-        if constexpr (IsShifted<T>::value) return sum9(f) + shift[s];
-        else return sum9(f);
-    };
-    auto densities = [&](int yo, int jc, float f[2][9]) {
+    auto densities = [&](int yo, int jc, C f[9]) -> float2 {
         pull_row(yo, jc, k, f);
-        const int sl = yo & 3;
-        ring[sl][0][lane + 1] = dens ? density(f[0], 0) : 0.0f;
-        ring[sl][1][lane + 1] = dens ? density(f[1], 1) : 0.0f;
+        const float2 sum = sum_cells(f);
+        ring[yo & 3][lane + 1] = swap2(density_of<T>(sum, shift));
         if (halo) {
-            float fh[2][9];
+            C fh[9];
             pull_row(yo, jc, kh, fh);
-            ring[sl][0][sh] = density(fh[0], 0);
-            ring[sl][1][sh] = density(fh[1], 1);
+            ring[yo & 3][sh] = swap2(density_of<T>(sum_cells(fh), shift));
         }
+        return sum;
     };
     auto zero_row = [&](int yo) {   // the virtual wall rows y = -1 and y = ny
-        const int sl = yo & 3;
-        ring[sl][0][lane + 1] = 0.0f;
-        ring[sl][1][lane + 1] = 0.0f;
-        if (halo) { ring[sl][0][sh] = 0.0f; ring[sl][1][sh] = 0.0f; }
+        ring[yo & 3][lane + 1] = splat(0.0f);
+        if (halo) ring[yo & 3][sh] = splat(0.0f);
     };
 
     // jn: stage of row y + 1 during the collision of row y (rows are consecutive from
     // rfirst, so the stage of row r is (r - rfirst) mod S)
-    float fa[2][9], fb[2][9];
+    C fa[9], fb[9];
+    float2 da, db = splat(0.0f);
     int jy = (y0 - rfirst) % S;   // stage of row y0 (a one-time division)
     if (y0 > 0) {
         wait_upto(y0);
@@ -920,16 +888,16 @@ __device__ __forceinline__ void dec_tile(const T* __restrict__ fin, T* __restric
         zero_row(y0 - 1);
     }
     wait_upto(y0 + 1);
-    densities(y0, jy, fa);
+    da = densities(y0, jy, fa);
     release_upto(y0 - 2);
     if (wid == 0)
         while (next <= rlast && next - S <= y0 - 2) issue_next();
     int jn = wrap(jy + 1);
 
-    auto row = [&](int y, float cur[2][9], float nxt[2][9]) {
+    auto row = [&](int y, const C cur[9], float2 dcur, C nxt[9], float2& dnxt) {
         if (y + 1 < g.ny) {
             wait_upto(y + 2);
-            densities(y + 1, jn, nxt);
+            dnxt = densities(y + 1, jn, nxt);
         } else {
             zero_row(y + 1);
         }
@@ -938,35 +906,22 @@ __device__ __forceinline__ void dec_tile(const T* __restrict__ fin, T* __restric
             while (next <= rlast && next - S <= y - 1) issue_next();
         jn = wrap(jn + 1);
         if (owner) {
-            const int s0 = (y - 1) & 3, s1 = y & 3, s2 = (y + 1) & 3;
-            const int c = lane + 1;
-            Nbr pA, pB;
-            pA.E = ring[s1][0][c + 1]; pA.W = ring[s1][0][c - 1];
-            pA.N = ring[s2][0][c];     pA.S = ring[s0][0][c];
-            pA.NE = ring[s2][0][c + 1]; pA.NW = ring[s2][0][c - 1];
-            pA.SE = ring[s0][0][c + 1]; pA.SW = ring[s0][0][c - 1];
-            pB.E = ring[s1][1][c + 1]; pB.W = ring[s1][1][c - 1];
-            pB.N = ring[s2][1][c];     pB.S = ring[s0][1][c];
-            pB.NE = ring[s2][1][c + 1]; pB.NW = ring[s2][1][c - 1];
-            pB.SE = ring[s0][1][c + 1]; pB.SW = ring[s0][1][c - 1];
-            if constexpr (IsShifted<T>::value) {
-                collide_shifted(cur, pA, pB, ph, y, g.ny, flag);
-                store_site_sr<T>(fout, g, y, x, cur, seed);
-            } else {
-                collide_site<true>(cur, pA, pB, ph, y, g.ny, flag);
-                store_site<T>(fout, g, y, x, cur, shift);
-            }
+            C out[9];
+            if (!collide_cells<T, true>(cur, dcur, ring_nbr(ring[(y - 1) & 3], ring[y & 3], ring[(y + 1) & 3], lane + 1),
+                                        g.ny, ph, y, site_index(g, y, x), seed, out))
+                atomicOr(flag, 1);
+            store_cells(fout, g, y, x, out);
         }
     };
     for (int y = y0; y < y1; y += 2) {
-        row(y, fa, fb);
-        if (y + 1 < y1) row(y + 1, fb, fa);
+        row(y, fa, da, fb, db);
+        if (y + 1 < y1) row(y + 1, fb, db, fa, da);
     }
 }
 
 template <typename T, int TW>
 __global__ void __launch_bounds__(TW, 512 / TW)
-step_dec_kernel(const T* __restrict__ fin, T* __restrict__ fout, Grid g, Physics ph, int* flag) {
+step_dec_kernel(const Cell<T>* __restrict__ fin, Cell<T>* __restrict__ fout, Grid g, Physics ph, int* flag) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ DecRingT<TW> sR;
     const int y0 = (int)(((long long)blockIdx.y * g.ny) / gridDim.y);
@@ -981,256 +936,145 @@ step_dec_kernel(const T* __restrict__ fin, T* __restrict__ fout, Grid g, Physics
 // block_tile with tiles of kWideTileW columns, but half as many threads: thread t
 // owns the neighbouring columns x0 + 2t and x0 + 2t + 1.  The per-row work that does
 // not depend on the site (the waits, stage addressing, the block barrier, the copy
-// issue, loop control) is then shared by two sites, and a column pair's stores are
-// one 32-bit store per plane.  Registers stay low because a site's populations are
-// pulled again after the barrier (the densities pass before it keeps only sums), so
-// a stage is refilled only once the row two below the current one is done with: one
-// row less of prefetch than block_tile.
-// The arithmetic, and the stochastic rounding's random bits, are those of
-// block_tile: the results are identical bit for bit.
+// issue, loop control, constants) is then shared by two sites, and a column pair's
+// cells are one 64-bit store per direction.  The arithmetic, and the stochastic
+// rounding's random bits, are those of block_tile: the results are identical bit for
+// bit.
 // ---------------------------------------------------------------------------
 constexpr int kPairThreads = kWideTileW / 2;
-template <typename T> using PairRingT = float[4][2][kWideTileW + 2];
+constexpr int kPairStages = 5;
+// Densities as (B, A): slot 2 + c holds column x0 + c (a thread's pair 16-byte
+// aligned), slots 1 and kWideTileW + 2 the halo columns.
+typedef float2 PairRing[4][kWideTileW + 4];
 
 template <typename T>
 __host__ __device__ constexpr size_t pair_smem_bytes() {
-    return (size_t)kBlockStages * 18 * BlockWin<T, kWideTileW>::value * sizeof(T) + kBlockStages * sizeof(uint64_t);
+    return (size_t)kPairStages * (9 * BlockWin<T, kWideTileW>::value * sizeof(Cell<T>) + sizeof(uint64_t));
 }
 
-// The 18 values of site (x, y) with store_site_sr's random bits added below the
-// 16-bit mantissa: rounding them toward zero gives store_site_sr's stochastic rounding.
-template <typename T> struct SrBits;
-template <> struct SrBits<__half> { static constexpr int kDrop = 13; };
-template <> struct SrBits<__nv_bfloat16> { static constexpr int kDrop = 16; };
+template <typename C> __device__ __forceinline__ C cell_of_bits(uint32_t v) { return *reinterpret_cast<const C*>(&v); }
+template <typename C> __device__ __forceinline__ uint32_t bits_of_cell(C v) { return *reinterpret_cast<const uint32_t*>(&v); }
 
-template <typename T>
-__device__ __forceinline__ void dither_site(const Grid& g, int y, int x, const float h[2][9], uint32_t seed,
-                                            float d[2][9]) {
-    const uint32_t site = g.nx_total > 0 ? (uint32_t)y * (uint32_t)g.nx_total + (uint32_t)(g.x_offset + x)
-                                         : (uint32_t)y * (uint32_t)g.nx + (uint32_t)x;
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-        uint32_t r = hash_lowbias32((site * 2u + (uint32_t)s) ^ seed);
-#pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            r = r * 747796405u + 2891336453u;
-            d[s][i] = __uint_as_float(__float_as_uint(h[s][i]) + (r >> (32 - SrBits<T>::kDrop)));
-        }
-    }
-}
-
-// Two values rounded toward zero and packed: lo in bits 0-15, hi in bits 16-31.
-template <typename T> __device__ __forceinline__ uint32_t pack_rz(float lo, float hi);
-template <> __device__ __forceinline__ uint32_t pack_rz<__half>(float lo, float hi) {
-    uint32_t d;
-    asm("cvt.rz.f16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
-    return d;
-}
-template <> __device__ __forceinline__ uint32_t pack_rz<__nv_bfloat16>(float lo, float hi) {
-    uint32_t d;
-    asm("cvt.rz.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
-    return d;
-}
-template <typename T> __device__ __forceinline__ T to_rz(float v);
-template <> __device__ __forceinline__ __half to_rz<__half>(float v) { return __float2half_rz(v); }
-template <> __device__ __forceinline__ __nv_bfloat16 to_rz<__nv_bfloat16>(float v) { return __float2bfloat16_rz(v); }
-
-template <typename T>
-__device__ __forceinline__ void pair_tile(const T* __restrict__ fin, T* __restrict__ fout, const Grid& g,
-                                          const Physics& ph, int x0, int y0, int y1, unsigned char* dsm,
-                                          PairRingT<T>& sR, uint32_t seed, int* flag) {
-    constexpr int TW = kWideTileW;
-    constexpr int W = BlockWin<T, TW>::value;
-    constexpr int kAlign = BlockWin<T, TW>::kAlign;
-    T* stage = reinterpret_cast<T*>(dsm);
-    uint64_t* bar = reinterpret_cast<uint64_t*>(dsm + (size_t)kBlockStages * 18 * W * sizeof(T));
+template <typename T, bool kWalls>
+__device__ __forceinline__ void pair_sweep(const Cell<T>* __restrict__ fin, Cell<T>* __restrict__ fout, const Grid& g,
+                                           const Physics& ph, int x0, int y0, int y1, unsigned char* dsm, PairRing& sR,
+                                           uint32_t seed, int* flag) {
+    typedef Cell<T> C;
+    constexpr int TW = kWideTileW, S = kPairStages;
+    constexpr int W = BlockWin<T, TW>::value, slack = BlockWin<T, TW>::kSlack;
+    static_assert(sizeof(C) == 4 && W % 2 == 0 && slack % 2 == 0, "column pairs are 8-byte aligned");
+    TileRows<T, TW, S, false> R(fin, g, x0, y0, y1, dsm, flag);
     const int t = threadIdx.x;
-    const int rfirst = max(y0 - 2, 0);
-    const int rlast = min(y1 + 1, g.ny - 1);
     const int xa = x0 + 2 * t;
     const bool own_a = xa < g.nx, own_b = xa + 1 < g.nx;
-    const bool dens_a = xa <= g.nx, dens_b = xa + 1 <= g.nx;   // column nx: ghost of column 0
-    const int e0 = g.origin + x0 - 2;
-    const int slack = e0 % kAlign;
+    const bool edge = xa < 2 || xa + 1 >= g.nx - 2;
     const int ka = 2 * t + 2 + slack;   // window column of xa
     // threads 64 / 65: the halo columns x0 - 1 / x0 + TW
     const bool halo = t == 64 || t == 65;
     const int kh = t == 64 ? 1 + slack : TW + 2 + slack;
-    const int sh = t == 64 ? 0 : TW + 1;
-    const T* win = fin + (e0 - slack);
-    const uint32_t row_bytes = W * sizeof(T);
-
-    if (t == 0) {
-        for (int j = 0; j < kBlockStages; ++j) mbar_init(&bar[j], 1);
-        mbar_fence_init();
-    }
-    __syncthreads();
-    int next = rfirst;
-    auto issue = [&](int r) {   // warp 0, all lanes
-        const int j = (r - rfirst) % kBlockStages;
-        uint64_t* b = &bar[j];
-        const uint32_t planes = tile_row_planes(r, y0, y1, g.ny);
-        if (t == 0) mbar_expect_tx(b, (uint32_t)__popc(planes) * row_bytes);
-        __syncwarp();
-        if (t < 18 && ((planes >> t) & 1u))
-            bulk_copy_g2s(stage + (size_t)j * 18 * W + t * W, win + (size_t)r * g.pitch + (size_t)t * g.plane,
-                          row_bytes, b);
-    };
-    if (t < 32)
-        for (; next <= rlast && next < rfirst + kBlockStages; ++next) issue(next);
-    auto wait_row = [&](int r) {
-        if (r >= rfirst && r <= rlast)
-            mbar_wait(&bar[(r - rfirst) % kBlockStages], (uint32_t)(((r - rfirst) / kBlockStages) & 1), flag);
-    };
-    auto stage_of = [&](int r) -> const T* {
-        const int rr = min(max(r, rfirst), rlast);
-        return stage + (size_t)((rr - rfirst) % kBlockStages) * 18 * W;
-    };
-    auto pull_row = [&](int yo, const T* sS, const T* sC, const T* sN, int kk, float f[2][9]) {
-        if (yo > 0 && yo < g.ny - 1)
-            pull_block<T, TW>(sS, sC, sN, false, false, kk, f);
-        else
-            pull_block<T, TW>(sS, sC, sN, yo == 0, yo == g.ny - 1, kk, f);
-    };
-    // densities of row yo into ring slot yo & 3 (16-bit storage holds h = f - w rho0),
-    // from the stages of rows yo - 1, yo, yo + 1
-    auto densities = [&](int yo, const T* sS, const T* sC, const T* sN) {
-        const int sl = yo & 3;
-        float f[2][9];
-        pull_row(yo, sS, sC, sN, ka, f);
-        sR[sl][0][2 * t + 1] = dens_a ? sum9(f[0]) + ph.shift[0] : 0.0f;
-        sR[sl][1][2 * t + 1] = dens_a ? sum9(f[1]) + ph.shift[1] : 0.0f;
-        pull_row(yo, sS, sC, sN, ka + 1, f);
-        sR[sl][0][2 * t + 2] = dens_b ? sum9(f[0]) + ph.shift[0] : 0.0f;
-        sR[sl][1][2 * t + 2] = dens_b ? sum9(f[1]) + ph.shift[1] : 0.0f;
-        if (halo) {
-            pull_row(yo, sS, sC, sN, kh, f);
-            sR[sl][0][sh] = sum9(f[0]) + ph.shift[0];
-            sR[sl][1][sh] = sum9(f[1]) + ph.shift[1];
-        }
-    };
-    auto zero_row = [&](int yo) {
-        const int sl = yo & 3;
-        sR[sl][0][2 * t + 1] = 0.0f; sR[sl][1][2 * t + 1] = 0.0f;
-        sR[sl][0][2 * t + 2] = 0.0f; sR[sl][1][2 * t + 2] = 0.0f;
-        if (halo) { sR[sl][0][sh] = 0.0f; sR[sl][1][sh] = 0.0f; }
-    };
-    // neighbour densities of the thread's first (b = 0) or second (b = 1) site on row y:
-    // ring columns 2t .. 2t + 3 of rows y - 1, y, y + 1 as two aligned float2 loads per
-    // row and component (consecutive lanes read consecutive 8-byte words)
-    auto neighbours = [&](int y, int b, Nbr& pA, Nbr& pB) {
-        const int s0 = (y - 1) & 3, s1 = y & 3, s2 = (y + 1) & 3;
+    const int sh = t == 64 ? 1 : TW + 2;
+    const float2 shift = shift_of(ph);
+    C* q = fout + (size_t)y0 * g.pitch + g.origin + xa;
+    uint32_t site = site_index(g, y0, xa);
+    const uint32_t site_row = site_index(g, 1, xa) - site_index(g, 0, xa);
+    bool good = true;
+    // sums of the stored values of rows y and y + 1
+    float2 da = splat(0.0f), db = splat(0.0f), na = splat(0.0f), nb = splat(0.0f);
+    // the pair's cells of row yo: directions without an x shift (and bounced-back ones)
+    // are one 64-bit load
+    auto pull_pair = [&](int yo, const C* st, C fa[9], C fb[9]) {
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            Nbr& p = c == 0 ? pA : pB;
-            const float2 L0 = *reinterpret_cast<const float2*>(&sR[s0][c][2 * t]);
-            const float2 R0 = *reinterpret_cast<const float2*>(&sR[s0][c][2 * t + 2]);
-            const float2 L1 = *reinterpret_cast<const float2*>(&sR[s1][c][2 * t]);
-            const float2 R1 = *reinterpret_cast<const float2*>(&sR[s1][c][2 * t + 2]);
-            const float2 L2 = *reinterpret_cast<const float2*>(&sR[s2][c][2 * t]);
-            const float2 R2 = *reinterpret_cast<const float2*>(&sR[s2][c][2 * t + 2]);
-            if (b == 0) {   // ring column 2t + 1
-                p.W = L1.x; p.E = R1.x;
-                p.SW = L0.x; p.S = L0.y; p.SE = R0.x;
-                p.NW = L2.x; p.N = L2.y; p.NE = R2.x;
-            } else {        // ring column 2t + 2
-                p.W = L1.y; p.E = R1.y;
-                p.SW = L0.y; p.S = R0.x; p.SE = R0.y;
-                p.NW = L2.y; p.N = R2.x; p.NE = R2.y;
+        for (int i = 0; i < 9; ++i) {
+            const C* p = st + i * W + ka;
+            if (cx(i) == 0 || (kWalls && ((cy(i) == 1 && yo == 0) || (cy(i) == -1 && yo == g.ny - 1)))) {
+                const uint2 v = *reinterpret_cast<const uint2*>(p);
+                fa[i] = cell_of_bits<C>(v.x);
+                fb[i] = cell_of_bits<C>(v.y);
+            } else {
+                fa[i] = p[-cx(i)];
+                fb[i] = p[1 - cx(i)];
             }
         }
     };
-    // collide the thread's site b (window column ka + b, column xa + b) of row y; out:
-    // its values with the stochastic rounding's bits added, to be rounded toward zero
-    auto site = [&](int y, const T* sS, const T* sC, const T* sN, int b, float out[2][9]) {
-        float h[2][9];
-        pull_row(y, sS, sC, sN, ka + b, h);
-        Nbr pA, pB;
-        neighbours(y, b, pA, pB);
-        collide_shifted(h, pA, pB, ph, y, g.ny, flag);
-        dither_site<T>(g, y, xa + b, h, seed, out);
-    };
-    auto ghost = [&](int y, int x, const float v[2][9]) {   // periodic copies of the two first / last columns
-        if (x < 2 || x >= g.nx - 2) {
-            T* qg = fout + (size_t)y * g.pitch + g.origin + x + (x < 2 ? g.nx : -g.nx);
-#pragma unroll
-            for (int s = 0; s < 2; ++s)
-#pragma unroll
-                for (int i = 0; i < 9; ++i) qg[(size_t)(s * 9 + i) * g.plane] = to_rz<T>(v[s][i]);
+    auto densities = [&](int yo, const C* st) {
+        float2* ring = sR[yo & 3];
+        da = na;
+        db = nb;
+        if (kWalls && (yo < 0 || yo >= g.ny)) {   // a virtual wall row
+            *reinterpret_cast<float4*>(&ring[2 * t + 2]) = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (halo) ring[sh] = splat(0.0f);
+            return;
+        }
+        C fa[9], fb[9];
+        pull_pair(yo, st, fa, fb);
+        na = sum_cells(fa);
+        nb = sum_cells(fb);
+        const float2 ra = density_of<T>(na, shift), rb = density_of<T>(nb, shift);
+        *reinterpret_cast<float4*>(&ring[2 * t + 2]) = make_float4(ra.y, ra.x, rb.y, rb.x);
+        if (halo) {
+            pull_stage<W>(st, kWalls && yo == 0, kWalls && yo == g.ny - 1, kh, fa);
+            ring[sh] = swap2(density_of<T>(sum_cells(fa), shift));
         }
     };
-
-    if (y0 > 0) {
-        wait_row(y0 - 2); wait_row(y0 - 1); wait_row(y0);
-        densities(y0 - 1, stage_of(y0 - 2), stage_of(y0 - 1), stage_of(y0));
-    } else {
-        zero_row(y0 - 1);
-    }
-    wait_row(y0 - 1); wait_row(y0); wait_row(y0 + 1);
-    densities(y0, stage_of(y0 - 1), stage_of(y0), stage_of(y0 + 1));
-    __syncthreads();
-    if (t < 32) {
-        fence_proxy_async_smem();
-        for (; next <= rlast && next - kBlockStages <= y0 - 2; ++next) issue(next);
-    }
-    // stage of row y (advanced by one per row, no division): rows y - 1 .. y + 2 sit in
-    // the stages beside it.  A row outside [rfirst, rlast] maps to some stage, but its
-    // pull is never read (bounce-back on the wall rows takes the centre row instead).
-    constexpr int S = kBlockStages;
-    constexpr size_t kStageElems = (size_t)18 * W;
-    int jy = y0 - rfirst;
-    uint32_t pq = (uint32_t)(((y0 + 2 - rfirst) / S) & 1);   // phase of the wait for row y + 2
-    for (int y = y0; y < y1; ++y) {
-        const int jm = jy == 0 ? S - 1 : jy - 1;
-        const int jp = jy == S - 1 ? 0 : jy + 1;
-        const int jq = jp == S - 1 ? 0 : jp + 1;
-        const T* sS = stage + jm * kStageElems;
-        const T* sC = stage + jy * kStageElems;
-        const T* sN = stage + jp * kStageElems;
-        if (y + 1 < g.ny) {
-            if (y + 2 <= rlast) mbar_wait(&bar[jq], pq, flag);
-            densities(y + 1, sC, sN, stage + jq * kStageElems);
-        } else {
-            zero_row(y + 1);
-        }
-        __syncthreads();
-        // every thread is past its reads of rows < y - 1 (the sites below pull row
-        // y - 1 again after the barrier): refill those stages
-        if (t < 32) {
-            fence_proxy_async_smem();
-            for (; next <= rlast && next - kBlockStages <= y - 2; ++next) issue(next);
-        }
+    auto collide = [&](int y, const C* st) {
         if (own_a) {
-            float va[2][9], vb[2][9];
-            site(y, sS, sC, sN, 0, va);
-            T* q = fout + (size_t)y * g.pitch + g.origin + xa;
+            C fa[9], fb[9];
+            pull_pair(y, st, fa, fb);
+            // columns xa - 1, xa, xa + 1 and xa + 2 of rows y - 1, y, y + 1
+            const float2 *S0 = &sR[(y - 1) & 3][2 * t + 2], *S1 = &sR[y & 3][2 * t + 2], *S2 = &sR[(y + 1) & 3][2 * t + 2];
+            const float4 ab0 = *reinterpret_cast<const float4*>(S0), ab1 = *reinterpret_cast<const float4*>(S1),
+                         ab2 = *reinterpret_cast<const float4*>(S2);
+            const float2 a0 = make_float2(ab0.x, ab0.y), b0 = make_float2(ab0.z, ab0.w);
+            const float2 a1 = make_float2(ab1.x, ab1.y), b1 = make_float2(ab1.z, ab1.w);
+            const float2 a2 = make_float2(ab2.x, ab2.y), b2 = make_float2(ab2.z, ab2.w);
+            Nbr2 p;
+            p.W = S1[-1]; p.E = b1;
+            p.S = a0; p.SW = S0[-1]; p.SE = b0;
+            p.N = a2; p.NW = S2[-1]; p.NE = b2;
+            good &= collide_cells<T, kWalls>(fa, da, p, g.ny, ph, y, site, seed, fa);
             if (own_b) {
-                site(y, sS, sC, sN, 1, vb);
-                // one conversion and one 32-bit store per plane for the column pair
+                p.W = a1; p.E = S1[2];
+                p.S = b0; p.SW = a0; p.SE = S0[2];
+                p.N = b2; p.NW = a2; p.NE = S2[2];
+                good &= collide_cells<T, kWalls>(fb, db, p, g.ny, ph, y, site + 1, seed, fb);
 #pragma unroll
-                for (int s = 0; s < 2; ++s)
-#pragma unroll
-                    for (int i = 0; i < 9; ++i)
-                        *reinterpret_cast<uint32_t*>(q + (size_t)(s * 9 + i) * g.plane) = pack_rz<T>(va[s][i], vb[s][i]);
-                ghost(y, xa + 1, vb);
+                for (int i = 0; i < 9; ++i)
+                    *reinterpret_cast<uint2*>(q + (size_t)i * g.plane) = make_uint2(bits_of_cell(fa[i]), bits_of_cell(fb[i]));
             } else {
 #pragma unroll
-                for (int s = 0; s < 2; ++s)
-#pragma unroll
-                    for (int i = 0; i < 9; ++i) q[(size_t)(s * 9 + i) * g.plane] = to_rz<T>(va[s][i]);
+                for (int i = 0; i < 9; ++i) q[(size_t)i * g.plane] = fa[i];
             }
-            ghost(y, xa, va);
+            if (edge) {   // periodic ghost copies of the two first / last columns
+#pragma unroll
+                for (int b = 0; b < 2; ++b) {
+                    const int x = xa + b;
+                    if (x < g.nx && (x < 2 || x >= g.nx - 2)) {
+                        C* qg = q + b + (x < 2 ? g.nx : -g.nx);
+#pragma unroll
+                        for (int i = 0; i < 9; ++i) qg[(size_t)i * g.plane] = b == 0 ? fa[i] : fb[i];
+                    }
+                }
+            }
         }
-        pq ^= (uint32_t)(jy == S - 3);   // row y + 3 sits in stage jy + 3: a new fill once it wraps to 0
-        jy = jp;
-    }
+        q += g.pitch;
+        site += site_row;
+    };
+    sweep_tile(R, densities, collide);
+    if (!good) atomicOr(flag, 1);
+}
+template <typename T>
+__device__ __forceinline__ void pair_tile(const Cell<T>* __restrict__ fin, Cell<T>* __restrict__ fout, const Grid& g,
+                                          const Physics& ph, int x0, int y0, int y1, unsigned char* dsm, PairRing& sR,
+                                          uint32_t seed, int* flag) {
+    if (tile_has_walls(y0, y1, g.ny)) pair_sweep<T, true>(fin, fout, g, ph, x0, y0, y1, dsm, sR, seed, flag);
+    else pair_sweep<T, false>(fin, fout, g, ph, x0, y0, y1, dsm, sR, seed, flag);
 }
 
 template <typename T>
 __global__ void __launch_bounds__(kPairThreads, 4)
-step_pair_kernel(const T* __restrict__ fin, T* __restrict__ fout, Grid g, Physics ph, int* flag) {
+step_pair_kernel(const Cell<T>* __restrict__ fin, Cell<T>* __restrict__ fout, Grid g, Physics ph, int* flag) {
     extern __shared__ __align__(128) unsigned char dsm[];
-    __shared__ __align__(16) PairRingT<T> sR;
+    __shared__ __align__(16) PairRing sR;
     const int y0 = (int)(((long long)blockIdx.y * g.ny) / gridDim.y);
     const int y1 = (int)(((long long)(blockIdx.y + 1) * g.ny) / gridDim.y);
     const uint32_t seed = launch_seed(ph);
@@ -1241,8 +1085,8 @@ step_pair_kernel(const T* __restrict__ fin, T* __restrict__ fout, Grid g, Physic
 // One grid: block (bx, by) of TW threads takes columns [TW bx, TW bx + TW) and the
 // by-th of gridDim.y tiles of (nearly) equal height.
 template <typename T, int TW>
-__global__ void __launch_bounds__(TW, 512 / TW)
-step_block_kernel(const T* __restrict__ fin, T* __restrict__ fout, Grid g, Physics ph, int* flag) {
+__global__ void __launch_bounds__(TW, TileCfg<T, TW>::kBlocks)
+step_block_kernel(const Cell<T>* __restrict__ fin, Cell<T>* __restrict__ fout, Grid g, Physics ph, int* flag) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ BlockRingT<TW> sR;
     const int y0 = (int)(((long long)blockIdx.y * g.ny) / gridDim.y);
@@ -1256,7 +1100,7 @@ step_block_kernel(const T* __restrict__ fin, T* __restrict__ fout, Grid g, Physi
 // (block_tile's kWithhold), so that every bounded wait gives up and raises bit 2 of the
 // guard.  Its output is garbage; the step counters are left alone.
 __global__ void __launch_bounds__(kBlockTileW, 512 / kBlockTileW)
-step_block_timeout_kernel(const float* __restrict__ fin, float* __restrict__ fout, Grid g, Physics ph, int* flag) {
+step_block_timeout_kernel(const float2* __restrict__ fin, float2* __restrict__ fout, Grid g, Physics ph, int* flag) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ BlockRingT<kBlockTileW> sR;
     const int y0 = (int)(((long long)blockIdx.y * g.ny) / gridDim.y);
@@ -1271,15 +1115,11 @@ step_block_timeout_kernel(const float* __restrict__ fin, float* __restrict__ fou
 // the member's grid, physics and storage type; no member waits for another, so
 // uneven grids need no barrier.
 // ---------------------------------------------------------------------------
-template <int TW, bool kPaired>
-__global__ void __launch_bounds__(TW, 512 / TW)
+template <int TW>
+__global__ void __launch_bounds__(TW, 768 / TW)
 ensemble_step_kernel(const EnsMember* __restrict__ members, int n, int parity) {
     extern __shared__ __align__(128) unsigned char dsm[];
-    // density ring: the block tile's, or with kPaired also the paired tile's (16-bit members)
-    constexpr size_t kRing = kPaired && sizeof(PairRingT<__half>) > sizeof(BlockRingT<TW>) ? sizeof(PairRingT<__half>)
-                                                                                         : sizeof(BlockRingT<TW>);
-    __shared__ __align__(16) unsigned char ring[kRing];
-    BlockRingT<TW>& sR = *reinterpret_cast<BlockRingT<TW>*>(ring);
+    __shared__ BlockRingT<TW> sR;
     const int tile = blockIdx.x;
     int lo = 0, hi = n - 1;   // last member whose first tile is <= tile
     while (lo < hi) {
@@ -1301,48 +1141,38 @@ ensemble_step_kernel(const EnsMember* __restrict__ members, int n, int parity) {
     advance_step(ph, local == 0 && threadIdx.x == 0);
     switch (M.storage) {
         case LBM_STORE_F16:
-            if constexpr (kPaired)
-                pair_tile<__half>((const __half*)fin, (__half*)fout, M.grid, ph, tx * kWideTileW, y0, y1, dsm,
-                                  *reinterpret_cast<PairRingT<__half>*>(ring), seed, M.flag);
-            else
-                block_tile<__half, TW>((const __half*)fin, (__half*)fout, M.grid, ph, tx * TW, y0, y1, dsm, sR, seed,
-                                       M.flag);
+            block_tile<__half, TW>((const __half2*)fin, (__half2*)fout, M.grid, ph, tx * TW, y0, y1, dsm, sR, seed,
+                                   M.flag);
             break;
         case LBM_STORE_BF16:
-            if constexpr (kPaired)
-                pair_tile<__nv_bfloat16>((const __nv_bfloat16*)fin, (__nv_bfloat16*)fout, M.grid, ph, tx * kWideTileW,
-                                         y0, y1, dsm, *reinterpret_cast<PairRingT<__nv_bfloat16>*>(ring), seed, M.flag);
-            else
-                block_tile<__nv_bfloat16, TW>((const __nv_bfloat16*)fin, (__nv_bfloat16*)fout, M.grid, ph, tx * TW, y0,
-                                              y1, dsm, sR, seed, M.flag);
+            block_tile<__nv_bfloat16, TW>((const __nv_bfloat162*)fin, (__nv_bfloat162*)fout, M.grid, ph, tx * TW, y0, y1,
+                                          dsm, sR, seed, M.flag);
             break;
         default:
-            block_tile<float, TW>((const float*)fin, (float*)fout, M.grid, ph, tx * TW, y0, y1, dsm, sR, seed,
-                                  M.flag);
+            block_tile<float, TW>((const float2*)fin, (float2*)fout, M.grid, ph, tx * TW, y0, y1, dsm, sR, seed, M.flag);
     }
 }
 
+// kEnsNarrow (0) and 128: 128-column tiles
+static bool ens_wide(int tile_x) { return tile_x == kWideTileW; }
+
 int ensemble_tile_cols(int storage, int tile_x) {
-    if (tile_x == kEnsPaired) return storage == LBM_STORE_F32 ? kBlockTileW : kWideTileW;
-    return tile_x;
+    (void)storage;
+    return ens_wide(tile_x) ? kWideTileW : kBlockTileW;
 }
 
 size_t block_tile_smem_bytes(int storage, int tile_x) {
-    if (tile_x == kEnsPaired)
-        return storage == LBM_STORE_F32 ? block_smem_bytes<float>() : pair_smem_bytes<__half>();
-    if (tile_x == kWideTileW)
+    if (ens_wide(tile_x))
         return storage == LBM_STORE_F32 ? block_smem_bytes<float, kWideTileW>() : block_smem_bytes<__half, kWideTileW>();
     return storage == LBM_STORE_F32 ? block_smem_bytes<float>() : block_smem_bytes<__half>();
 }
 
-template <int TW, bool kPaired>
+template <int TW>
 static cudaError_t ensemble_attr() {
     static bool attr_set = false;
     if (!attr_set) {
-        const size_t smem = kPaired ? std::max(block_smem_bytes<float, TW>(), pair_smem_bytes<__half>())
-                                    : block_smem_bytes<float, TW>();
-        cudaError_t e = cudaFuncSetAttribute(ensemble_step_kernel<TW, kPaired>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = cudaFuncSetAttribute(ensemble_step_kernel<TW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)block_smem_bytes<float, TW>());
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
@@ -1352,22 +1182,14 @@ static cudaError_t ensemble_attr() {
 // Resident blocks of the ensemble kernel of tile width tile_x for `smem` bytes.
 int ensemble_slots(size_t smem, int tile_x, cudaError_t* err) {
     int dev = 0, sms = 0, occ = 0;
-    cudaError_t e = tile_x == kWideTileW ? ensemble_attr<kWideTileW, false>()
-                    : tile_x == kEnsPaired ? ensemble_attr<kBlockTileW, true>()
-                                           : ensemble_attr<kBlockTileW, false>();
+    const bool wide = ens_wide(tile_x);
+    cudaError_t e = wide ? ensemble_attr<kWideTileW>() : ensemble_attr<kBlockTileW>();
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) {
-        if (tile_x == kWideTileW)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, ensemble_step_kernel<kWideTileW, false>, kWideTileW,
-                                                              smem);
-        else if (tile_x == kEnsPaired)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, ensemble_step_kernel<kBlockTileW, true>, kBlockTileW,
-                                                              smem);
-        else
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, ensemble_step_kernel<kBlockTileW, false>,
-                                                              kBlockTileW, smem);
-    }
+    if (e == cudaSuccess)
+        e = wide ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, ensemble_step_kernel<kWideTileW>, kWideTileW, smem)
+                 : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, ensemble_step_kernel<kBlockTileW>, kBlockTileW,
+                                                                 smem);
     if (err) *err = e;
     return std::max(1, sms * occ);
 }
@@ -1375,41 +1197,36 @@ int ensemble_slots(size_t smem, int tile_x, cudaError_t* err) {
 cudaError_t launch_ensemble_step(const EnsMember* d_members, int n, int total_tiles, int parity, size_t smem,
                                  int tile_x, cudaStream_t st) {
     (void)cudaGetLastError();
-    cudaError_t e = cudaSuccess;
-    if (tile_x == kWideTileW) {
-        if ((e = ensemble_attr<kWideTileW, false>()) != cudaSuccess) return e;
-        ensemble_step_kernel<kWideTileW, false><<<total_tiles, kWideTileW, smem, st>>>(d_members, n, parity);
-    } else if (tile_x == kEnsPaired) {
-        if ((e = ensemble_attr<kBlockTileW, true>()) != cudaSuccess) return e;
-        ensemble_step_kernel<kBlockTileW, true><<<total_tiles, kBlockTileW, smem, st>>>(d_members, n, parity);
-    } else {
-        if ((e = ensemble_attr<kBlockTileW, false>()) != cudaSuccess) return e;
-        ensemble_step_kernel<kBlockTileW, false><<<total_tiles, kBlockTileW, smem, st>>>(d_members, n, parity);
-    }
+    cudaError_t e = ens_wide(tile_x) ? ensemble_attr<kWideTileW>() : ensemble_attr<kBlockTileW>();
+    if (e != cudaSuccess) return e;
+    if (ens_wide(tile_x))
+        ensemble_step_kernel<kWideTileW><<<total_tiles, kWideTileW, smem, st>>>(d_members, n, parity);
+    else
+        ensemble_step_kernel<kBlockTileW><<<total_tiles, kBlockTileW, smem, st>>>(d_members, n, parity);
     return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
-// Two-pass step: densities into psi, then pull + collide reading psi neighbours.
+// Two-pass step: densities, as (B, A), into psi, then pull + collide reading psi
+// neighbours.
 // ---------------------------------------------------------------------------
 template <typename T>
 __global__ void __launch_bounds__(kThreadsX)
-density_kernel(const T* __restrict__ fin, float* __restrict__ psi, Grid g, Physics ph) {
+density_kernel(const Cell<T>* __restrict__ fin, float2* __restrict__ psi, Grid g, Physics ph) {
     const int x = blockIdx.x * kThreadsX + threadIdx.x;
     const int y = blockIdx.y;
     if (x >= g.nx) return;
     const int xm = x == 0 ? g.nx - 1 : x - 1;
     const int xp = x == g.nx - 1 ? 0 : x + 1;
-    float f[2][9];
-    pull_site<T>(fin, g, ph.shift, y, x, xm, xp, f);
-    psi[(size_t)y * g.pitch + x] = sum9(f[0]);
-    psi[g.plane + (size_t)y * g.pitch + x] = sum9(f[1]);
+    float2 f[9];
+    pull_site<T>(fin, g, shift_of(ph), y, x, xm, xp, f);
+    psi[(size_t)y * g.pitch + x] = swap2(sum9_2(f));
 }
 
 template <typename T>
 __global__ void __launch_bounds__(kThreadsX)
-collide_kernel(const T* __restrict__ fin, const float* __restrict__ psi, T* __restrict__ fout,
-               Grid g, Physics ph, int* flag) {
+collide_kernel(const Cell<T>* __restrict__ fin, const float2* __restrict__ psi, Cell<T>* __restrict__ fout, Grid g,
+               Physics ph, int* flag) {
     const int x = blockIdx.x * kThreadsX + threadIdx.x;
     const int y = blockIdx.y;
     const uint32_t seed = launch_seed(ph);
@@ -1417,30 +1234,23 @@ collide_kernel(const T* __restrict__ fin, const float* __restrict__ psi, T* __re
     if (x >= g.nx) return;
     const int xm = x == 0 ? g.nx - 1 : x - 1;
     const int xp = x == g.nx - 1 ? 0 : x + 1;
-    float f[2][9];
-    pull_site<T>(fin, g, ph.shift, y, x, xm, xp, f);
-    Nbr p[2];
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-        const float* q = psi + (size_t)s * g.plane;
-        const float* r0 = q + (size_t)y * g.pitch;
-        p[s].E = __ldg(r0 + xp);
-        p[s].W = __ldg(r0 + xm);
-        if (y + 1 < g.ny) {
-            const float* r = q + (size_t)(y + 1) * g.pitch;
-            p[s].N = __ldg(r + x); p[s].NE = __ldg(r + xp); p[s].NW = __ldg(r + xm);
-        } else {
-            p[s].N = p[s].NE = p[s].NW = 0.0f;
-        }
-        if (y > 0) {
-            const float* r = q + (size_t)(y - 1) * g.pitch;
-            p[s].S = __ldg(r + x); p[s].SE = __ldg(r + xp); p[s].SW = __ldg(r + xm);
-        } else {
-            p[s].S = p[s].SE = p[s].SW = 0.0f;
-        }
+    float2 f[9];
+    pull_site<T>(fin, g, shift_of(ph), y, x, xm, xp, f);
+    const float2* r = psi + (size_t)y * g.pitch;
+    Nbr2 p;
+    p.E = __ldg(r + xp);
+    p.W = __ldg(r + xm);
+    p.N = p.NE = p.NW = p.S = p.SE = p.SW = splat(0.0f);
+    if (y + 1 < g.ny) {
+        const float2* q = r + g.pitch;
+        p.N = __ldg(q + x); p.NE = __ldg(q + xp); p.NW = __ldg(q + xm);
     }
-    collide_site<IsShifted<T>::value == false>(f, p[0], p[1], ph, y, g.ny, flag);
-    store_step<T>(fout, g, y, x, f, ph.shift, seed);
+    if (y > 0) {
+        const float2* q = r - g.pitch;
+        p.S = __ldg(q + x); p.SE = __ldg(q + xp); p.SW = __ldg(q + xm);
+    }
+    if (!collide_site<Exact<T>::value, true>(f, sum9_2(f), p, ph, y, g.ny)) atomicOr(flag, 1);
+    store_step<T>(fout, g, y, x, f, shift_of(ph), seed);
 }
 
 // ---------------------------------------------------------------------------
@@ -1458,61 +1268,79 @@ __device__ __forceinline__ void init_rho(const double* y0, int x, int y, double 
 // y0 holds the interface heights of columns -1 .. nx (y0[x + 1]): the population a
 // site sends towards x + c_i is that of the site it reaches, beside the grid too.
 template <typename T>
-__global__ void init_kernel(T* __restrict__ fout, Grid g, float sA, float sB, const double* __restrict__ y0,
+__global__ void init_kernel(Cell<T>* __restrict__ fout, Grid g, float sA, float sB, const double* __restrict__ y0,
                             double mA, double mB, double eps, double width) {
     const int x = blockIdx.x * kThreadsX + threadIdx.x;
     const int y = blockIdx.y;
     if (x >= g.nx) return;
-    const float shift[2] = {sA, sB};
+    const float2 shift = make_float2(sA, sB);
     double here[2];
     y0 += 1;
     init_rho(y0, x, y, mA, mB, eps, width, here[0], here[1]);
-    float f[2][9];
+    float2 f[9];
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
         const int ty = y + cy(i);
         const int tx = x + cx(i);
         double r[2] = {here[0], here[1]};
         if (ty >= 0 && ty < g.ny) init_rho(y0, tx, ty, mA, mB, eps, width, r[0], r[1]);
-        for (int s = 0; s < 2; ++s) f[s][i] = (float)(wd(i) * r[s]);
+        f[i] = make_float2((float)(wd(i) * r[0]), (float)(wd(i) * r[1]));
     }
     store_site<T>(fout, g, y, x, f, shift);
 }
 
 template <typename T, typename V>
-__global__ void pull_to_host_kernel(const T* __restrict__ fin, Grid g, float sA, float sB, V* __restrict__ S) {
+__global__ void pull_to_host_kernel(const Cell<T>* __restrict__ fin, Grid g, float sA, float sB, V* __restrict__ S) {
     const int x = blockIdx.x * kThreadsX + threadIdx.x;
     const int y = blockIdx.y;
     if (x >= g.nx) return;
-    const float shift[2] = {sA, sB};
     // the columns beside the grid from the ghost columns (periodic copies, or a split
     // grid's neighbours)
-    float f[2][9];
-    pull_site<T>(fin, g, shift, y, x, x - 1, x + 1, f);
-    const size_t n = (size_t)g.nx * g.ny;
-    for (int s = 0; s < 2; ++s)
-        for (int i = 0; i < 9; ++i) S[(size_t)(s * 9 + i) * n + (size_t)y * g.nx + x] = (V)f[s][i];
+    float2 f[9];
+    pull_site<T>(fin, g, make_float2(sA, sB), y, x, x - 1, x + 1, f);
+    const size_t n = (size_t)g.nx * g.ny, k = (size_t)y * g.nx + x;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        S[(size_t)i * n + k] = (V)f[i].x;
+        S[(size_t)(9 + i) * n + k] = (V)f[i].y;
+    }
 }
 
 template <typename T, typename V>
-__global__ void push_from_host_kernel(const V* __restrict__ S, Grid g, float sA, float sB, T* __restrict__ fout) {
+__global__ void push_from_host_kernel(const V* __restrict__ S, Grid g, float sA, float sB, Cell<T>* __restrict__ fout) {
     const int x = blockIdx.x * kThreadsX + threadIdx.x;
     const int y = blockIdx.y;
     if (x >= g.nx) return;
-    const float shift[2] = {sA, sB};
     const size_t n = (size_t)g.nx * g.ny;
-    float f[2][9];
-    for (int s = 0; s < 2; ++s) {
-        for (int i = 0; i < 9; ++i) {
-            const int ty = y + cy(i);
-            const int tx = (x + cx(i) + g.nx) % g.nx;
-            const V v = (ty >= 0 && ty < g.ny)
-                ? S[(size_t)(s * 9 + i) * n + (size_t)ty * g.nx + tx]
-                : S[(size_t)(s * 9 + opp(i)) * n + (size_t)y * g.nx + x];
-            f[s][i] = (float)v;
-        }
+    const int xm = x == 0 ? g.nx - 1 : x - 1;
+    const int xp = x == g.nx - 1 ? 0 : x + 1;
+    float2 f[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        const int ty = y + cy(i);
+        const int tx = cx(i) == 0 ? x : (cx(i) == 1 ? xp : xm);
+        const size_t k = (ty >= 0 && ty < g.ny) ? (size_t)i * n + (size_t)ty * g.nx + tx
+                                                : (size_t)opp(i) * n + (size_t)y * g.nx + x;
+        f[i] = make_float2((float)S[k], (float)S[9 * n + k]);
     }
-    store_site<T>(fout, g, y, x, f, shift);
+    store_site<T>(fout, g, y, x, f, make_float2(sA, sB));
+}
+
+// State files hold [component][direction][ny][pitch] planes with the ghost columns;
+// column 0 sits `origin` values into a row.  V: the bits of a stored value.
+template <typename V, bool kToPlanes>
+__global__ void planes_kernel(V* __restrict__ cells, Grid g, V* __restrict__ planes, int pitch, int origin) {
+    const int x = blockIdx.x * kThreadsX + threadIdx.x - 2;
+    const int y = blockIdx.y;
+    if (x >= g.nx + 2) return;
+#pragma unroll
+    for (int p = 0; p < 18; ++p) {
+        const int s = p / 9, i = p % 9;
+        V* c = cells + 2 * ((size_t)i * g.plane + (size_t)y * g.pitch + g.origin + x) + s;
+        V* q = planes + ((size_t)p * g.ny + y) * pitch + origin + x;
+        if (kToPlanes) *q = *c;
+        else *c = *q;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1559,7 +1387,7 @@ static cudaError_t launch_block(const StepLaunch& L, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     const int gx = (g.nx + TW - 1) / TW;
     dim3 grid(gx, block_tiles_y(g.ny, gx, L.tile_y, slots, kMinTileRows));
-    step_block_kernel<T, TW><<<grid, TW, block_smem_bytes<T, TW>(), st>>>((const T*)L.fin, (T*)L.fout, g, L.phys,
+    step_block_kernel<T, TW><<<grid, TW, block_smem_bytes<T, TW>(), st>>>((const Cell<T>*)L.fin, (Cell<T>*)L.fout, g, L.phys,
                                                                            L.flag);
     return cudaGetLastError();
 }
@@ -1592,10 +1420,11 @@ static cudaError_t launch_dec(const StepLaunch& L, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     const int gx = (g.nx + TW - 1) / TW;
     dim3 grid(gx, block_tiles_y(g.ny, gx, L.tile_y, slots, kMinTileRows));
-    step_dec_kernel<T, TW><<<grid, TW, dec_smem_bytes<T, TW>(), st>>>((const T*)L.fin, (T*)L.fout, g, L.phys, L.flag);
+    step_dec_kernel<T, TW><<<grid, TW, dec_smem_bytes<T, TW>(), st>>>((const Cell<T>*)L.fin, (Cell<T>*)L.fout, g, L.phys, L.flag);
     return cudaGetLastError();
 }
 
+// Paired tiles go down to 8 rows so that the wave is full.
 template <typename T>
 static cudaError_t launch_pair(const StepLaunch& L, cudaStream_t st) {
     static int slots = 0;
@@ -1613,21 +1442,18 @@ static cudaError_t launch_pair(const StepLaunch& L, cudaStream_t st) {
     }
     const Grid& g = L.grid;
     const int gx = (g.nx + kWideTileW - 1) / kWideTileW;
-    // tiles down to 8 rows so that the wave is full: at 1024x2048 152 x 4 tiles of
-    // 13-14 rows run 11 % faster than 128 x 4 of 16 (measured with tile_y 14)
     dim3 grid(gx, block_tiles_y(g.ny, gx, L.tile_y, slots, 8));
-    step_pair_kernel<T><<<grid, kPairThreads, pair_smem_bytes<T>(), st>>>((const T*)L.fin, (T*)L.fout, g, L.phys,
-                                                                           L.flag);
+    step_pair_kernel<T><<<grid, kPairThreads, pair_smem_bytes<T>(), st>>>((const Cell<T>*)L.fin, (Cell<T>*)L.fout, g,
+                                                                           L.phys, L.flag);
     return cudaGetLastError();
 }
 
-// Columns per block tile of the block-staged kernel: tile_x when it is 128 or 256;
-// otherwise 256 for 16-bit storage, and for FP32 when the 256-column tiles hold at
-// least kWideMinRows rows (tile_y, or the rows of the one-wave default).  Measured
-// on GB300: the wider tile reads 6 % less halo and wins wherever the tiles are tall
-// (FP32 at 10000x5000: 0.858 of the HBM peak against 0.832) and with 16-bit storage
-// at every size tried (+1.6 to +4.6 %); FP32 tiles of 27 rows (1024x2048) are 0.6 %
-// slower, the barrier of 8 warps costing more per row than the halo saves.
+// Columns per one-column-per-thread tile: tile_x when it is 128 or 256; otherwise 256
+// for 16-bit storage, and for FP32 when the 256-column tiles hold at least kWideMinRows
+// rows (tile_y, or the rows of the one-wave default).  The wider tile reads half the halo
+// columns and wins where tiles are tall (FP32 at 10000x5000: 1101 us a step against 1119);
+// tiles of 27 rows (1024x2048) run 51.4 us at 128 columns and 53.3 at 256, the barrier of 8
+// warps costing more per row than the halo saves.
 template <typename T>
 static cudaError_t block_tile_width(const Grid& g, int tile_x, int tile_y, int* tw) {
     constexpr int kWideMinRows = 64;
@@ -1655,20 +1481,18 @@ static cudaError_t launch_step_t(const StepLaunch& L, int kernel, cudaStream_t s
     const int bx = (g.nx + kThreadsX - 1) / kThreadsX;
     if (kernel == LBM_KERNEL_TWO_PASS) {
         dim3 grid(bx, g.ny);
-        density_kernel<T><<<grid, kThreadsX, 0, st>>>((const T*)L.fin, L.psi, g, L.phys);
-        collide_kernel<T><<<grid, kThreadsX, 0, st>>>((const T*)L.fin, L.psi, (T*)L.fout, g, L.phys, L.flag);
-    } else if (kernel == LBM_KERNEL_STAGED) {
-        // 16-bit storage at the default width: the paired-column tile (same results bit
-        // for bit; equal at 1024x2048, 1.23x the 256-thread tile at 10000x5000)
+        density_kernel<T><<<grid, kThreadsX, 0, st>>>((const Cell<T>*)L.fin, (float2*)L.psi, g, L.phys);
+        collide_kernel<T><<<grid, kThreadsX, 0, st>>>((const Cell<T>*)L.fin, (float2*)L.psi, (Cell<T>*)L.fout, g, L.phys, L.flag);
+    } else if (kernel == LBM_KERNEL_STAGED || kernel == LBM_KERNEL_PAIRED) {
+        // 16-bit storage at the default width: the paired-column tile (same results bit for
+        // bit; FP16 at 1024x2048 36.2 us a step against 38.1 of the 256-thread tile, at
+        // 10000x5000 783 against 859, at 1501x999 27.1 against 35.7)
         if constexpr (IsShifted<T>::value)
-            if (L.tile_x == 0) return launch_pair<T>(L, st);
+            if (kernel == LBM_KERNEL_PAIRED || L.tile_x == 0) return launch_pair<T>(L, st);
         int tw = 0;
         cudaError_t e = block_tile_width<T>(g, L.tile_x, L.tile_y, &tw);
         if (e != cudaSuccess) return e;
         return tw == kWideTileW ? launch_block<T, kWideTileW>(L, st) : launch_block<T, kBlockTileW>(L, st);
-    } else if (kernel == LBM_KERNEL_PAIRED) {
-        if constexpr (IsShifted<T>::value) return launch_pair<T>(L, st);
-        else return cudaErrorInvalidValue;
     } else if (kernel == LBM_KERNEL_DECOUPLED) {
         int tw = 0;
         cudaError_t e = block_tile_width<T>(g, L.tile_x, L.tile_y, &tw);
@@ -1685,7 +1509,7 @@ static cudaError_t launch_step_t(const StepLaunch& L, int kernel, cudaStream_t s
             attr_set = true;
         }
         dim3 grid((g.nx + kPipeOwned - 1) / kPipeOwned, (g.ny + ty - 1) / ty);
-        step_pipe_kernel<T><<<grid, kThreadsX, smem, st>>>((const T*)L.fin, (T*)L.fout, g, L.phys, ty, L.flag);
+        step_pipe_kernel<T><<<grid, kThreadsX, smem, st>>>((const Cell<T>*)L.fin, (Cell<T>*)L.fout, g, L.phys, ty, L.flag);
     } else if (kernel == LBM_KERNEL_WARP) {
         const int ty = L.tile_y > 0 ? L.tile_y : default_tile_y();
         const size_t smem = warp_kernel_smem_bytes<T>();
@@ -1699,12 +1523,12 @@ static cudaError_t launch_step_t(const StepLaunch& L, int kernel, cudaStream_t s
         const int tiles_x = (g.nx + kWarpOwned - 1) / kWarpOwned;
         const int tiles = tiles_x * ((g.ny + ty - 1) / ty);
         const int blocks = (tiles + kWarpsPerBlock - 1) / kWarpsPerBlock;
-        step_warp_kernel<T><<<blocks, kThreadsX, smem, st>>>((const T*)L.fin, (T*)L.fout, g, L.phys, ty, tiles_x,
+        step_warp_kernel<T><<<blocks, kThreadsX, smem, st>>>((const Cell<T>*)L.fin, (Cell<T>*)L.fout, g, L.phys, ty, tiles_x,
                                                                tiles, L.flag);
     } else {
         const int ty = L.tile_y > 0 ? L.tile_y : 16;
         dim3 grid(bx, (g.ny + ty - 1) / ty);
-        step_fused_kernel<T><<<grid, kThreadsX, 0, st>>>((const T*)L.fin, (T*)L.fout, g, L.phys, ty, L.flag);
+        step_fused_kernel<T><<<grid, kThreadsX, 0, st>>>((const Cell<T>*)L.fin, (Cell<T>*)L.fout, g, L.phys, ty, L.flag);
     }
     return cudaGetLastError();
 }
@@ -1731,7 +1555,7 @@ cudaError_t launch_step_test_timeout(const StepLaunch& L, cudaStream_t st) {
     }
     const int gx = (g.nx + kBlockTileW - 1) / kBlockTileW;
     dim3 grid(gx, std::max(1, std::min(g.ny / 8, 16)));
-    step_block_timeout_kernel<<<grid, kBlockTileW, smem, st>>>((const float*)L.fin, (float*)L.fout, g, L.phys, L.flag);
+    step_block_timeout_kernel<<<grid, kBlockTileW, smem, st>>>((const float2*)L.fin, (float2*)L.fout, g, L.phys, L.flag);
     return cudaGetLastError();
 }
 
@@ -1741,13 +1565,13 @@ cudaError_t launch_init(void* fout, const Grid& g, int storage, const float shif
     dim3 grid((g.nx + kThreadsX - 1) / kThreadsX, g.ny);
     switch (storage) {
         case LBM_STORE_F16:
-            init_kernel<__half><<<grid, kThreadsX, 0, st>>>((__half*)fout, g, shift[0], shift[1], y0, mass_A, mass_B, minority, width);
+            init_kernel<__half><<<grid, kThreadsX, 0, st>>>((__half2*)fout, g, shift[0], shift[1], y0, mass_A, mass_B, minority, width);
             break;
         case LBM_STORE_BF16:
-            init_kernel<__nv_bfloat16><<<grid, kThreadsX, 0, st>>>((__nv_bfloat16*)fout, g, shift[0], shift[1], y0, mass_A, mass_B, minority, width);
+            init_kernel<__nv_bfloat16><<<grid, kThreadsX, 0, st>>>((__nv_bfloat162*)fout, g, shift[0], shift[1], y0, mass_A, mass_B, minority, width);
             break;
         default:
-            init_kernel<float><<<grid, kThreadsX, 0, st>>>((float*)fout, g, shift[0], shift[1], y0, mass_A, mass_B, minority, width);
+            init_kernel<float><<<grid, kThreadsX, 0, st>>>((float2*)fout, g, shift[0], shift[1], y0, mass_A, mass_B, minority, width);
     }
     return cudaGetLastError();
 }
@@ -1758,14 +1582,14 @@ static cudaError_t launch_pull_to_host(const void* fin, const Grid& g, int stora
     dim3 grid((g.nx + kThreadsX - 1) / kThreadsX, g.ny);
     switch (storage) {
         case LBM_STORE_F16:
-            pull_to_host_kernel<__half, V><<<grid, kThreadsX, 0, st>>>((const __half*)fin, g, shift[0], shift[1], S);
+            pull_to_host_kernel<__half, V><<<grid, kThreadsX, 0, st>>>((const __half2*)fin, g, shift[0], shift[1], S);
             break;
         case LBM_STORE_BF16:
-            pull_to_host_kernel<__nv_bfloat16, V><<<grid, kThreadsX, 0, st>>>((const __nv_bfloat16*)fin, g, shift[0],
+            pull_to_host_kernel<__nv_bfloat16, V><<<grid, kThreadsX, 0, st>>>((const __nv_bfloat162*)fin, g, shift[0],
                                                                               shift[1], S);
             break;
         default:
-            pull_to_host_kernel<float, V><<<grid, kThreadsX, 0, st>>>((const float*)fin, g, shift[0], shift[1], S);
+            pull_to_host_kernel<float, V><<<grid, kThreadsX, 0, st>>>((const float2*)fin, g, shift[0], shift[1], S);
     }
     return cudaGetLastError();
 }
@@ -1776,16 +1600,35 @@ static cudaError_t launch_push_from_host(const V* S, const Grid& g, int storage,
     dim3 grid((g.nx + kThreadsX - 1) / kThreadsX, g.ny);
     switch (storage) {
         case LBM_STORE_F16:
-            push_from_host_kernel<__half, V><<<grid, kThreadsX, 0, st>>>(S, g, shift[0], shift[1], (__half*)fout);
+            push_from_host_kernel<__half, V><<<grid, kThreadsX, 0, st>>>(S, g, shift[0], shift[1], (__half2*)fout);
             break;
         case LBM_STORE_BF16:
             push_from_host_kernel<__nv_bfloat16, V><<<grid, kThreadsX, 0, st>>>(S, g, shift[0], shift[1],
-                                                                                (__nv_bfloat16*)fout);
+                                                                                (__nv_bfloat162*)fout);
             break;
         default:
-            push_from_host_kernel<float, V><<<grid, kThreadsX, 0, st>>>(S, g, shift[0], shift[1], (float*)fout);
+            push_from_host_kernel<float, V><<<grid, kThreadsX, 0, st>>>(S, g, shift[0], shift[1], (float2*)fout);
     }
     return cudaGetLastError();
+}
+
+template <bool kToPlanes>
+static cudaError_t launch_planes(void* pops, const Grid& g, int storage, void* planes, int pitch, int origin,
+                                 cudaStream_t st) {
+    dim3 grid((g.nx + 4 + kThreadsX - 1) / kThreadsX, g.ny);
+    if (storage == LBM_STORE_F32)
+        planes_kernel<uint32_t, kToPlanes><<<grid, kThreadsX, 0, st>>>((uint32_t*)pops, g, (uint32_t*)planes, pitch, origin);
+    else
+        planes_kernel<uint16_t, kToPlanes><<<grid, kThreadsX, 0, st>>>((uint16_t*)pops, g, (uint16_t*)planes, pitch, origin);
+    return cudaGetLastError();
+}
+cudaError_t launch_cells_to_planes(const void* pops, const Grid& g, int storage, void* planes, int pitch, int origin,
+                                   cudaStream_t st) {
+    return launch_planes<true>(const_cast<void*>(pops), g, storage, planes, pitch, origin, st);
+}
+cudaError_t launch_planes_to_cells(const void* planes, int pitch, int origin, const Grid& g, int storage, void* pops,
+                                   cudaStream_t st) {
+    return launch_planes<false>(pops, g, storage, const_cast<void*>(planes), pitch, origin, st);
 }
 
 cudaError_t launch_pull_to_double(const void* fin, const Grid& g, int storage, const float shift[2], double* S,
