@@ -28,6 +28,14 @@ __device__ __forceinline__ Nbr2 ring_nbr(const float2* S, const float2* C, const
     return p;
 }
 
+// Programmatic dependent launch: a step's blocks may become resident while the step
+// before it drains; they wait here, before their first access to global memory, until
+// that step has completed and its writes are visible.
+__device__ __forceinline__ void wait_previous_step() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // ---------------------------------------------------------------------------
 // Fused pull stream-collide.  A block owns kThreadsX columns and tile_y rows and
 // sweeps its rows bottom-up.  Each thread keeps the populations of its column for
@@ -1077,6 +1085,7 @@ step_pair_kernel(const Cell<T>* __restrict__ fin, Cell<T>* __restrict__ fout, Gr
     __shared__ __align__(16) PairRing sR;
     const int y0 = (int)(((long long)blockIdx.y * g.ny) / gridDim.y);
     const int y1 = (int)(((long long)(blockIdx.y + 1) * g.ny) / gridDim.y);
+    wait_previous_step();
     const uint32_t seed = launch_seed(ph);
     advance_step(ph, blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0);
     pair_tile<T>(fin, fout, g, ph, blockIdx.x * kWideTileW, y0, y1, dsm, sR, seed, flag);
@@ -1091,6 +1100,7 @@ step_block_kernel(const Cell<T>* __restrict__ fin, Cell<T>* __restrict__ fout, G
     __shared__ BlockRingT<TW> sR;
     const int y0 = (int)(((long long)blockIdx.y * g.ny) / gridDim.y);
     const int y1 = (int)(((long long)(blockIdx.y + 1) * g.ny) / gridDim.y);
+    wait_previous_step();
     const uint32_t seed = launch_seed(ph);
     advance_step(ph, blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0);
     block_tile<T, TW>(fin, fout, g, ph, blockIdx.x * TW, y0, y1, dsm, sR, seed, flag);
@@ -1346,15 +1356,21 @@ __global__ void planes_kernel(V* __restrict__ cells, Grid g, V* __restrict__ pla
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
-// Row tiles of the block-staged kernel: tile_y > 0 asks for at most tile_y rows per
-// tile; 0 fills the device's resident block slots exactly once (one wave, every SM
-// equally loaded) unless that leaves fewer than min_rows rows per tile.
-constexpr int kMinTileRows = 16;   // shortest default tile of the one-column-per-thread tiles
-int block_tiles_y(int ny, int tiles_x, int tile_y, int slots, int min_rows) {
-    if (tile_y > 0) return (ny + tile_y - 1) / tile_y;
-    const int per_wave = std::max(1, slots / tiles_x);
-    const int fit = std::max(1, ny / min_rows);
-    return std::min(per_wave, fit);
+// Row tiles of the staged kernels: tile_y > 0 asks for at most tile_y rows per tile; 0
+// makes the tiles as short as the device's resident block slots allow in one wave.  A
+// launch on a small grid is a serial chain of row barriers, one per row of a tile and two
+// before it, so the shortest tiles win down to one row although they read three rows for
+// each they write (us per step, FP32: 128x256 24.8 with 16-row tiles, 4.0 with 1-row ones;
+// 512x512 17.4 and 8.1 with 3 rows; 512x1024 19.4 and 12.6 with 5), while a second wave
+// costs more than shorter tiles gain (512x256: 1 row, 1024 tiles in 912 slots 7.7, 2 rows
+// 6.0).
+int block_tiles_y(int ny, int tiles_x, int tile_y, int slots) {
+    int rows = tile_y;
+    if (rows <= 0) {
+        const int per_wave = std::max(1, slots / tiles_x);
+        rows = (ny + per_wave - 1) / per_wave;
+    }
+    return (ny + rows - 1) / rows;
 }
 
 // Resident blocks of step_block_kernel<T, TW> on the current device (set up once per
@@ -1379,6 +1395,30 @@ static cudaError_t block_slots(int* slots) {
     return cudaSuccess;
 }
 
+// A launch that may start while the kernel before it on the stream drains (the kernels
+// call wait_previous_step), where that pays: for launches that leave room for the next
+// one's blocks (128x256 FP32 4.0 -> 3.5 us a step) and for those that fill the slots of
+// 128-thread blocks (512x1024 12.65 -> 12.26, 1024x2048 51.8 -> 51.0).  In between, blocks
+// that start early take the free slots of some SMs and leave the wave uneven (512x512, 684
+// blocks in 912 slots, 7.8 -> 8.2; 10000x5000, 280 in 304, 1103 -> 1131).
+template <typename... P, typename... A>
+static cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, int threads, size_t smem, int slots, cudaStream_t st,
+                                    A... args) {
+    const long long blocks = (long long)grid.x * grid.y;
+    const bool early = 3 * blocks <= slots || (threads == 128 && 100 * blocks >= 88LL * slots);
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = early ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 template <typename T, int TW>
 static cudaError_t launch_block(const StepLaunch& L, cudaStream_t st) {
     const Grid& g = L.grid;
@@ -1386,10 +1426,9 @@ static cudaError_t launch_block(const StepLaunch& L, cudaStream_t st) {
     cudaError_t e = block_slots<T, TW>(&slots);
     if (e != cudaSuccess) return e;
     const int gx = (g.nx + TW - 1) / TW;
-    dim3 grid(gx, block_tiles_y(g.ny, gx, L.tile_y, slots, kMinTileRows));
-    step_block_kernel<T, TW><<<grid, TW, block_smem_bytes<T, TW>(), st>>>((const Cell<T>*)L.fin, (Cell<T>*)L.fout, g, L.phys,
-                                                                           L.flag);
-    return cudaGetLastError();
+    dim3 grid(gx, block_tiles_y(g.ny, gx, L.tile_y, slots));
+    return launch_dependent(step_block_kernel<T, TW>, grid, TW, block_smem_bytes<T, TW>(), slots, st, (const Cell<T>*)L.fin,
+                            (Cell<T>*)L.fout, g, L.phys, L.flag);
 }
 
 // Resident blocks of step_dec_kernel<T, TW> (attribute set once per instantiation).
@@ -1419,12 +1458,11 @@ static cudaError_t launch_dec(const StepLaunch& L, cudaStream_t st) {
     cudaError_t e = dec_slots<T, TW>(&slots);
     if (e != cudaSuccess) return e;
     const int gx = (g.nx + TW - 1) / TW;
-    dim3 grid(gx, block_tiles_y(g.ny, gx, L.tile_y, slots, kMinTileRows));
+    dim3 grid(gx, block_tiles_y(g.ny, gx, L.tile_y, slots));
     step_dec_kernel<T, TW><<<grid, TW, dec_smem_bytes<T, TW>(), st>>>((const Cell<T>*)L.fin, (Cell<T>*)L.fout, g, L.phys, L.flag);
     return cudaGetLastError();
 }
 
-// Paired tiles go down to 8 rows so that the wave is full.
 template <typename T>
 static cudaError_t launch_pair(const StepLaunch& L, cudaStream_t st) {
     static int slots = 0;
@@ -1442,14 +1480,13 @@ static cudaError_t launch_pair(const StepLaunch& L, cudaStream_t st) {
     }
     const Grid& g = L.grid;
     const int gx = (g.nx + kWideTileW - 1) / kWideTileW;
-    dim3 grid(gx, block_tiles_y(g.ny, gx, L.tile_y, slots, 8));
-    step_pair_kernel<T><<<grid, kPairThreads, pair_smem_bytes<T>(), st>>>((const Cell<T>*)L.fin, (Cell<T>*)L.fout, g,
-                                                                           L.phys, L.flag);
-    return cudaGetLastError();
+    dim3 grid(gx, block_tiles_y(g.ny, gx, L.tile_y, slots));
+    return launch_dependent(step_pair_kernel<T>, grid, kPairThreads, pair_smem_bytes<T>(), slots, st, (const Cell<T>*)L.fin,
+                            (Cell<T>*)L.fout, g, L.phys, L.flag);
 }
 
 // Columns per one-column-per-thread tile: tile_x when it is 128 or 256; otherwise 256
-// for 16-bit storage, and for FP32 when the 256-column tiles hold at least kWideMinRows
+// for 16-bit storage unless 128 span the grid, and for FP32 when the 256-column tiles hold at least kWideMinRows
 // rows (tile_y, or the rows of the one-wave default).  The wider tile reads half the halo
 // columns and wins where tiles are tall (FP32 at 10000x5000: 1101 us a step against 1119);
 // tiles of 27 rows (1024x2048) run 51.4 us at 128 columns and 53.3 at 256, the barrier of 8
@@ -1462,14 +1499,14 @@ static cudaError_t block_tile_width(const Grid& g, int tile_x, int tile_y, int* 
         return cudaSuccess;
     }
     if (IsShifted<T>::value) {
-        *tw = kWideTileW;
+        *tw = g.nx > kBlockTileW ? kWideTileW : kBlockTileW;
         return cudaSuccess;
     }
     int slots = 0;
     cudaError_t e = block_slots<T, kWideTileW>(&slots);
     if (e != cudaSuccess) return e;
     const int gx = (g.nx + kWideTileW - 1) / kWideTileW;
-    const int rows = tile_y > 0 ? tile_y : g.ny / block_tiles_y(g.ny, gx, 0, slots, kMinTileRows);
+    const int rows = tile_y > 0 ? tile_y : g.ny / block_tiles_y(g.ny, gx, 0, slots);
     *tw = rows >= kWideMinRows ? kWideTileW : kBlockTileW;
     return cudaSuccess;
 }
@@ -1486,9 +1523,10 @@ static cudaError_t launch_step_t(const StepLaunch& L, int kernel, cudaStream_t s
     } else if (kernel == LBM_KERNEL_STAGED || kernel == LBM_KERNEL_PAIRED) {
         // 16-bit storage at the default width: the paired-column tile (same results bit for
         // bit; FP16 at 1024x2048 36.2 us a step against 38.1 of the 256-thread tile, at
-        // 10000x5000 783 against 859, at 1501x999 27.1 against 35.7)
+        // 10000x5000 783 against 859, at 1501x999 27.1 against 35.7), except where one
+        // 128-column tile spans the grid (128x256: 4.6 us against 5.1)
         if constexpr (IsShifted<T>::value)
-            if (kernel == LBM_KERNEL_PAIRED || L.tile_x == 0) return launch_pair<T>(L, st);
+            if (kernel == LBM_KERNEL_PAIRED || (L.tile_x == 0 && g.nx > kBlockTileW)) return launch_pair<T>(L, st);
         int tw = 0;
         cudaError_t e = block_tile_width<T>(g, L.tile_x, L.tile_y, &tw);
         if (e != cudaSuccess) return e;
