@@ -109,9 +109,9 @@ typedef struct {
                               * LBM_KERNEL_PAIRED kernel), for FP32 256 when the 256-column tiles
                               * are at least 64 rows tall, else 128.  Other kernels ignore it.
                               * Ensembles (the first member's value): 128 or 256 columns, one
-                              * per thread, for every member; 0 = blocks of 128 threads, FP32
-                              * members in 128-column tiles and 16-bit members in paired
-                              * 256-column tiles (lbm_ens_tune picks among the three). */
+                              * per thread, for every member; 0 = 16-bit members in paired
+                              * 256-column tiles, FP32 members in 128-column ones, or 256
+                              * where tiles are tall (lbm_ens_tune picks among the three). */
     int32_t wall_mode;       /* pseudopotential beyond the walls in the Shan-Chen force (Section 2
                               * leaves it open): 0 = none (psi = 0 on the virtual rows y = -1 and
                               * y = ny); 1 = mirror (those rows hold the wall rows' own psi: a
@@ -287,13 +287,15 @@ lbm_status lbm_tune(lbm_handle* h, const char* cache_path, int32_t* tile_y, doub
 lbm_status lbm_get_params(lbm_handle* h, lbm_params* out);
 
 /* ---- Ensembles of independent realisations (Section 2: at least 10 runs per
- * experiment).  One kernel launch per time step advances every member; chunks
- * of steps are replayed as CUDA graphs.  Members may differ in grid, physics and
- * storage; each uses the staged kernel and its own workspace. ---- */
+ * experiment).  One kernel launch per time step advances all members of a chain (up
+ * to two chains per storage type, side by side on streams of the ensemble that fork
+ * from its stream and join it again within a call); chunks of steps are replayed as
+ * CUDA graphs.  Members may differ in grid, physics and storage; each uses the staged
+ * kernel and its own workspace. ---- */
 typedef struct lbm_ensemble lbm_ensemble;
 
 /* n parameter sets (1..256); tile_y of members[0] is the rows per tile of every
- * member (0: chosen so that the tiles fill the device's block slots in whole waves).  cuda_stream: a cudaStream_t shared by all members, or NULL for one owned
+ * member (0: chosen from the members' sizes and the device's block slots).  cuda_stream: a cudaStream_t shared by all members, or NULL for one owned
  * by the ensemble. */
 lbm_status lbm_ens_create(int32_t n, const lbm_params* members, void* cuda_stream, lbm_ensemble** out);
 
@@ -312,7 +314,7 @@ lbm_status lbm_ens_diagnostics(lbm_ensemble* e, lbm_diag* out);
 
 /* Pick the tile shape for the whole ensemble by timing candidates: the three tile
  * widths of lbm_params.tile_x (128, 256, 0 = paired 16-bit tiles) times tile heights
- * (0, the slot-filling default, among them); states are kept.  tile_y receives the
+ * (0, the default but at least 12 rows, among them); states are kept.  tile_y receives the
  * rows per tile in use.  The initial width is the first member's tile_x when it is
  * 128 or 256, else 0. */
 lbm_status lbm_ens_tune(lbm_ensemble* e, int32_t* tile_y, double* ms_per_step);

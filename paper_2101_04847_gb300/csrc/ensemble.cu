@@ -1,12 +1,16 @@
 // Ensembles of independent realisations (the paper runs at least 10 per
-// experiment, Section 2): one kernel launch per time step advances every member
-// (ensemble_step_kernel, step_kernels.cu: the block-staged tile code over a flat
-// list of every member's tiles), and chunks of steps are captured in CUDA graphs.  Members may differ in grid size, physics and storage type; each
-// member is a full lbm_handle (init, diagnostics, fields, checkpoints) that only
-// the ensemble steps.
+// experiment, Section 2): members may differ in grid size, physics and storage type;
+// each is a full lbm_handle (init, diagnostics, fields, checkpoints) that only the
+// ensemble steps.  The members of one storage type form chains; one launch per time
+// step advances a chain (ensemble_step_kernel, step_kernels.cu: the single-grid tile
+// code over a flat list of its members' tiles).  Members never wait for one another, so
+// the chains run side by side on streams of their own, joined at the end of a call: one
+// chain's blocks fill the SMs that the end of another's launch leaves idle.  Chunks of
+// steps are captured in CUDA graphs.
 #include "lbm_internal.cuh"
 
 #include <algorithm>
+#include <cmath>
 #include <string>
 #include <vector>
 
@@ -14,6 +18,7 @@ namespace {
 
 constexpr int kEnsGraphChunk = 50;
 constexpr int kEnsMaxMembers = 256;
+constexpr int kTuneMinRows = 12;   // shortest tile that lbm_ens_tune picks
 
 lbm_status ens_fail(lbm_status st, const std::string& msg) {
     lbm::set_last_error(msg);
@@ -28,19 +33,31 @@ lbm_status ens_fail(lbm_status st, const std::string& msg) {
 
 }  // namespace
 
+// Members of one storage type advanced by one launch per time step.
+struct EnsChain {
+    lbm::EnsKernel kernel;
+    int storage = 0;
+    std::vector<lbm_handle*> members;
+    int begin = 0;        // its first member in the table
+    int tiles = 0;
+    cudaStream_t stream = nullptr;   // the ensemble's own for the first chain
+    cudaEvent_t done = nullptr;      // the other chains': joins them to the ensemble's stream
+};
+
 struct lbm_ensemble {
     std::vector<lbm_handle*> members;
+    std::vector<EnsChain> chains;
     std::vector<lbm::EnsMember> table;
     lbm::EnsMember* d_table = nullptr;
-    int total_tiles = 0;
     int tile_x = lbm::kEnsAuto;      // 128 or 256 columns per tile (one per thread), or kEnsAuto
     int tile_y = 0;       // requested rows per tile; 0: chosen from the device's block slots
     int rows = 0;         // rows per tile in use
-    size_t smem = 0;      // dynamic shared memory per block (largest storage type present)
+    int min_rows = 1;     // at least so many rows when chosen (the tuner's shapes: kTuneMinRows)
     int parity = 0;
     int64_t step = 0;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
+    cudaEvent_t fork = nullptr;
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
 };
 
@@ -59,67 +76,96 @@ int tiles_of(const lbm::Grid& g, int tile_x, int rows, int* tx, int* ty) {
     return *tx * *ty;
 }
 
-// Rows per tile when none is requested: the height whose tile count fills the
-// resident block slots in whole waves best, weighted by the share of rows that
-// are not halo (3 halo rows per tile).
-int auto_rows(const lbm_ensemble* e, int slots) {
-    int best = 32;
-    double best_score = -1.0;
-    for (int rows = 12; rows <= 256; ++rows) {
-        long long tiles = 0;
-        for (lbm_handle* h : e->members) {
-            int tx, ty;
-            tiles += tiles_of(lbm::handle_grid(h), lbm::ensemble_tile_cols(lbm::handle_params(h).storage, e->tile_x),
-                              rows, &tx, &ty);
-        }
-        const long long waves = (tiles + slots - 1) / slots;
-        const double score = (double)tiles / (double)(waves * slots) * rows / (rows + 3.0);
-        if (score > best_score + 1e-9) {
-            best_score = score;
-            best = rows;
-        }
-    }
-    return best;
+// Rows per tile when none is requested: about two waves of tiles over all chains together.
+// Short tiles read more halo rows, tall ones leave the chains too few blocks to fill the
+// slots the others leave.  us per step: ten FP32 256x512 members 41.3 with 2 rows, 35.8
+// with 4, 41.8 with 12 (0.9 waves); sixteen FP16 512x1024 120.9 with 16, 117.7 with 24, 132
+// with 48; ten FP32 1024x2048 502 with 16, 485 with 48 and 64, 539 with 187 (one wave).  A
+// launch that fits the slots is fastest with one row (one 128x256 member 4.0, 4.6 with 2);
+// beyond that two rows are the least that pay (eight 128x256 members 14.5 with 1, 10.2).
+constexpr int kMaxAutoRows = 48;
+constexpr int kWideRows = 16;     // FP32 tiles of so many rows are 256 columns wide
+int auto_rows(double waves_of_one_row, int min_rows) {
+    if (waves_of_one_row <= 1.0) return min_rows;
+    const int rows = (int)std::ceil(std::min(waves_of_one_row / 2.0, (double)kMaxAutoRows));
+    return std::max({2, rows, min_rows});
 }
 
-// (Re)build the member table for the current tile height and upload it.
+// The chains of an ensemble: its members by storage type, each type's in up to
+// kChainsPerType chains of about equal size.  Two cover each other's ends of launches
+// (sixteen FP16 512x1024 members 140 us a step in one chain, 118 in two; ten FP32
+// 1024x2048 511 and 485); more gain nothing further (116 to 121, 485).
+constexpr int kChainsPerType = 2;
+lbm_status ens_build_chains(lbm_ensemble* e) {
+    for (int st : {LBM_STORE_F32, LBM_STORE_F16, LBM_STORE_BF16}) {
+        std::vector<lbm_handle*> of;
+        for (lbm_handle* h : e->members)
+            if (lbm::handle_params(h).storage == st) of.push_back(h);
+        const int n = std::min<int>(kChainsPerType, (int)of.size());
+        std::vector<EnsChain> part(n);
+        std::vector<double> size(n, 0.0);
+        auto sites = [](lbm_handle* h) { return (double)lbm::handle_grid(h).nx * lbm::handle_grid(h).ny; };
+        std::stable_sort(of.begin(), of.end(), [&](lbm_handle* a, lbm_handle* b) { return sites(a) > sites(b); });
+        for (lbm_handle* h : of) {   // the largest first, each to the smallest chain
+            const int k = (int)(std::min_element(size.begin(), size.end()) - size.begin());
+            part[k].members.push_back(h);
+            size[k] += sites(h);
+        }
+        for (EnsChain& c : part) {
+            c.storage = st;
+            if (e->chains.empty()) {
+                c.stream = e->stream;
+            } else {
+                cudaError_t err = cudaStreamCreateWithFlags(&c.stream, cudaStreamNonBlocking);
+                if (err == cudaSuccess) err = cudaEventCreateWithFlags(&c.done, cudaEventDisableTiming);
+                if (err != cudaSuccess) {
+                    if (c.stream) cudaStreamDestroy(c.stream);
+                    return ens_fail(LBM_ECUDA, std::string("ensemble stream: ") + cudaGetErrorString(err));
+                }
+            }
+            e->chains.push_back(c);
+        }
+    }
+    if (e->chains.size() > 1)
+        ENS_TRY(cudaEventCreateWithFlags(&e->fork, cudaEventDisableTiming), "ensemble event");
+    return LBM_OK;
+}
+
+// (Re)build the member table for the current tile shape and upload it.
 lbm_status ens_build_table(lbm_ensemble* e) {
     e->table.clear();
-    e->smem = 0;
-    for (lbm_handle* h : e->members)
-        e->smem = std::max(e->smem, lbm::block_tile_smem_bytes(lbm::handle_params(h).storage, e->tile_x));
-    if (e->tile_y > 0) {
-        e->rows = e->tile_y;
-    } else {
-        cudaError_t err = cudaSuccess;
-        const int slots = lbm::ensemble_slots(e->smem, e->tile_x, &err);
-        ENS_TRY(err, "ensemble occupancy");
-        e->rows = auto_rows(e, slots);
+    double waves = 0.0;   // of one-row tiles, all chains
+    for (EnsChain& c : e->chains) {
+        c.kernel = lbm::ensemble_kernel(c.storage, e->tile_x);
+        int slots = 1, tx, ty;
+        ENS_TRY(lbm::ensemble_slots(c.kernel, &slots), "ensemble occupancy");
+        for (lbm_handle* h : c.members) waves += (double)tiles_of(lbm::handle_grid(h), c.kernel.cols, 1, &tx, &ty) / slots;
     }
-    // Tiles of one storage type are contiguous in the flat list, so that the blocks
-    // resident at one time mostly run one instantiation of the tile code (mixing
-    // them on an SM thrashes its instruction cache).
-    std::vector<lbm_handle*> order;
-    for (int st : {LBM_STORE_F32, LBM_STORE_F16, LBM_STORE_BF16})
-        for (lbm_handle* h : e->members)
-            if (lbm::handle_params(h).storage == st) order.push_back(h);
-    int begin = 0;
-    for (lbm_handle* h : order) {
-        lbm::EnsMember m;
-        m.grid = lbm::handle_grid(h);
-        m.phys = lbm::handle_phys(h);
-        m.buf[0] = lbm::handle_buffer(h, 0);
-        m.buf[1] = lbm::handle_buffer(h, 1);
-        m.flag = lbm::handle_flag(h);
-        m.storage = lbm::handle_params(h).storage;
-        m.step_ctr = lbm::handle_step_counters(h);
-        const int tiles = tiles_of(m.grid, lbm::ensemble_tile_cols(m.storage, e->tile_x), e->rows, &m.tiles_x,
-                                   &m.tiles_y);
-        m.tile_begin = begin;
-        begin += tiles;
-        e->table.push_back(m);
+    e->rows = e->tile_y > 0 ? e->tile_y : auto_rows(waves, e->min_rows);
+    for (EnsChain& c : e->chains) {
+        // tall FP32 tiles: 256 columns, as on one grid (ten 1024x2048 members 486 -> 461 us a
+        // step, sixteen 512x1024 209 -> 192; short ones lose, eight 128x256 10 -> 13)
+        if (e->tile_x == lbm::kEnsAuto && c.storage == LBM_STORE_F32 && e->rows >= kWideRows) {
+            c.kernel = lbm::ensemble_kernel(c.storage, lbm::kWideTileW);
+            int slots = 1;
+            ENS_TRY(lbm::ensemble_slots(c.kernel, &slots), "ensemble occupancy");
+        }
+        c.begin = (int)e->table.size();
+        c.tiles = 0;
+        for (lbm_handle* h : c.members) {
+            lbm::EnsMember m;
+            m.grid = lbm::handle_grid(h);
+            m.phys = lbm::handle_phys(h);
+            m.buf[0] = lbm::handle_buffer(h, 0);
+            m.buf[1] = lbm::handle_buffer(h, 1);
+            m.flag = lbm::handle_flag(h);
+            m.step_ctr = lbm::handle_step_counters(h);
+            const int tiles = tiles_of(m.grid, c.kernel.cols, e->rows, &m.tiles_x, &m.tiles_y);
+            m.tile_begin = c.tiles;
+            c.tiles += tiles;
+            e->table.push_back(m);
+        }
     }
-    e->total_tiles = begin;
     ENS_TRY(cudaMemcpyAsync(e->d_table, e->table.data(), e->table.size() * sizeof(lbm::EnsMember),
                             cudaMemcpyHostToDevice, e->stream), "upload member table");
     ENS_TRY(cudaStreamSynchronize(e->stream), "sync");
@@ -127,13 +173,32 @@ lbm_status ens_build_table(lbm_ensemble* e) {
     return LBM_OK;
 }
 
-lbm_status ens_launch(lbm_ensemble* e, int64_t n) {
-    for (int64_t k = 0; k < n; ++k) {
-        ENS_TRY(lbm::launch_ensemble_step(e->d_table, (int)e->members.size(), e->total_tiles, e->parity, e->smem,
-                                          e->tile_x, e->stream),
-                "ensemble step");
-        e->parity ^= 1;
+// n steps from the given parity: the chains fork from the ensemble's stream and join it
+// again whatever happens in between.
+cudaError_t ens_launch_steps(lbm_ensemble* e, int parity, int64_t n) {
+    cudaError_t err = cudaSuccess;
+    if (n <= 0) return err;
+    if (e->chains.size() > 1 && (err = cudaEventRecord(e->fork, e->stream)) != cudaSuccess) return err;
+    for (EnsChain& c : e->chains) {
+        const bool side = c.stream != e->stream;
+        cudaError_t ce = side ? cudaStreamWaitEvent(c.stream, e->fork, 0) : cudaSuccess;
+        for (int64_t k = 0; k < n && ce == cudaSuccess; ++k)
+            ce = lbm::launch_ensemble_step(c.kernel, e->d_table + c.begin, (int)c.members.size(), c.tiles,
+                                           (int)((parity + k) & 1), c.stream);
+        if (err == cudaSuccess) err = ce;
     }
+    for (EnsChain& c : e->chains)
+        if (c.stream != e->stream) {
+            cudaError_t ce = cudaEventRecord(c.done, c.stream);
+            if (ce == cudaSuccess) ce = cudaStreamWaitEvent(e->stream, c.done, 0);
+            if (err == cudaSuccess) err = ce;
+        }
+    return err;
+}
+
+lbm_status ens_launch(lbm_ensemble* e, int64_t n) {
+    ENS_TRY(ens_launch_steps(e, e->parity, n), "ensemble step");
+    e->parity ^= (int)(n & 1);
     return LBM_OK;
 }
 
@@ -142,17 +207,14 @@ lbm_status ens_graph(lbm_ensemble* e, cudaGraphExec_t* out) {
     if (!e->graph[par]) {
         cudaGraph_t g = nullptr;
         ENS_TRY(cudaStreamBeginCapture(e->stream, cudaStreamCaptureModeThreadLocal), "begin capture");
-        for (int k = 0; k < kEnsGraphChunk; ++k) {
-            cudaError_t err = lbm::launch_ensemble_step(e->d_table, (int)e->members.size(), e->total_tiles,
-                                                        (par + k) & 1, e->smem, e->tile_x, e->stream);
-            if (err != cudaSuccess) {
-                cudaStreamEndCapture(e->stream, &g);
-                if (g) cudaGraphDestroy(g);
-                return ens_fail(LBM_ECUDA, std::string("capture ensemble step: ") + cudaGetErrorString(err));
-            }
+        cudaError_t err = ens_launch_steps(e, par, kEnsGraphChunk);
+        const cudaError_t end = cudaStreamEndCapture(e->stream, &g);
+        if (err == cudaSuccess) err = end;
+        if (err != cudaSuccess) {
+            if (g) cudaGraphDestroy(g);
+            return ens_fail(LBM_ECUDA, std::string("capture ensemble step: ") + cudaGetErrorString(err));
         }
-        ENS_TRY(cudaStreamEndCapture(e->stream, &g), "end capture");
-        cudaError_t err = cudaGraphInstantiate(&e->graph[par], g, 0);
+        err = cudaGraphInstantiate(&e->graph[par], g, 0);
         cudaGraphDestroy(g);
         if (err != cudaSuccess) return ens_fail(LBM_ECUDA, std::string("instantiate: ") + cudaGetErrorString(err));
     }
@@ -172,6 +234,11 @@ void lbm_ens_destroy(lbm_ensemble* e) {
         lbm::handle_set_ensemble(h, false);
         lbm_destroy(h);
     }
+    for (EnsChain& c : e->chains) {
+        if (c.done) cudaEventDestroy(c.done);
+        if (c.stream && c.stream != e->stream) cudaStreamDestroy(c.stream);
+    }
+    if (e->fork) cudaEventDestroy(e->fork);
     if (e->d_table) cudaFree(e->d_table);
     if (e->own_stream && e->stream) cudaStreamDestroy(e->stream);
     delete e;
@@ -214,7 +281,8 @@ lbm_status lbm_ens_create(int32_t n, const lbm_params* params, void* cuda_stream
         lbm_ens_destroy(e);
         return ens_fail(LBM_ENOMEM, "member table");
     }
-    lbm_status st = ens_build_table(e);
+    lbm_status st = ens_build_chains(e);
+    if (st == LBM_OK) st = ens_build_table(e);
     if (st != LBM_OK) {
         const std::string msg = lbm_last_error();
         lbm_ens_destroy(e);
@@ -272,7 +340,8 @@ lbm_status lbm_ens_diagnostics(lbm_ensemble* e, lbm_diag* out) {
 
 lbm_status lbm_ens_tune(lbm_ensemble* e, int32_t* tile_y_out, double* ms_out) {
     if (!e) return ens_fail(LBM_EINVAL, "ensemble is NULL");
-    const int cand[] = {0, 12, 16, 20, 24, 32, 48, 64, 96};   // 0: the slot-filling default
+    e->min_rows = kTuneMinRows;
+    const int cand[] = {0, 12, 16, 20, 24, 32, 48, 64, 96};   // 0: the default
     const int widths[] = {lbm::kEnsAuto, lbm::kBlockTileW, lbm::kWideTileW};
     cudaEvent_t a, b;
     ENS_TRY(cudaEventCreate(&a), "event");

@@ -70,7 +70,8 @@ struct Grid {
 // ensemble kernel's and the narrow single-grid tile, and the wide single-grid tile.
 constexpr int kBlockTileW = 128;
 constexpr int kWideTileW = 256;
-// Ensemble tile width 0: chosen by the library (128 columns).
+// Ensemble tile width 0: FP32 members in tiles of 128 columns (one per thread), 16-bit
+// members in paired-column tiles of 256 (two per thread).
 constexpr int kEnsAuto = 0;
 
 struct StepLaunch {
@@ -91,24 +92,26 @@ struct EnsMember {
     Physics phys;
     void* buf[2];        // the two population buffers (input = buf[parity])
     int* flag;           // the member's guard flag
-    int storage;         // lbm_storage
     uint32_t* step_ctr;  // the member's two time-step counters (see Physics)
-    int tiles_x;         // block tiles along x (ensemble_tile_cols columns each)
+    int tiles_x;         // block tiles along x (EnsKernel::cols columns each)
     int tiles_y;         // block tiles along y (rows split evenly)
-    int tile_begin;      // index of the member's first tile in the flat list
+    int tile_begin;      // index of the member's first tile in its chain's flat list
 };
 
 // ensemble / tiling helpers (step_kernels.cu)
 int warp_tiles(const Grid& g, int tile_y, int* tiles_x);
 int default_tile_y();
-// columns of one ensemble tile of a member with this storage (tile_x 128, 256 or kEnsAuto)
-int ensemble_tile_cols(int storage, int tile_x);
-// dynamic shared memory of one block tile for a storage type
-size_t block_tile_smem_bytes(int storage, int tile_x);
-// resident blocks of the ensemble kernel on the current device with `smem` bytes each
-int ensemble_slots(size_t smem, int tile_x, cudaError_t* err);
-cudaError_t launch_ensemble_step(const EnsMember* d_members, int n, int total_tiles, int parity, size_t smem,
-                                 int tile_x, cudaStream_t st);
+// The ensemble kernel of one storage type at tile width tile_x (128, 256 or kEnsAuto):
+// columns per tile, threads and dynamic shared memory per block.
+struct EnsKernel {
+    void (*fn)(const EnsMember*, int, int);
+    int cols, threads;
+    size_t smem;
+};
+EnsKernel ensemble_kernel(int storage, int tile_x);
+cudaError_t ensemble_slots(const EnsKernel& k, int* slots);
+cudaError_t launch_ensemble_step(const EnsKernel& k, const EnsMember* d_members, int n, int tiles, int parity,
+                                 cudaStream_t st);
 
 // handle accessors for the ensemble (lbm_api.cu)
 void* handle_buffer(lbm_handle* h, int k);

@@ -1119,17 +1119,25 @@ step_block_timeout_kernel(const float2* __restrict__ fin, float2* __restrict__ f
 }
 
 // ---------------------------------------------------------------------------
-// Ensemble step: one launch advances every member by one time step.  Block b takes
-// tile b of the flat list that concatenates the members' block tiles (members in
-// order, each member's tiles row-major) and runs the block-staged tile code with
-// the member's grid, physics and storage type; no member waits for another, so
-// uneven grids need no barrier.
+// Ensemble step: one launch advances every member of one storage type by one time step.
+// Block b takes tile b of the flat list that concatenates the members' tiles (members in
+// order, each member's tiles row-major) and runs the tile code of the single-grid kernels
+// with the member's grid and physics; no member waits for another, so uneven grids need
+// no barrier.  TW 128 or 256: one column per thread; kEnsAuto: FP32 in 128-column tiles,
+// 16-bit storage in paired 256-column tiles.
 // ---------------------------------------------------------------------------
-template <int TW>
-__global__ void __launch_bounds__(TW, 768 / TW)
+template <typename T, int TW> struct EnsTile {
+    static constexpr bool kPaired = TW == kEnsAuto && IsShifted<T>::value;
+    static constexpr int kCols = kPaired ? kWideTileW : (TW == kEnsAuto ? kBlockTileW : TW);
+    static constexpr int kThreads = kPaired ? kPairThreads : kCols;
+    static constexpr int kBlocks = kPaired ? 4 : TileCfg<T, kCols>::kBlocks;
+};
+
+template <typename T, int TW>
+__global__ void __launch_bounds__(EnsTile<T, TW>::kThreads, EnsTile<T, TW>::kBlocks)
 ensemble_step_kernel(const EnsMember* __restrict__ members, int n, int parity) {
+    typedef EnsTile<T, TW> E;
     extern __shared__ __align__(128) unsigned char dsm[];
-    __shared__ BlockRingT<TW> sR;
     const int tile = blockIdx.x;
     int lo = 0, hi = n - 1;   // last member whose first tile is <= tile
     while (lo < hi) {
@@ -1142,77 +1150,62 @@ ensemble_step_kernel(const EnsMember* __restrict__ members, int n, int parity) {
     const int tx = local % M.tiles_x, ty = local / M.tiles_x;
     const int y0 = (int)(((long long)ty * M.grid.ny) / M.tiles_y);
     const int y1 = (int)(((long long)(ty + 1) * M.grid.ny) / M.tiles_y);
-    const void* fin = M.buf[parity];
-    void* fout = M.buf[parity ^ 1];
+    const Cell<T>* fin = (const Cell<T>*)M.buf[parity];
+    Cell<T>* fout = (Cell<T>*)M.buf[parity ^ 1];
     Physics ph = M.phys;   // the member's counters, read / written as this parity dictates
     ph.step_in = M.step_ctr + parity;
     ph.step_out = M.step_ctr + (parity ^ 1);
     const uint32_t seed = launch_seed(ph);
     advance_step(ph, local == 0 && threadIdx.x == 0);
-    switch (M.storage) {
-        case LBM_STORE_F16:
-            block_tile<__half, TW>((const __half2*)fin, (__half2*)fout, M.grid, ph, tx * TW, y0, y1, dsm, sR, seed,
-                                   M.flag);
-            break;
-        case LBM_STORE_BF16:
-            block_tile<__nv_bfloat16, TW>((const __nv_bfloat162*)fin, (__nv_bfloat162*)fout, M.grid, ph, tx * TW, y0, y1,
-                                          dsm, sR, seed, M.flag);
-            break;
-        default:
-            block_tile<float, TW>((const float2*)fin, (float2*)fout, M.grid, ph, tx * TW, y0, y1, dsm, sR, seed, M.flag);
+    if constexpr (E::kPaired) {
+        __shared__ __align__(16) PairRing sR;
+        pair_tile<T>(fin, fout, M.grid, ph, tx * E::kCols, y0, y1, dsm, sR, seed, M.flag);
+    } else {
+        __shared__ BlockRingT<E::kCols> sR;
+        block_tile<T, E::kCols>(fin, fout, M.grid, ph, tx * E::kCols, y0, y1, dsm, sR, seed, M.flag);
     }
 }
 
-// kEnsNarrow (0) and 128: 128-column tiles
-static bool ens_wide(int tile_x) { return tile_x == kWideTileW; }
-
-int ensemble_tile_cols(int storage, int tile_x) {
-    (void)storage;
-    return ens_wide(tile_x) ? kWideTileW : kBlockTileW;
+template <typename T, int TW>
+static EnsKernel ens_kernel_of() {
+    typedef EnsTile<T, TW> E;
+    EnsKernel k;
+    k.fn = ensemble_step_kernel<T, TW>;
+    k.cols = E::kCols;
+    k.threads = E::kThreads;
+    if constexpr (E::kPaired) k.smem = pair_smem_bytes<T>();
+    else k.smem = block_smem_bytes<T, E::kCols>();
+    return k;
 }
-
-size_t block_tile_smem_bytes(int storage, int tile_x) {
-    if (ens_wide(tile_x))
-        return storage == LBM_STORE_F32 ? block_smem_bytes<float, kWideTileW>() : block_smem_bytes<__half, kWideTileW>();
-    return storage == LBM_STORE_F32 ? block_smem_bytes<float>() : block_smem_bytes<__half>();
+template <typename T>
+static EnsKernel ens_kernel_of(int tile_x) {
+    return tile_x == kWideTileW ? ens_kernel_of<T, kWideTileW>()
+           : tile_x == kBlockTileW ? ens_kernel_of<T, kBlockTileW>() : ens_kernel_of<T, kEnsAuto>();
 }
-
-template <int TW>
-static cudaError_t ensemble_attr() {
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(ensemble_step_kernel<TW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)block_smem_bytes<float, TW>());
-        if (e != cudaSuccess) return e;
-        attr_set = true;
+EnsKernel ensemble_kernel(int storage, int tile_x) {
+    switch (storage) {
+        case LBM_STORE_F16: return ens_kernel_of<__half>(tile_x);
+        case LBM_STORE_BF16: return ens_kernel_of<__nv_bfloat16>(tile_x);
+        default: return ens_kernel_of<float>(tile_x);
     }
-    return cudaSuccess;
 }
 
-// Resident blocks of the ensemble kernel of tile width tile_x for `smem` bytes.
-int ensemble_slots(size_t smem, int tile_x, cudaError_t* err) {
+// Resident blocks of an ensemble kernel on the current device (its dynamic shared memory
+// allowed first).
+cudaError_t ensemble_slots(const EnsKernel& k, int* slots) {
     int dev = 0, sms = 0, occ = 0;
-    const bool wide = ens_wide(tile_x);
-    cudaError_t e = wide ? ensemble_attr<kWideTileW>() : ensemble_attr<kBlockTileW>();
+    cudaError_t e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem);
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess)
-        e = wide ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, ensemble_step_kernel<kWideTileW>, kWideTileW, smem)
-                 : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, ensemble_step_kernel<kBlockTileW>, kBlockTileW,
-                                                                 smem);
-    if (err) *err = e;
-    return std::max(1, sms * occ);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k.fn, k.threads, k.smem);
+    *slots = std::max(1, sms * occ);
+    return e;
 }
 
-cudaError_t launch_ensemble_step(const EnsMember* d_members, int n, int total_tiles, int parity, size_t smem,
-                                 int tile_x, cudaStream_t st) {
+cudaError_t launch_ensemble_step(const EnsKernel& k, const EnsMember* d_members, int n, int tiles, int parity,
+                                 cudaStream_t st) {
     (void)cudaGetLastError();
-    cudaError_t e = ens_wide(tile_x) ? ensemble_attr<kWideTileW>() : ensemble_attr<kBlockTileW>();
-    if (e != cudaSuccess) return e;
-    if (ens_wide(tile_x))
-        ensemble_step_kernel<kWideTileW><<<total_tiles, kWideTileW, smem, st>>>(d_members, n, parity);
-    else
-        ensemble_step_kernel<kBlockTileW><<<total_tiles, kBlockTileW, smem, st>>>(d_members, n, parity);
+    k.fn<<<tiles, k.threads, k.smem, st>>>(d_members, n, parity);
     return cudaGetLastError();
 }
 
