@@ -493,8 +493,8 @@ step_pipe_kernel(const Cell<T>* __restrict__ fin, Cell<T>* __restrict__ fout, Gr
 // stores and address arithmetic (FP32 492 -> 323 instructions per site, paired FP16 500 ->
 // 361), a window of TW + 4 FP32 cells needs no alignment slack (34 sectors read per 32
 // owned at 128 columns, 36 before), and a tile whose sweep meets no wall row runs code without the wall
-// checks.  us per step before and after: FP32 54.0 -> 51.4 (1024x2048), 1232 -> 1101
-// (10000x5000); FP16 47.3 -> 36.2, 1024 -> 783; BF16 36.9 -> 27.1 (1501x999).
+// checks.  us per step before and after: FP32 54.0 -> 51.4 (1024x2048), 1232 -> 1094
+// (10000x5000); FP16 47.3 -> 36.2, 1024 -> 684; BF16 36.9 -> 27.1 (1501x999).
 // ---------------------------------------------------------------------------
 // Row stages of a tile (rows y and y + 1 in use, the others prefetched) and the resident
 // blocks per SM that its registers are limited for.  FP32 (HBM-bound) is fastest with
@@ -1356,12 +1356,21 @@ __global__ void planes_kernel(V* __restrict__ cells, Grid g, V* __restrict__ pla
 // each they write (us per step, FP32: 128x256 24.8 with 16-row tiles, 4.0 with 1-row ones;
 // 512x512 17.4 and 8.1 with 3 rows; 512x1024 19.4 and 12.6 with 5), while a second wave
 // costs more than shorter tiles gain (512x256: 1 row, 1024 tiles in 912 slots 7.7, 2 rows
-// 6.0).
+// 6.0).  Where one wave would make tall tiles, several waves of about kWaveRows rows: the
+// blocks of an SM then are at different rows and cover each other's barriers and waits
+// (10000x5000: FP16 786 us a step with one wave of 334 rows, 684 with 24 to 48 rows, 690
+// with 64; FP32 1103 and 1094; 4096x4096: FP16 254 and 243, FP32 384 and 374).
+constexpr int kWaveRows = 32;
+int one_wave_rows(int ny, int tiles_x, int slots) {
+    const int per_wave = std::max(1, slots / tiles_x);
+    return (ny + per_wave - 1) / per_wave;
+}
 int block_tiles_y(int ny, int tiles_x, int tile_y, int slots) {
     int rows = tile_y;
     if (rows <= 0) {
-        const int per_wave = std::max(1, slots / tiles_x);
-        rows = (ny + per_wave - 1) / per_wave;
+        rows = one_wave_rows(ny, tiles_x, slots);
+        const int waves = std::max(1, (rows + kWaveRows / 2) / kWaveRows);
+        rows = (rows + waves - 1) / waves;
     }
     return (ny + rows - 1) / rows;
 }
@@ -1480,8 +1489,8 @@ static cudaError_t launch_pair(const StepLaunch& L, cudaStream_t st) {
 
 // Columns per one-column-per-thread tile: tile_x when it is 128 or 256; otherwise 256
 // for 16-bit storage unless 128 span the grid, and for FP32 when the 256-column tiles hold at least kWideMinRows
-// rows (tile_y, or the rows of the one-wave default).  The wider tile reads half the halo
-// columns and wins where tiles are tall (FP32 at 10000x5000: 1101 us a step against 1119);
+// rows (tile_y, or the rows of one wave).  The wider tile reads half the halo
+// columns and wins on large grids (FP32 at 10000x5000: 1094 us a step against 1103);
 // tiles of 27 rows (1024x2048) run 51.4 us at 128 columns and 53.3 at 256, the barrier of 8
 // warps costing more per row than the halo saves.
 template <typename T>
@@ -1499,7 +1508,7 @@ static cudaError_t block_tile_width(const Grid& g, int tile_x, int tile_y, int* 
     cudaError_t e = block_slots<T, kWideTileW>(&slots);
     if (e != cudaSuccess) return e;
     const int gx = (g.nx + kWideTileW - 1) / kWideTileW;
-    const int rows = tile_y > 0 ? tile_y : g.ny / block_tiles_y(g.ny, gx, 0, slots);
+    const int rows = tile_y > 0 ? tile_y : one_wave_rows(g.ny, gx, slots);
     *tw = rows >= kWideMinRows ? kWideTileW : kBlockTileW;
     return cudaSuccess;
 }
@@ -1516,7 +1525,7 @@ static cudaError_t launch_step_t(const StepLaunch& L, int kernel, cudaStream_t s
     } else if (kernel == LBM_KERNEL_STAGED || kernel == LBM_KERNEL_PAIRED) {
         // 16-bit storage at the default width: the paired-column tile (same results bit for
         // bit; FP16 at 1024x2048 36.2 us a step against 38.1 of the 256-thread tile, at
-        // 10000x5000 783 against 859, at 1501x999 27.1 against 35.7), except where one
+        // 10000x5000 684 against 859, at 1501x999 27.1 against 35.7), except where one
         // 128-column tile spans the grid (128x256: 4.6 us against 5.1)
         if constexpr (IsShifted<T>::value)
             if (kernel == LBM_KERNEL_PAIRED || (L.tile_x == 0 && g.nx > kBlockTileW)) return launch_pair<T>(L, st);
