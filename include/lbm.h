@@ -479,8 +479,7 @@ void lbm_closure_destroy(lbm_closure* c);
  * the device-wide synchronisation a cudaMalloc / cudaFree can cause.  The paper
  * has no counterpart; this is an embedding interface.
  *
- * Same physics and FP32 arithmetic as lbm_step (the two-pass form: a density pass,
- * then collision and streaming).  pops_in and pops_out are device arrays of
+ * Same physics and FP32 arithmetic as lbm_step, in one kernel.  pops_in and pops_out are device arrays of
  * 2*9*ny*nx floats, [component][direction][y][x], holding post-streaming
  * populations (the layout of lbm_get_populations, in FP32); they must not overlap
  * at all (LBM_EINVAL if they do).  pops_out receives the populations one step
@@ -490,18 +489,11 @@ void lbm_closure_destroy(lbm_closure* c);
  * A CUDA error already pending when the call is made is returned as LBM_ECUDA
  * (and left pending); a launch failure is returned as LBM_ECUDA naming the kernel.
  *
- * Scratch: the densities go to a fixed device array inside the library of
- * 2 * 2^20 floats (8 MiB), held by every GPU that loads the library until the
- * process exits; grids with nx * ny > 2^20 are rejected with LBM_EINVAL.  A call
- * made outside a stream capture looks up that array's device address in the
- * current context (cudaGetSymbolAddress) and remembers it for the device; a call
- * made while cuda_stream is capturing uses the remembered address, so make one
- * call on each device before any stream capture, and again after a device reset
- * (cudaDeviceReset) or a switch to another context on that device, which
- * invalidate it (LBM_ESTATE if no address is remembered).  All calls share the
- * array: calls whose kernels overlap on the GPU (different streams, or threads)
- * race and give wrong results; serialise them.  No NaN / negative-density report:
- * use lbm_step on a handle for that. */
+ * No scratch memory is used; grids with nx * ny > 2^20 are rejected with LBM_EINVAL.
+ * The first call on a device looks up how many blocks it holds and remembers that; make
+ * it before any stream capture (LBM_ESTATE otherwise).  Calls on different arrays may
+ * overlap on the GPU.  No NaN / negative-density report: use lbm_step on a handle for
+ * that. */
 lbm_status lbm_step_noalloc(const lbm_params* p, const float* pops_in, float* pops_out, void* cuda_stream);
 
 #ifdef __cplusplus
