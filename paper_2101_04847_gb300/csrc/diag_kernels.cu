@@ -14,17 +14,20 @@
 // The moments are exact sums of the FP32 populations.  Block partials and the
 // final sums are FP64, in a fixed order, so the results are deterministic.
 //
-// Passes over a grid of 32x8-thread blocks, each covering 32 columns x 64 rows
-// (a thread takes 8 rows):
-//   D1 moments   : rho_A, rho_B, j (sum over components) per site; masses
-//   D2 velocity  : physical velocity u = (j + F/2) / rho; E_k, E_p, buoyancy,
-//                  row sums of phi and of the mass fraction, crossing counts
-//   D3 tensors   : P^K, K^(tau), grad u + grad u^T per site; <u.grad p_b>, omega^2
-//   D4 divergence: <u . div P^K>, <u . div K^(tau)>, <u . div(grad u + grad u^T)>
-//   D5 reduce    : per-term and per-row sums of the block partials
-// Scratch (8-byte units per site): M[4] (rho_A, rho_B, jx, jy), U[2] (ux, uy),
-// T[9] (Pxx Pxy Pyy Kxx Kxy Kyy Sxx Sxy Syy), all dfl; the field extraction
-// reuses T[0..3] for rho_A, rho_B, ux, uy as doubles.
+// Two values are worked on at once, as the lanes of the packed FP32 instructions
+// (dfl2): the two components, the two axes, or the two stresses.
+//
+// The diagnostics are one sweep over the populations (diag_sweep_kernel) and a reduction
+// of its block partials.  The terms <u . div T> of the stresses T are taken by parts: with
+// centred differences D, sum_y u(y) (D T)(y) over the averaged rows equals
+// -sum_y T(y) (D u~)(y), u~ being u on those rows and 0 elsewhere (x is periodic), exactly.
+// T is then needed at its own site only, contracted with velocity gradients, and no
+// intermediate field is stored.
+//
+// The fields (densities and velocity of every site) take two passes of 32x8-thread
+// blocks, each covering 32 columns x 64 rows (a thread takes 8 rows): moments_kernel
+// and velocity_kernel.  Scratch (8-byte units per site): M[4] (rho_A, rho_B, jx, jy) as
+// dfl, then the results at diag_fields_offset as doubles.
 #include "lattice.cuh"
 
 #include <algorithm>
@@ -91,51 +94,18 @@ struct DiagArgs {
     int r0, r1;         // averaged rows [r0, r1)
     // physics constants as dfl: G, body force, wall forces (G_wall / 6), external accelerations
     dfl G, gx, gw6[2], gext[2];
-    dfl cs2, w1, w2, kappa, G4, cK, floor_prod;
-    dfl* M;             // [4][ny][nx]: rho_A, rho_B, jx, jy
-    dfl* U;             // [2][ny][nx]: ux, uy
-    dfl* T;             // [9][ny][nx]
-    double* F;          // [4][ny][nx] doubles (field extraction; aliases T)
+    dfl cs2, w1, w2, kappa, Gcs2, cK, floor_prod;
+    dfl* M;             // [4][ny][nx]: rho_A, rho_B, jx, jy (fields)
+    double* F;          // [4][ny][nx] doubles (fields)
     double* partials;   // [kDiagTerms][nblocks]
     double* rowpart;    // [ny][nbx]: row partials of phi
     double* rowpart_c;  // [ny][nbx]: row partials of the mass fraction rho_A / (rho_A + rho_B)
-    int nblocks, nbx;   // blocks in total / along x
+    int nblocks, nbx;   // blocks of the sweep in total / along x
     int mirror;         // 1: the pseudopotential beyond a wall is the wall row's (wall_mode 1)
 };
 
 __device__ __forceinline__ int row_of(int r) { return blockIdx.y * BY + threadIdx.y + r * DY; }
 
-__device__ __forceinline__ dfl warp_sum(dfl v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const dfl w = {__shfl_down_sync(0xffffffffu, v.hi, o), __shfl_down_sync(0xffffffffu, v.lo, o)};
-        v = v + w;
-    }
-    return v;
-}
-
-// Block sums of N per-thread values into partials[(term0 + k) * nblocks + block].
-template <int N>
-__device__ __forceinline__ void block_sums(const dfl (&v)[N], const DiagArgs& a, int term0) {
-    __shared__ double sm[N][DY];
-    const int lane = threadIdx.x, warp = threadIdx.y;
-#pragma unroll
-    for (int k = 0; k < N; ++k) {
-        const dfl s = warp_sum(v[k]);
-        if (lane == 0) sm[k][warp] = to_d(s);
-    }
-    __syncthreads();
-    if (warp == 0 && lane < N) {
-        double s = 0.0;
-#pragma unroll
-        for (int w = 0; w < DY; ++w) s += sm[lane][w];
-        a.partials[(size_t)(term0 + lane) * a.nblocks + blockIdx.y * gridDim.x + blockIdx.x] = s;
-    }
-}
-
-__device__ __forceinline__ dfl at(const dfl* f, const DiagArgs& a, int x, int y) {
-    return f[(size_t)y * a.nx + x];
-}
 // a density field's value as the Shan-Chen force sees it: beyond a wall 0, or with
 // the mirror the wall row's own value
 __device__ __forceinline__ dfl at0(const dfl* f, const DiagArgs& a, int x, int y) {
@@ -162,7 +132,6 @@ template <typename T>
 __global__ void __launch_bounds__(DX * DY) moments_kernel(const Cell<T>* __restrict__ fin, DiagArgs a,
                                                          float sA, float sB) {
     const int x = blockIdx.x * DX + threadIdx.x;
-    dfl v[2] = {{0.0f, 0.0f}, {0.0f, 0.0f}};
 #pragma unroll 1
     for (int r = 0; r < RY; ++r) {
         const int y = row_of(r);
@@ -191,10 +160,7 @@ __global__ void __launch_bounds__(DX * DY) moments_kernel(const Cell<T>* __restr
         a.M[a.n + k] = rho[1];
         a.M[2 * a.n + k] = jx[0] + jx[1];
         a.M[3 * a.n + k] = jy[0] + jy[1];
-        v[0] = v[0] + rho[0];
-        v[1] = v[1] + rho[1];
     }
-    block_sums<2>(v, a, T_MASS_A);
 }
 
 // sum_i w_i psi(x + c_i) c_i of a density field (the virtual wall rows as at0 gives them)
@@ -210,198 +176,389 @@ __device__ __forceinline__ void nbr_sum_d(const dfl* f, const DiagArgs& a, int x
     sy = (N - S) * a.w1 + (d + (NW - SE)) * a.w2;
 }
 
-// accumulate = 0: fields only (rho_A, rho_B, ux, uy as doubles into F)
-__global__ void __launch_bounds__(DX * DY) velocity_kernel(DiagArgs a, int lo, int hi, int accumulate) {
+// rho_A, rho_B and the physical velocity of every site as doubles into F
+__global__ void __launch_bounds__(DX * DY) velocity_kernel(DiagArgs a) {
     const int x = blockIdx.x * DX + threadIdx.x;
-    dfl v[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) v[q] = {0.0f, 0.0f};
 #pragma unroll 1
     for (int r = 0; r < RY; ++r) {
         const int y = row_of(r);
-        const bool valid = x < a.nx && y >= lo && y < hi && y < a.ny;
-        const bool avg = valid && y >= a.r0 && y < a.r1;
-        dfl phi = {0.0f, 0.0f}, cA = {0.0f, 0.0f};
-        if (valid) {
-            const size_t k = (size_t)y * a.nx + x;
-            const dfl rA = a.M[k], rB = a.M[a.n + k], jx = a.M[2 * a.n + k], jy = a.M[3 * a.n + k];
-            dfl nAx, nAy, nBx, nBy;
-            nbr_sum_d(a.M, a, x, y, nAx, nAy);
-            nbr_sum_d(a.M + a.n, a, x, y, nBx, nBy);
-            // wall force: sum_i w_i S(x + c_i) c_i = (0, -1/6) on row 0, (0, 1/6) on row ny-1
-            dfl wA = {0.0f, 0.0f}, wB = {0.0f, 0.0f};
-            if (y == 0) { wA = wA + a.gw6[0]; wB = wB + a.gw6[1]; }
-            if (y == a.ny - 1) { wA = wA - a.gw6[0]; wB = wB - a.gw6[1]; }
-            const dfl aAx = a.gx - a.G * nBx, aAy = (wA + a.gext[0]) - a.G * nBy;
-            const dfl aBx = a.gx - a.G * nAx, aBy = (wB + a.gext[1]) - a.G * nAy;
-            const dfl Fx = rA * aAx + rB * aBx, Fy = rA * aAy + rB * aBy;
-            const dfl rho = rA + rB;
-            const dfl ux = dfl_div(jx + Fx * 0.5f, rho), uy = dfl_div(jy + Fy * 0.5f, rho);
-            a.U[k] = ux;
-            a.U[a.n + k] = uy;
-            if (!accumulate) {
-                a.F[k] = to_d(rA);
-                a.F[a.n + k] = to_d(rB);
-                a.F[2 * a.n + k] = to_d(ux);
-                a.F[3 * a.n + k] = to_d(uy);
-            }
-            phi = rA - rB;
-            if (rho.hi > 0.0f) cA = dfl_div(rA, rho);
-            if (avg) {
-                v[0] = v[0] + rho * (ux * ux + uy * uy) * 0.5f;
-                v[1] = v[1] + phi * (float)y;
-                v[2] = v[2] + uy * phi;
-                v[3] = v[3] + rho;
-                // crossing counts of (phi > 0) for pairs starting at (x, y); the sign
-                // of hi is the sign of the exact difference
-                const int xm = x == 0 ? a.nx - 1 : x - 1;
-                const int xp = x == a.nx - 1 ? 0 : x + 1;
-                auto positive = [&](size_t kk) { return (a.M[kk] - a.M[a.n + kk]).hi > 0.0f; };
-                const bool b = phi.hi > 0.0f;
-                if (b != positive((size_t)y * a.nx + xp)) v[4].hi += 1.0f;
-                if (y + 1 < a.r1) {
-                    const size_t up = (size_t)(y + 1) * a.nx;
-                    if (b != positive(up + x)) v[5].hi += 1.0f;
-                    if (b != positive(up + xp)) v[6].hi += 1.0f;
-                    if (b != positive(up + xm)) v[7].hi += 1.0f;
-                }
-            }
-        }
-        if (accumulate) {   // uniform over the launch
-            // row partial of phi: one warp is one row of 32 columns
-            const dfl rs = warp_sum(avg ? phi : dfl{0.0f, 0.0f});
-            const dfl rc = warp_sum(avg ? cA : dfl{0.0f, 0.0f});
-            if (threadIdx.x == 0 && y < a.ny && y >= a.r0 && y < a.r1) {
-                a.rowpart[(size_t)y * a.nbx + blockIdx.x] = to_d(rs);
-                a.rowpart_c[(size_t)y * a.nbx + blockIdx.x] = to_d(rc);
-            }
-        }
-    }
-    if (!accumulate) return;
-    const dfl e[4] = {v[0], v[1], v[2], v[3]};
-    block_sums<4>(e, a, T_EK);
-    __syncthreads();
-    const dfl c[4] = {v[4], v[5], v[6], v[7]};
-    block_sums<4>(c, a, T_N0);
-}
-
-__global__ void __launch_bounds__(DX * DY) tensor_kernel(DiagArgs a) {
-    const int x = blockIdx.x * DX + threadIdx.x;
-    dfl v[2] = {{0.0f, 0.0f}, {0.0f, 0.0f}};
-#pragma unroll 1
-    for (int r = 0; r < RY; ++r) {
-        const int y = row_of(r);
-        const bool valid = x < a.nx && y >= a.r0 - 1 && y < a.r1 + 1;
-        const bool avg = valid && y >= a.r0 && y < a.r1;
-        if (!valid) continue;
-        const int xm = x == 0 ? a.nx - 1 : x - 1;
-        const int xp = x == a.nx - 1 ? 0 : x + 1;
-        const dfl* A = a.M;
-        const dfl* B = a.M + a.n;
-        const dfl rA = at(A, a, x, y), rB = at(B, a, x, y);
-        const dfl rAE = at(A, a, xp, y), rAW = at(A, a, xm, y), rAN = at(A, a, x, y + 1), rAS = at(A, a, x, y - 1);
-        const dfl rBE = at(B, a, xp, y), rBW = at(B, a, xm, y), rBN = at(B, a, x, y + 1), rBS = at(B, a, x, y - 1);
-        const dfl phi = rA - rB;
-        const dfl phE = rAE - rBE, phW = rAW - rBW, phN = rAN - rBN, phS = rAS - rBS;
-        // Korteweg stress (Section 2, Eq. "Korteweg stress tensor")
-        const dfl px = (phE - phW) * 0.5f, py = (phN - phS) * 0.5f;
-        const dfl lap = ((phE + phW) + (phN + phS)) - phi * 4.0f;
-        const dfl iso = -(a.kappa * phi * lap) - (a.kappa * (px * px + py * py)) * 0.5f;
-        // tau-dependent stress (Section 2, Eq. "Spurious contribution")
-        const dfl dAx = (rAE - rAW) * 0.5f, dAy = (rAN - rAS) * 0.5f;
-        const dfl dBx = (rBE - rBW) * 0.5f, dBy = (rBN - rBS) * 0.5f;
-        const dfl vx = rB * dAx - rA * dBx, vy = rB * dAy - rA * dBy;
-        dfl prod = rA * rB;
-        if (prod.hi < a.floor_prod.hi || (prod.hi == a.floor_prod.hi && prod.lo < a.floor_prod.lo)) prod = a.floor_prod;
-        const dfl coef = dfl_div(a.cK, prod * (rA + rB));
-        // velocity gradient (symmetrised)
-        const dfl* UX = a.U;
-        const dfl* UY = a.U + a.n;
-        const dfl uxE = at(UX, a, xp, y), uxW = at(UX, a, xm, y), uxN = at(UX, a, x, y + 1), uxS = at(UX, a, x, y - 1);
-        const dfl uyE = at(UY, a, xp, y), uyW = at(UY, a, xm, y), uyN = at(UY, a, x, y + 1), uyS = at(UY, a, x, y - 1);
-        const dfl dxux = (uxE - uxW) * 0.5f, dyux = (uxN - uxS) * 0.5f;
-        const dfl dxuy = (uyE - uyW) * 0.5f, dyuy = (uyN - uyS) * 0.5f;
+        if (x >= a.nx || y >= a.ny) break;
         const size_t k = (size_t)y * a.nx + x;
-        const size_t n = a.n;
-        const dfl kpx = a.kappa * px;
-        a.T[k] = iso + kpx * px;
-        a.T[n + k] = kpx * py;
-        a.T[2 * n + k] = iso + a.kappa * py * py;
-        const dfl cvx = coef * vx;
-        a.T[3 * n + k] = cvx * vx;
-        a.T[4 * n + k] = cvx * vy;
-        a.T[5 * n + k] = coef * vy * vy;
-        a.T[6 * n + k] = dxux * 2.0f;
-        a.T[7 * n + k] = dxuy + dyux;
-        a.T[8 * n + k] = dyuy * 2.0f;
-        if (avg) {
-            // bulk pressure p_b = cs2 (rho_A + rho_B) + G cs2 / 4 ((rho_A + rho_B)^2 - phi^2)
-            auto pb = [&](dfl sA, dfl sB, dfl ph) {
-                const dfl sum = sA + sB;
-                return a.cs2 * sum + a.G4 * (sum * sum - ph * ph);
-            };
-            const dfl pE = pb(rAE, rBE, phE), pW = pb(rAW, rBW, phW);
-            const dfl pN = pb(rAN, rBN, phN), pS = pb(rAS, rBS, phS);
-            const dfl ux = at(UX, a, x, y), uy = at(UY, a, x, y);
-            v[0] = v[0] + (ux * (pE - pW) + uy * (pN - pS)) * 0.5f;
-            const dfl om = dxuy - dyux;
-            v[1] = v[1] + om * om;
+        const dfl rA = a.M[k], rB = a.M[a.n + k], jx = a.M[2 * a.n + k], jy = a.M[3 * a.n + k];
+        dfl nAx, nAy, nBx, nBy;
+        nbr_sum_d(a.M, a, x, y, nAx, nAy);
+        nbr_sum_d(a.M + a.n, a, x, y, nBx, nBy);
+        // wall force: sum_i w_i S(x + c_i) c_i = (0, -1/6) on row 0, (0, 1/6) on row ny-1
+        dfl wA = {0.0f, 0.0f}, wB = {0.0f, 0.0f};
+        if (y == 0) { wA = wA + a.gw6[0]; wB = wB + a.gw6[1]; }
+        if (y == a.ny - 1) { wA = wA - a.gw6[0]; wB = wB - a.gw6[1]; }
+        const dfl aAx = a.gx - a.G * nBx, aAy = (wA + a.gext[0]) - a.G * nBy;
+        const dfl aBx = a.gx - a.G * nAx, aBy = (wB + a.gext[1]) - a.G * nAy;
+        const dfl Fx = rA * aAx + rB * aBx, Fy = rA * aAy + rB * aBy;
+        const dfl rho = rA + rB;
+        const dfl ux = dfl_div(jx + Fx * 0.5f, rho), uy = dfl_div(jy + Fy * 0.5f, rho);
+        a.F[k] = to_d(rA);
+        a.F[a.n + k] = to_d(rB);
+        a.F[2 * a.n + k] = to_d(ux);
+        a.F[3 * a.n + k] = to_d(uy);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// two dfl values as the lanes of packed FP32 operations
+// ---------------------------------------------------------------------------
+struct dfl2 { float2 hi, lo; };
+
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ dfl2 two_sum2(float2 a, float2 b) {
+    const float2 s = add2(a, b);
+    const float2 bb = sub2(s, a);
+    return {s, add2(sub2(a, sub2(s, bb)), sub2(b, bb))};
+}
+__device__ __forceinline__ dfl2 two_diff2(float2 a, float2 b) {
+    const float2 s = sub2(a, b);
+    const float2 bb = sub2(s, a);
+    return {s, sub2(sub2(a, sub2(s, bb)), add2(b, bb))};
+}
+__device__ __forceinline__ dfl2 fast_two_sum2(float2 a, float2 b) {
+    const float2 s = add2(a, b);
+    return {s, sub2(b, sub2(s, a))};
+}
+// Sums to within 2^-47 of |a| + |b|, the error that the operands' own low parts carry.
+__device__ __forceinline__ dfl2 operator+(dfl2 a, dfl2 b) {
+    const dfl2 s = two_sum2(a.hi, b.hi);
+    return fast_two_sum2(s.hi, add2(s.lo, add2(a.lo, b.lo)));
+}
+__device__ __forceinline__ dfl2 operator-(dfl2 a, dfl2 b) {
+    const dfl2 s = two_diff2(a.hi, b.hi);
+    return fast_two_sum2(s.hi, add2(s.lo, sub2(a.lo, b.lo)));
+}
+__device__ __forceinline__ dfl2 operator*(dfl2 a, dfl2 b) {
+    const float2 p = mul2(a.hi, b.hi);
+    float2 e = fma2(a.hi, b.hi, neg2(p));
+    e = fma2(a.hi, b.lo, fma2(a.lo, b.hi, e));
+    return fast_two_sum2(p, e);
+}
+__device__ __forceinline__ dfl2 times(dfl2 a, float2 b) {
+    const float2 p = mul2(a.hi, b);
+    return fast_two_sum2(p, fma2(a.lo, b, fma2(a.hi, b, neg2(p))));
+}
+__device__ __forceinline__ dfl2 scaled(dfl2 a, float b) { return {mul2(a.hi, splat(b)), mul2(a.lo, splat(b))}; }   // b a power of two
+__device__ __forceinline__ dfl2 both(dfl a) { return {splat(a.hi), splat(a.lo)}; }
+__device__ __forceinline__ dfl2 pair(dfl a, dfl b) { return {make_float2(a.hi, b.hi), make_float2(a.lo, b.lo)}; }
+__device__ __forceinline__ dfl first(dfl2 a) { return {a.hi.x, a.lo.x}; }
+__device__ __forceinline__ dfl second(dfl2 a) { return {a.hi.y, a.lo.y}; }
+__device__ __forceinline__ dfl2 swapped(dfl2 a) { return {swap2(a.hi), swap2(a.lo)}; }
+// the lanes' first values of a and b, and their second values: a transpose
+__device__ __forceinline__ dfl2 firsts(dfl2 a, dfl2 b) { return pair(first(a), first(b)); }
+__device__ __forceinline__ dfl2 seconds(dfl2 a, dfl2 b) { return pair(second(a), second(b)); }
+// a / b by one correction step of the FP32 quotient a * inv, inv = 1 / b.hi
+__device__ __forceinline__ dfl2 quotient(dfl2 a, dfl2 b, float2 inv) {
+    const float2 q = mul2(a.hi, inv);
+    const dfl2 r = a - times(b, q);
+    return fast_two_sum2(q, mul2(r.hi, inv));
+}
+// Exact sums of dfl terms, as Acc: the TwoSum errors and the terms' low parts in lo.
+struct Acc2 {
+    float2 hi = {0.0f, 0.0f}, lo = {0.0f, 0.0f};
+    __device__ __forceinline__ void add(float2 v) {
+        const dfl2 s = two_sum2(hi, v);
+        hi = s.hi;
+        lo = add2(lo, s.lo);
+    }
+    __device__ __forceinline__ void add(dfl2 v) {
+        add(v.hi);
+        lo = add2(lo, v.lo);
+    }
+    __device__ __forceinline__ dfl2 value() const { return fast_two_sum2(hi, lo); }
+};
+
+// ---------------------------------------------------------------------------
+// The diagnostics sweep.  A block of kSweepT threads owns kSweepCols columns and the
+// by-th of gridDim.y tiles of rows, swept bottom up; thread t handles column
+// x0 + t - 2, the two outermost on each side only for their neighbours.  Each iteration
+// takes the moments of row m (from the stored populations), the velocity of row m - 1 and
+// the terms of row m - 2; densities and velocities are exchanged through rings in shared
+// memory.  Row sums of phi and the mass fraction are taken kRowBatch rows at a time, 16
+// threads to a row.
+//
+// Bound by issue: about 1.7 k mostly packed FP32 instructions per site against 72 bytes
+// read.  The four passes it replaces stored 15 dfl per site, read them again with their
+// neighbours and worked one value at a time: 389 us at 1024x2048 and 19 for the reduction, 188 and 5 now. Errors against 64 bits stay
+// at 1e-15 to 5e-15 of the terms.
+// ---------------------------------------------------------------------------
+constexpr int kSweepT = 128, kSweepCols = kSweepT - 4;
+constexpr int kRowBatch = 8;
+
+struct SweepShared {
+    float4 rho[8][kSweepT];            // (A.hi, B.hi, A.lo, B.lo) of row r in slot r & 7
+    float4 u[4][kSweepT];              // (ux.hi, uy.hi, ux.lo, uy.lo) of row r in slot r & 3
+    float4 rows[kRowBatch][kSweepT];   // (phi.hi, c.hi, phi.lo, c.lo) of the batch's rows
+    double sums[kDiagTerms][kSweepT / 32];
+};
+__device__ __forceinline__ dfl2 dfl2_of(float4 v) { return {make_float2(v.x, v.y), make_float2(v.z, v.w)}; }
+__device__ __forceinline__ float4 float4_of(dfl2 v) { return make_float4(v.hi.x, v.hi.y, v.lo.x, v.lo.y); }
+// sign of rho_A - rho_B, exact for normalised values
+__device__ __forceinline__ bool phi_positive(float4 r) { return r.x > r.y || (r.x == r.y && r.z > r.w); }
+
+template <typename T>
+__global__ void __launch_bounds__(kSweepT, 4)
+diag_sweep_kernel(const Cell<T>* __restrict__ fin, DiagArgs a, float2 shift) {
+    __shared__ SweepShared sm;
+    const int t = threadIdx.x;
+    const int x = blockIdx.x * kSweepCols + t - 2;
+    const int xw = (x + a.nx) % a.nx;   // periodic; columns past nx + 1 only feed threads that own none
+    const bool own = t >= 2 && t < kSweepT - 2 && x < a.nx;
+    const int ty0 = (int)(((long long)blockIdx.y * a.ny) / gridDim.y);
+    const int ty1 = (int)(((long long)(blockIdx.y + 1) * a.ny) / gridDim.y);
+    const int r0 = a.r0, r1 = a.r1;
+
+    Acc2 mass, ek_visc, om_by, ep_rho, fk_ft, iso_pb;
+    int n0 = 0, n90 = 0, n45 = 0, n135 = 0;
+    const dfl2 zero = {splat(0.0f), splat(0.0f)};
+    dfl2 j = zero;   // momentum of the row whose velocity is next
+    Cell<T> c[9];    // row m's cells, loaded one iteration ahead
+    auto load = [&](int m) {
+        if (m < 0 || m >= a.ny) return;
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            const int sy = m - cy(i);
+            const bool inside = sy >= 0 && sy < a.ny;
+            c[i] = __ldg(fin + (inside ? (size_t)i * a.g.plane + (size_t)sy * a.g.pitch + a.g.origin + (xw - cx(i))
+                                       : (size_t)opp(i) * a.g.plane + (size_t)m * a.g.pitch + a.g.origin + xw));
         }
-    }
-    block_sums<2>(v, a, T_FLUX_PB);
-}
-
-__device__ __forceinline__ void div_at(const dfl* Txx, const dfl* Txy, const dfl* Tyy, const DiagArgs& a,
-                                       int x, int y, int xm, int xp, dfl& dx, dfl& dy) {
-    dx = ((at(Txx, a, xp, y) - at(Txx, a, xm, y)) + (at(Txy, a, x, y + 1) - at(Txy, a, x, y - 1))) * 0.5f;
-    dy = ((at(Txy, a, xp, y) - at(Txy, a, xm, y)) + (at(Tyy, a, x, y + 1) - at(Tyy, a, x, y - 1))) * 0.5f;
-}
-
-__global__ void __launch_bounds__(DX * DY) divergence_kernel(DiagArgs a) {
-    const int x = blockIdx.x * DX + threadIdx.x;
-    dfl v[3] = {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}};
+    };
+    load(ty0 - 2);
+    int batched = 0;   // rows in sm.rows, the last of them row `last`
+    auto flush_rows = [&](int last) {
+        __syncthreads();
+        const int r = t >> 4, l = t & 15;
+        if (r < batched) {   // whole groups of 16 lanes
+            dfl2 v = dfl2_of(sm.rows[r][l]);
 #pragma unroll 1
-    for (int r = 0; r < RY; ++r) {
-        const int y = row_of(r);
-        if (x >= a.nx || y < a.r0 || y >= a.r1) continue;
-        const int xm = x == 0 ? a.nx - 1 : x - 1;
-        const int xp = x == a.nx - 1 ? 0 : x + 1;
-        const size_t n = a.n;
-        const dfl ux = at(a.U, a, x, y), uy = at(a.U + n, a, x, y);
-        dfl dx, dy;
-        div_at(a.T, a.T + n, a.T + 2 * n, a, x, y, xm, xp, dx, dy);
-        v[0] = v[0] + (ux * dx + uy * dy);
-        div_at(a.T + 3 * n, a.T + 4 * n, a.T + 5 * n, a, x, y, xm, xp, dx, dy);
-        v[1] = v[1] + (ux * dx + uy * dy);
-        div_at(a.T + 6 * n, a.T + 7 * n, a.T + 8 * n, a, x, y, xm, xp, dx, dy);
-        v[2] = v[2] + (ux * dx + uy * dy);
+            for (int k = 1; k < kSweepT / 16; ++k) v = v + dfl2_of(sm.rows[r][l + 16 * k]);
+            const unsigned mask = (t & 16) ? 0xffff0000u : 0x0000ffffu;
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) {
+                const dfl2 w = {make_float2(__shfl_down_sync(mask, v.hi.x, o, 16), __shfl_down_sync(mask, v.hi.y, o, 16)),
+                                make_float2(__shfl_down_sync(mask, v.lo.x, o, 16), __shfl_down_sync(mask, v.lo.y, o, 16))};
+                v = v + w;
+            }
+            if (l == 0) {
+                const size_t k = (size_t)(last - batched + 1 + r) * a.nbx + blockIdx.x;
+                a.rowpart[k] = to_d(first(v));
+                a.rowpart_c[k] = to_d(second(v));
+            }
+        }
+        batched = 0;
+        __syncthreads();
+    };
+
+#pragma unroll 1
+    for (int m = ty0 - 2; m < ty1 + 2; ++m) {
+        // --- moments of row m
+        const dfl2 jm = j;   // momentum of row m - 1
+        if (m >= 0 && m < a.ny) {
+            float2 f[9];
+#pragma unroll
+            for (int i = 0; i < 9; ++i) f[i] = cell_pops<T>(c[i], i, shift);
+            load(m + 1);
+            Acc2 r, qx, qy;
+            r.hi = f[0];
+            qx.hi = f[1];
+            qy.hi = f[2];
+#pragma unroll
+            for (int i = 1; i < 9; ++i) r.add(f[i]);
+            qx.add(neg2(f[3])); qx.add(f[5]); qx.add(neg2(f[7])); qx.add(f[8]); qx.add(neg2(f[6]));
+            qy.add(neg2(f[4])); qy.add(f[5]); qy.add(neg2(f[7])); qy.add(f[6]); qy.add(neg2(f[8]));
+            const dfl2 rho = r.value(), jx = qx.value(), jy = qy.value();
+            sm.rho[m & 7][t] = float4_of(rho);
+            j = firsts(jx, jy) + seconds(jx, jy);
+            if (own && m >= ty0 && m < ty1) mass.add(rho);
+        } else {
+            load(m + 1);
+        }
+        __syncthreads();
+        // --- velocity of row m - 1 (interior rows only: crop >= 3)
+        const int yu = m - 1;
+        if (yu >= r0 - 2 && yu < r1 + 2 && yu > ty0 - 2 && t >= 1 && t < kSweepT - 1) {
+            const float4 *rS = &sm.rho[(yu - 1) & 7][t], *rC = &sm.rho[yu & 7][t], *rN = &sm.rho[(yu + 1) & 7][t];
+            const dfl2 d = dfl2_of(rN[1]) - dfl2_of(rS[-1]), e = dfl2_of(rS[1]) - dfl2_of(rN[-1]);
+            const dfl2 ew = dfl2_of(rC[1]) - dfl2_of(rC[-1]), ns = dfl2_of(rN[0]) - dfl2_of(rS[0]);
+            // sum_i w_i psi(x + c_i) c_i of both components: (4 (E - W) + (NE - SW) + (SE - NW)) / 36, ...
+            const dfl2 w2 = both(a.w2);
+            const dfl2 sx = (scaled(ew, 4.0f) + (d + e)) * w2, sy = (scaled(ns, 4.0f) + (d - e)) * w2;
+            const dfl2 rc = dfl2_of(rC[0]), G = both(a.G);
+            const dfl2 ax = both(a.gx) - G * swapped(sx), ay = pair(a.gext[0], a.gext[1]) - G * swapped(sy);
+            const dfl2 Fx = rc * ax, Fy = rc * ay;
+            const dfl2 F = firsts(Fx, Fy) + seconds(Fx, Fy);
+            const dfl2 rho = rc + swapped(rc);
+            sm.u[yu & 3][t] = float4_of(quotient(jm + scaled(F, 0.5f), rho, splat(1.0f / rho.hi.x)));
+        }
+        __syncthreads();
+        // --- terms of row m - 2
+        const int y = m - 2;
+        if (y < ty0 || y < r0 - 1 || y > r1) continue;
+        const bool avg = y >= r0 && y < r1;
+        if (own) {
+            const float4 *rS = &sm.rho[(y - 1) & 7][t], *rC = &sm.rho[y & 7][t], *rN = &sm.rho[(y + 1) & 7][t];
+            const float4 *uS = &sm.u[(y - 1) & 3][t], *uC = &sm.u[y & 3][t], *uN = &sm.u[(y + 1) & 3][t];
+            const dfl2 r = dfl2_of(rC[0]);
+            // twice the density gradients of (A, B), then of phi, and the Laplacian of phi
+            const dfl2 E = dfl2_of(rC[1]), Wt = dfl2_of(rC[-1]), N = dfl2_of(rN[0]), S = dfl2_of(rS[0]);
+            const dfl2 gx = E - Wt, gy = N - S;
+            const dfl2 P = firsts(gx, gy) - seconds(gx, gy);   // 2 (px, py)
+            const dfl2 ew = E + Wt, ns = N + S;
+            const dfl2 lap2 = (ew + ns) - scaled(r, 4.0f);
+            // rho, phi
+            const dfl2 rA = both(first(r)), rB = {make_float2(r.hi.y, -r.hi.y), make_float2(r.lo.y, -r.lo.y)};
+            const dfl2 rp = rA + rB;
+            const dfl rho = first(rp), phi = second(rp);
+            // 2 v, v = rho_B grad rho_A - rho_A grad rho_B
+            const dfl2 rs = swapped(r);
+            const dfl2 cxv = rs * gx, cyv = rs * gy;
+            const dfl2 V = firsts(cxv, cyv) - seconds(cxv, cyv);
+            // twice the velocity gradients, and those of u~ (u on the averaged rows, else 0)
+            const dfl2 dxu = dfl2_of(uC[1]) - dfl2_of(uC[-1]);   // 2 (dx ux, dx uy)
+            const dfl2 dyu = dfl2_of(uN[0]) - dfl2_of(uS[0]);    // 2 (dy ux, dy uy)
+            dfl2 mx = dxu, my = dyu;
+            if (y <= r0 || y >= r1 - 1) {   // a row beside an edge of the averaged rows (uniform)
+                if (!avg) mx = zero;
+                const bool inN = y + 1 >= r0 && y + 1 < r1, inS = y - 1 >= r0 && y - 1 < r1;
+                my = (inN ? dfl2_of(uN[0]) : zero) - (inS ? dfl2_of(uS[0]) : zero);
+            }
+            // the divergence (A + D) and the shear of u~, doubled; the shear and the curl of u
+            const dfl A = first(mx), D = second(my);
+            const dfl2 trsh = pair(A, second(mx)) + pair(D, first(my));
+            const dfl2 curl = both(second(dxu)) +
+                              dfl2{make_float2(dyu.hi.x, -dyu.hi.x), make_float2(dyu.lo.x, -dyu.lo.x)};
+            const dfl2 tr = both(first(trsh)), A2 = both(A), D2 = both(D);
+            // q = X^2 A + X Y S + Y^2 D for (X, Y) = 2 grad phi and 2 v
+            const dfl2 X = firsts(P, V), Y = seconds(P, V);
+            const dfl2 q = X * (X * A2 + Y * both(second(trsh))) + Y * Y * D2;
+            // (lap phi, |2 grad phi|^2); rho_A rho_B and phi lap phi
+            const dfl2 PP = P * P;
+            const dfl2 ls = pair(first(lap2), first(PP)) +
+                            dfl2{make_float2(-lap2.hi.y, PP.hi.y), make_float2(-lap2.lo.y, PP.lo.y)};
+            const dfl2 pr = pair(first(r), phi) * pair(second(r), first(ls));
+            const dfl prod = first(pr);
+            dfl low = prod;
+            if (low.hi < a.floor_prod.hi || (low.hi == a.floor_prod.hi && low.lo < a.floor_prod.lo)) low = a.floor_prod;
+            // mass fraction and the tau stress's coefficient
+            const dfl lr = low * rho;
+            const dfl2 cq = quotient(pair(first(r), a.cK), pair(rho, lr), make_float2(1.0f / rho.hi, 1.0f / lr.hi));
+            // isotropic part of P^K over -kappa, times (A + D): kept times 2
+            const dfl ip = second(pr) + dfl{0.125f * ls.hi.y, 0.125f * ls.lo.y};
+            iso_pb.add(pair(ip * first(trsh), dfl{0.0f, 0.0f}));
+            // the other contractions with grad u~, kept times 8
+            fk_ft.add(q * pair(a.kappa, second(cq)));
+            // |u|^2; the contraction of the true gradients' normal parts with those of u~
+            const dfl2 uc = avg ? dfl2_of(uC[0]) : zero;
+            const dfl2 uu = uc * uc;
+            const dfl2 dd = pair(first(dxu), second(dyu)) * pair(A, D);
+            const dfl2 un = firsts(uu, dd) + seconds(uu, dd);
+            // rho |u|^2 and the viscous contraction, kept times 4
+            const dfl2 es = pair(rho, first(curl)) * pair(first(un), second(trsh));
+            ek_visc.add(es);
+            ek_visc.add(dfl2{make_float2(0.0f, 2.0f * un.hi.y), make_float2(0.0f, 2.0f * un.lo.y)});
+            if (avg) {
+                // u . grad p_b, p_b = cs2 rho + G cs2 rho_A rho_B, kept times 2: the difference of
+                // the products is (gA sB + gB sA) / 2 with the neighbours' differences g and sums s
+                const dfl2 mx2 = gx * swapped(ew), my2 = gy * swapped(ns);
+                const dfl2 gp = (firsts(gx, gy) + seconds(gx, gy)) * both(a.cs2) +
+                                (firsts(mx2, my2) + seconds(mx2, my2)) * scaled(both(a.Gcs2), 0.5f);
+                const dfl2 up = uc * gp;
+                iso_pb.add(dfl2{make_float2(0.0f, up.hi.x), make_float2(0.0f, up.lo.x)});
+                iso_pb.add(dfl2{make_float2(0.0f, up.hi.y), make_float2(0.0f, up.lo.y)});
+                const dfl om = second(curl);
+                om_by.add(pair(om, second(uc)) * pair(om, phi));
+                ep_rho.add(times(pair(phi, rho), make_float2((float)y, 1.0f)));
+                // crossing counts of (phi > 0) for pairs starting at (x, y)
+                const bool p = phi_positive(rC[0]);
+                n0 += p != phi_positive(rC[1]);
+                if (y + 1 < r1) {
+                    n90 += p != phi_positive(rN[0]);
+                    n45 += p != phi_positive(rN[1]);
+                    n135 += p != phi_positive(rN[-1]);
+                }
+                const dfl cA = rho.hi > 0.0f ? first(cq) : dfl{0.0f, 0.0f};
+                sm.rows[batched][t] = make_float4(phi.hi, cA.hi, phi.lo, cA.lo);
+            }
+        } else if (avg) {
+            sm.rows[batched][t] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        }
+        if (avg && (++batched == kRowBatch || y == r1 - 1 || y == ty1 - 1)) flush_rows(y);
     }
-    block_sums<3>(v, a, T_FLUX_K);
+
+    // block sums of the terms, FP64 from here on; the powers of two that the doubled
+    // gradients left, and the sign of the summation by parts, are taken off
+    const int lane = t & 31, warp = t >> 5;
+    const dfl2 iso = iso_pb.value();
+    const double kappa = to_d(a.kappa);
+    const dfl2 v[5] = {mass.value(), ek_visc.value(), om_by.value(), ep_rho.value(), fk_ft.value()};
+    const int term[10] = {T_MASS_A, T_MASS_B, T_EK, T_VISC, T_OMEGA2, T_BUOY, T_EP, T_RHO, T_FLUX_K, T_FLUX_TAU};
+    const double scale[10] = {1.0, 1.0, 0.5, -0.25, 0.25, 1.0, 1.0, 1.0, -0.125, -0.125};
+    auto warp_total = [&](double d, int k) {
+        for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xffffffffu, d, o);
+        if (lane == 0) sm.sums[k][warp] = d;
+    };
+#pragma unroll
+    for (int k = 0; k < 10; ++k) {
+        double d = scale[k] * to_d(k & 1 ? second(v[k / 2]) : first(v[k / 2]));
+        if (term[k] == T_FLUX_K) d += 0.5 * kappa * to_d(first(iso));   // the isotropic part
+        warp_total(d, term[k]);
+    }
+    warp_total(0.5 * to_d(second(iso)), T_FLUX_PB);
+    warp_total((double)n0, T_N0);
+    warp_total((double)n90, T_N90);
+    warp_total((double)n45, T_N45);
+    warp_total((double)n135, T_N135);
+    __syncthreads();
+    if (t < kDiagTerms) {
+        double d = 0.0;
+        for (int w = 0; w < kSweepT / 32; ++w) d += sm.sums[t][w];
+        a.partials[(size_t)t * a.nblocks + blockIdx.y * gridDim.x + blockIdx.x] = d;
+    }
 }
 
-// blocks [0, kDiagTerms): term sums over the block partials; the next r1 - r0 blocks:
-// row sums of phi; the last r1 - r0 blocks: row sums of the mass fraction.
+// blocks [0, kDiagTerms): term sums over the block partials; the next blocks, a warp to
+// each of the 2 (r1 - r0) rows: row sums of phi, then of the mass fraction.
 __global__ void __launch_bounds__(256) reduce_kernel(DiagArgs a, double* out) {
-    __shared__ double sm[256];
-    const int tid = threadIdx.x;
+    __shared__ double sm[8];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int nrows = a.r1 - a.r0;
+    const int k = (blockIdx.x - kDiagTerms) * 8 + warp;   // row
     double s = 0.0;
     if (blockIdx.x < kDiagTerms) {
         const double* p = a.partials + (size_t)blockIdx.x * a.nblocks;
         for (int b = tid; b < a.nblocks; b += 256) s += p[b];
-    } else {
-        const int nrows = a.r1 - a.r0;
-        const int k = blockIdx.x - kDiagTerms;
+    } else if (k < 2 * nrows) {
         const int y = a.r0 + (k < nrows ? k : k - nrows);
         const double* p = (k < nrows ? a.rowpart : a.rowpart_c) + (size_t)y * a.nbx;
-        for (int b = tid; b < a.nbx; b += 256) s += p[b];
+        for (int b = lane; b < a.nbx; b += 32) s += p[b];
     }
-    sm[tid] = s;
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (blockIdx.x >= kDiagTerms) {
+        if (lane == 0 && k < 2 * nrows) out[kDiagTerms + k] = s;
+        return;
+    }
+    if (lane == 0) sm[warp] = s;
     __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (tid < o) sm[tid] += sm[tid + o];
-        __syncthreads();
+    if (tid == 0) {
+        double v = 0.0;
+        for (int w = 0; w < 8; ++w) v += sm[w];
+        out[blockIdx.x] = v;
     }
-    if (tid == 0) out[blockIdx.x] = sm[0];
+}
+
+// Row tiles of the sweep on an nx x ny grid: about kSweepRows rows each, fewer where that
+// leaves block slots empty.
+constexpr int kSweepRows = 32, kSweepMinRows = 4, kSweepSlots = 600;
+int sweep_tiles_x(int nx) { return (nx + kSweepCols - 1) / kSweepCols; }
+int sweep_tiles_y(int nx, int ny) {
+    const int per_wave = std::max(1, kSweepSlots / sweep_tiles_x(nx));
+    const int rows = std::min(kSweepRows, std::max(kSweepMinRows, (ny + per_wave - 1) / per_wave));
+    return (ny + rows - 1) / rows;
 }
 
 DiagArgs make_args(const DiagLaunch& D) {
@@ -422,17 +579,15 @@ DiagArgs make_args(const DiagLaunch& D) {
     a.w1 = dfl_of(1.0 / 9.0);
     a.w2 = dfl_of(1.0 / 36.0);
     a.kappa = dfl_of(kCs2 * kCs2 * D.G / 4.0);
-    a.G4 = dfl_of(D.G * kCs2 / 4.0);
+    a.Gcs2 = dfl_of(D.G * kCs2);
     const double tm = D.tau_bar - 0.5;
     a.cK = dfl_of(kCs2 * kCs2 * tm * tm);
     a.floor_prod = dfl_of(1e-12);
     a.mirror = D.wall_mirror;
     a.M = reinterpret_cast<dfl*>(D.scratch);
-    a.U = reinterpret_cast<dfl*>(D.scratch + 4 * a.n);
-    a.T = reinterpret_cast<dfl*>(D.scratch + 6 * a.n);
     a.F = D.scratch + diag_fields_offset(a.nx, a.ny);
-    a.nbx = (a.nx + DX - 1) / DX;
-    a.nblocks = a.nbx * ((a.ny + BY - 1) / BY);
+    a.nbx = sweep_tiles_x(a.nx);
+    a.nblocks = a.nbx * sweep_tiles_y(a.nx, a.ny);
     a.partials = D.partials;
     a.rowpart = D.partials + (size_t)kDiagTerms * a.nblocks;
     a.rowpart_c = a.rowpart + (size_t)a.ny * a.nbx;
@@ -441,7 +596,7 @@ DiagArgs make_args(const DiagLaunch& D) {
 
 template <typename T>
 cudaError_t launch_moments(const DiagLaunch& D, const DiagArgs& a, cudaStream_t st) {
-    dim3 grid(a.nbx, (a.ny + BY - 1) / BY), block(DX, DY);
+    dim3 grid((a.nx + DX - 1) / DX, (a.ny + BY - 1) / BY), block(DX, DY);
     moments_kernel<T><<<grid, block, 0, st>>>((const Cell<T>*)D.fin, a, D.shift[0], D.shift[1]);
     return cudaGetLastError();
 }
@@ -539,24 +694,32 @@ cudaError_t launch_closure_features(const DiagLaunch& D, const float* rho2, cons
 size_t diag_scratch_doubles(int nx, int ny) { return (size_t)15 * nx * ny; }
 
 size_t diag_partials_doubles(int nx, int ny) {
-    const size_t gx = (nx + DX - 1) / DX, gy = (ny + BY - 1) / BY;
+    const size_t gx = sweep_tiles_x(nx), gy = sweep_tiles_y(nx, ny);
     return (size_t)kDiagTerms * gx * gy + (size_t)2 * ny * gx;
 }
 
 size_t diag_fields_offset(int nx, int ny) { return (size_t)6 * nx * ny; }
 
+template <typename T>
+static cudaError_t launch_sweep(const DiagLaunch& D, const DiagArgs& a, cudaStream_t st) {
+    const dim3 grid(a.nbx, a.nblocks / a.nbx);
+    diag_sweep_kernel<T><<<grid, kSweepT, 0, st>>>((const Cell<T>*)D.fin, a, make_float2(D.shift[0], D.shift[1]));
+    return cudaGetLastError();
+}
+
 cudaError_t launch_diagnostics(const DiagLaunch& D, cudaStream_t st) {
     (void)cudaGetLastError();   // a launch reports only its own error
-    DiagArgs a = make_args(D);
-    // The velocity gradient terms of D3/D4 need u two rows outside the averaged rows and
-    // u needs rho one row further out; crop >= 3 keeps all of them inside the grid.
-    cudaError_t e = moments(D, a, st);
+    const DiagArgs a = make_args(D);
+    // u is needed one row outside the rows with a stress and rho one row further out;
+    // crop >= 3 keeps all of them inside the grid
+    cudaError_t e;
+    switch (D.storage) {
+        case LBM_STORE_F16: e = launch_sweep<__half>(D, a, st); break;
+        case LBM_STORE_BF16: e = launch_sweep<__nv_bfloat16>(D, a, st); break;
+        default: e = launch_sweep<float>(D, a, st);
+    }
     if (e != cudaSuccess) return e;
-    dim3 grid(a.nbx, (a.ny + BY - 1) / BY), block(DX, DY);
-    velocity_kernel<<<grid, block, 0, st>>>(a, a.r0 - 2, a.r1 + 2, 1);
-    tensor_kernel<<<grid, block, 0, st>>>(a);
-    divergence_kernel<<<grid, block, 0, st>>>(a);
-    reduce_kernel<<<kDiagTerms + 2 * (a.r1 - a.r0), 256, 0, st>>>(a, D.out);
+    reduce_kernel<<<kDiagTerms + (2 * (a.r1 - a.r0) + 7) / 8, 256, 0, st>>>(a, D.out);
     return cudaGetLastError();
 }
 
@@ -565,8 +728,8 @@ cudaError_t launch_fields(const DiagLaunch& D, double* /*unused*/, cudaStream_t 
     DiagArgs a = make_args(D);
     cudaError_t e = moments(D, a, st);
     if (e != cudaSuccess) return e;
-    dim3 grid(a.nbx, (a.ny + BY - 1) / BY), block(DX, DY);
-    velocity_kernel<<<grid, block, 0, st>>>(a, 0, a.ny, 0);
+    dim3 grid((a.nx + DX - 1) / DX, (a.ny + BY - 1) / BY), block(DX, DY);
+    velocity_kernel<<<grid, block, 0, st>>>(a);
     return cudaGetLastError();
 }
 
