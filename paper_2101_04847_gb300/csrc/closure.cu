@@ -28,160 +28,334 @@ constexpr int kW1 = 0, kB1 = kW1 + kHid * kIn * 9;
 constexpr int kW2 = kB1 + kHid, kB2 = kW2 + kHid * kHid * 9;
 constexpr int kW3 = kB2 + kHid, kB3 = kW3 + kOut * kHid * 9;
 constexpr int kParams = kB3 + kOut;   // 11588
-constexpr int kTile = 16;
-constexpr int kChunk = 2048;          // pixels per weight-gradient block
+constexpr int kPartPixels = 512;      // pixels per weight-gradient partial, at least
 
 static_assert(kParams == 11588, "parameter count");
 
 __device__ __forceinline__ int wrapx(int x, int nx) { return x < 0 ? x + nx : (x >= nx ? x - nx : x); }
 
-// Load a (kTile+2)^2 tile of CH channels starting at channel c0 into smem
-// (periodic in x, zeros beyond the walls in y).
-template <int CH>
-__device__ __forceinline__ void load_tile(float (*s)[kTile + 2][kTile + 2], const float* __restrict__ a, int c0, int cmax,
-                                          int nx, int ny) {
-    const int tid = threadIdx.y * kTile + threadIdx.x;
-    const size_t n = (size_t)nx * ny;
-    for (int i = tid; i < CH * (kTile + 2) * (kTile + 2); i += kTile * kTile) {
-        const int c = i / ((kTile + 2) * (kTile + 2));
-        const int r = i % ((kTile + 2) * (kTile + 2));
-        const int yy = r / (kTile + 2), xx = r % (kTile + 2);
-        const int gy = blockIdx.y * kTile + yy - 1;
-        const int gx = wrapx((int)(blockIdx.x * kTile) + xx - 1, nx);
-        float v = 0.0f;
-        if (c0 + c < cmax && gy >= 0 && gy < ny && gx < nx) v = a[(size_t)(c0 + c) * n + (size_t)gy * nx + gx];
-        s[c][yy][xx] = v;
-    }
+// FP32 weights of the convolution kernels, from the BF16-rounded parameters, laid out
+// [input channel][tap][output channel] (taps row-major): the three layers, then the
+// transposed convolutions of the backward pass (taps mirrored) of layers 2 and 3.
+constexpr int kF1 = 0, kF2 = kF1 + kIn * 9 * kHid, kF3 = kF2 + kHid * 9 * kHid;
+constexpr int kT2 = kF3 + kHid * 9 * kOut, kT3 = kT2 + kHid * 9 * kHid;
+constexpr int kConvWeights = kT3 + kOut * 9 * kHid;
+
+__global__ void conv_weights_kernel(const float* __restrict__ p, float* __restrict__ w) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= kConvWeights) return;
+    int src;
+    auto forward = [&](int k, int base, int cin, int cout) {
+        const int o = k % cout, t = k / cout % 9, c = k / (cout * 9);
+        return base + (o * cin + c) * 9 + t;
+    };
+    auto mirrored = [&](int k, int base, int cin, int cout) {   // of the layer cin -> cout
+        const int c = k % cin, t = k / cin % 9, o = k / (cin * 9);
+        return base + (o * cin + c) * 9 + 8 - t;
+    };
+    if (i < kF2) src = forward(i - kF1, kW1, kIn, kHid);
+    else if (i < kF3) src = forward(i - kF2, kW2, kHid, kHid);
+    else if (i < kT2) src = forward(i - kF3, kW3, kHid, kOut);
+    else if (i < kT3) src = mirrored(i - kT2, kW2, kHid, kHid);
+    else src = mirrored(i - kT3, kW3, kHid, kOut);
+    w[i] = __bfloat162float(__float2bfloat16_rn(p[src]));
 }
 
-// out[o, y, x] = b[o] + sum_{c, dy, dx} w[o, c, dy+1, dx+1] in[c, y+dy, x+dx]  (optional ReLU)
-template <int CIN, int COUT, bool RELU>
-__global__ void __launch_bounds__(kTile * kTile)
-conv_fwd_kernel(const float* __restrict__ in, const __nv_bfloat16* __restrict__ w, const float* __restrict__ b,
-                float* __restrict__ out, int nx, int ny) {
-    constexpr int CH = CIN < 8 ? CIN : 8;
-    __shared__ float sw[COUT * CIN * 9];
-    __shared__ float st[CH][kTile + 2][kTile + 2];
-    const int tid = threadIdx.y * kTile + threadIdx.x;
-    for (int i = tid; i < COUT * CIN * 9; i += kTile * kTile) sw[i] = __bfloat162float(w[i]);
-    const int x = blockIdx.x * kTile + threadIdx.x, y = blockIdx.y * kTile + threadIdx.y;
-    float acc[COUT];
+// 3x3 convolution, x periodic, zeros beyond the walls:
+//   out[o, y, x] = b[o] + sum_{c, dy, dx} w[c][dy+1, dx+1][o] in[c, y+dy, x+dx].
+// Epi: what becomes of the sums (kMask: no bias, times act > 0).
+// A block computes a 32 x 16 pixel tile; a thread four neighbouring pixels of a row and
+// up to 16 output channels, as packed pairs of channels: per input channel 288 FFMA2
+// against 36 weight loads (16 bytes, broadcast), 6 input loads and 18 moves, so the FMA
+// pipe is what bounds it.  One pixel and all 32 channels per thread with scalar weight loads
+// took as many loads as FMAs: 506 us for the 32 -> 32 layer at 512x1024, 188 now.
+enum Epi { kBias, kBiasRelu, kMask };
+constexpr int kConvW = 32, kConvH = 16, kConvPitch = 36;   // tile; floats per staged row (34 used)
+
+template <int CIN, int COUT, Epi EPI>
+struct ConvCfg {
+    static constexpr int TO = COUT < 16 ? COUT : 16;               // output channels per thread
+    static constexpr int CH = CIN < 8 ? CIN : 8;                   // input channels staged at a time
+    static constexpr int kThreads = (kConvW / 4) * kConvH * (COUT / TO);
+};
+
+template <int CIN, int COUT, Epi EPI>
+__global__ void __launch_bounds__((ConvCfg<CIN, COUT, EPI>::kThreads), 2)
+conv_kernel(const float* __restrict__ in, const float* __restrict__ w, const float* __restrict__ b,
+            const float* __restrict__ act, float* __restrict__ out, int nx, int ny) {
+    typedef ConvCfg<CIN, COUT, EPI> K;
+    constexpr int TO = K::TO, CH = K::CH, T = K::kThreads;
+    __shared__ __align__(16) float si[CH][kConvH + 2][kConvPitch];
+    __shared__ __align__(16) float sw[CH * 9 * COUT];
+    const int tid = threadIdx.x;
+    const int tx = tid & 7, ty = (tid >> 3) & 15, half = tid >> 7;
+    const int bx = blockIdx.x * kConvW, by = blockIdx.y * kConvH;
+    const size_t n = (size_t)nx * ny;
+    float2 acc[4][TO / 2];
 #pragma unroll
-    for (int o = 0; o < COUT; ++o) acc[o] = b[o];
+    for (int o = 0; o < TO / 2; ++o) {
+        const float2 v = EPI == kMask ? splat(0.0f) : make_float2(b[half * TO + 2 * o], b[half * TO + 2 * o + 1]);
+#pragma unroll
+        for (int p = 0; p < 4; ++p) acc[p][o] = v;
+    }
+    // the staged pixels of this thread: where they lie in a plane (-1: zero) and in the tile
+    constexpr int kPixels = (kConvH + 2) * (kConvW + 2), kMine = (kPixels + T - 1) / T;
+    int64_t from[kMine];
+    int to[kMine];
+#pragma unroll
+    for (int q = 0; q < kMine; ++q) {
+        const int r = tid + q * T, yy = r / (kConvW + 2), xx = r % (kConvW + 2);
+        const int gy = by + yy - 1, gx = wrapx(bx + xx - 1, nx);
+        from[q] = gy >= 0 && gy < ny && gx < nx ? (int64_t)gy * nx + gx : -1;
+        to[q] = r < kPixels ? yy * kConvPitch + xx : -1;
+    }
+#pragma unroll 1
     for (int c0 = 0; c0 < CIN; c0 += CH) {
-        __syncthreads();
-        load_tile<CH>(st, in, c0, CIN, nx, ny);
+        float pre[CH][kMine];   // all loads in flight before the barrier
+        const float* plane = in + (size_t)c0 * n;
+#pragma unroll
+        for (int c = 0; c < CH; ++c)
+#pragma unroll
+            for (int q = 0; q < kMine; ++q)
+                pre[c][q] = from[q] >= 0 && to[q] >= 0 ? __ldg(plane + (size_t)c * n + from[q]) : 0.0f;
         __syncthreads();
 #pragma unroll
         for (int c = 0; c < CH; ++c)
 #pragma unroll
-            for (int k = 0; k < 9; ++k) {
-                const float v = st[c][threadIdx.y + k / 3][threadIdx.x + k % 3];
-#pragma unroll
-                for (int o = 0; o < COUT; ++o) acc[o] = fmaf(sw[(o * CIN + c0 + c) * 9 + k], v, acc[o]);
-            }
-    }
-    if (x < nx && y < ny) {
-        const size_t n = (size_t)nx * ny;
-#pragma unroll
-        for (int o = 0; o < COUT; ++o) out[(size_t)o * n + (size_t)y * nx + x] = RELU ? fmaxf(acc[o], 0.0f) : acc[o];
-    }
-}
-
-// din[c, y, x] = sum_{o, dy, dx} w[o, c, dy+1, dx+1] dout[o, y-dy, x-dx]; times (act[c] > 0) if MASK
-template <int CIN, int COUT, bool MASK>
-__global__ void __launch_bounds__(kTile * kTile)
-conv_bwd_data_kernel(const float* __restrict__ dout, const __nv_bfloat16* __restrict__ w, const float* __restrict__ act,
-                     float* __restrict__ din, int nx, int ny) {
-    constexpr int CH = COUT < 8 ? COUT : 8;
-    __shared__ float sw[COUT * CIN * 9];
-    __shared__ float st[CH][kTile + 2][kTile + 2];
-    const int tid = threadIdx.y * kTile + threadIdx.x;
-    for (int i = tid; i < COUT * CIN * 9; i += kTile * kTile) sw[i] = __bfloat162float(w[i]);
-    const int x = blockIdx.x * kTile + threadIdx.x, y = blockIdx.y * kTile + threadIdx.y;
-    float acc[CIN];
-#pragma unroll
-    for (int c = 0; c < CIN; ++c) acc[c] = 0.0f;
-    for (int o0 = 0; o0 < COUT; o0 += CH) {
-        __syncthreads();
-        load_tile<CH>(st, dout, o0, COUT, nx, ny);
+            for (int q = 0; q < kMine; ++q)
+                if (to[q] >= 0) (&si[c][0][0])[to[q]] = pre[c][q];
+        for (int i = tid; i < CH * 9 * COUT / 4; i += T)
+            reinterpret_cast<float4*>(sw)[i] = __ldg(reinterpret_cast<const float4*>(w + (size_t)c0 * 9 * COUT) + i);
         __syncthreads();
 #pragma unroll 1
-        for (int o = 0; o < CH; ++o)
+        for (int c = 0; c < CH; ++c) {
 #pragma unroll
-            for (int k = 0; k < 9; ++k) {
-                // dout at (y - dy, x - dx) with dy = k/3 - 1, dx = k%3 - 1
-                const float g = st[o][threadIdx.y + 2 - k / 3][threadIdx.x + 2 - k % 3];
+            for (int ky = 0; ky < 3; ++ky) {
+                const float* row = &si[c][ty + ky][4 * tx];
+                const float4 a = *reinterpret_cast<const float4*>(row);
+                const float2 e = *reinterpret_cast<const float2*>(row + 4);
+                const float2 v[6] = {splat(a.x), splat(a.y), splat(a.z), splat(a.w), splat(e.x), splat(e.y)};
 #pragma unroll
-                for (int c = 0; c < CIN; ++c) acc[c] = fmaf(sw[((o0 + o) * CIN + c) * 9 + k], g, acc[c]);
+                for (int kx = 0; kx < 3; ++kx) {
+                    const float4* wk = reinterpret_cast<const float4*>(sw + (c * 9 + ky * 3 + kx) * COUT + half * TO);
+#pragma unroll
+                    for (int q = 0; q < TO / 4; ++q) {
+                        const float4 w4 = wk[q];
+                        const float2 wa = make_float2(w4.x, w4.y), wb = make_float2(w4.z, w4.w);
+#pragma unroll
+                        for (int p = 0; p < 4; ++p) {
+                            acc[p][2 * q] = fma2(wa, v[p + kx], acc[p][2 * q]);
+                            acc[p][2 * q + 1] = fma2(wb, v[p + kx], acc[p][2 * q + 1]);
+                        }
+                    }
+                }
+            }
+        }
+    }
+    const int x = bx + 4 * tx, y = by + ty;
+    if (y >= ny) return;
+#pragma unroll
+    for (int o = 0; o < TO; ++o) {
+        const size_t k = (size_t)(half * TO + o) * n + (size_t)y * nx + x;
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+            if (x + p < nx) {
+                float v = o & 1 ? acc[p][o / 2].y : acc[p][o / 2].x;
+                if (EPI == kBiasRelu) v = fmaxf(v, 0.0f);
+                if (EPI == kMask) v = act[k + p] > 0.0f ? v : 0.0f;
+                out[k + p] = v;
             }
     }
-    if (x < nx && y < ny) {
-        const size_t n = (size_t)nx * ny;
-#pragma unroll
-        for (int c = 0; c < CIN; ++c) {
-            const size_t k = (size_t)c * n + (size_t)y * nx + x;
-            din[k] = MASK ? (act[k] > 0.0f ? acc[c] : 0.0f) : acc[c];
-        }
-    }
 }
 
-// Partial weight / bias gradients of one (o, c) pair over one chunk of pixels:
-// part[((p * COUT + o) * CIN + c) * 10 + k] (k < 9: weight tap, 9: bias when c == 0)
+template <int CIN, int COUT, Epi EPI>
+void launch_conv(const float* in, const float* w, const float* b, const float* act, float* out, int nx, int ny,
+                 cudaStream_t st) {
+    const dim3 grid((nx + kConvW - 1) / kConvW, (ny + kConvH - 1) / kConvH);
+    conv_kernel<CIN, COUT, EPI><<<grid, ConvCfg<CIN, COUT, EPI>::kThreads, 0, st>>>(in, w, b, act, out, nx, ny);
+}
+
+// Partial weight and bias gradients, part[block][COUT * CIN * 9 + COUT] in the parameters'
+// order: block b takes every gridDim.x-th tile of 32 x 4 pixels.
+//   dw[o][c][k] = sum_pixels dout[o, p] in[c, p + k],  db[o] = sum_pixels dout[o, p].
+// A thread owns 4 output channels and a pair of input channels (the lanes of the packed
+// FMAs) with all 9 taps: 72 sums in registers, 144 FFMA2 per four pixels against 13 shared
+// loads of 16 bytes.  Layers with 4 channels on one side split a row's pixels over 8
+// groups of threads.  The (o, c) pair per block it replaces read every input plane 32
+// times and loaded ten values for ten FMAs: 3460 us for the 32 -> 32 layer at 512x1024,
+// 226 now.  A partial covers at most a few hundred pixels and reduce_grad_kernel
+// adds them without rounding errors of its own: the gradient is 6e-8 off 64 bits at 512x1024,
+// 2.4e-7 before.
+constexpr int kWgThreads = 128, kWgW = 32, kWgH = 4;
+constexpr int kWgRow = kWgW + 2;                               // staged columns of a row
+template <int CIN, int COUT> struct WgCfg {
+    static constexpr int kWorkers = (COUT / 4) * (CIN / 2);    // threads that cover all (o, c, k)
+    static constexpr int kGroups = kWgThreads / kWorkers;      // pixel groups
+    // float2 per staged channel pair, 16 bytes beyond a multiple of 128 bytes apart, so that the
+    // loads of 8 neighbouring pairs meet different banks
+    static constexpr int kPlane = ((kWgH + 2) * kWgRow * 8 / 128 * 128 + 144) / 8;
+    static constexpr int kOut = COUT * CIN * 9 + COUT;
+    static constexpr size_t kStage = (size_t)(CIN / 2) * kPlane * 8 + (size_t)COUT * kWgH * kWgW * 4;
+    static constexpr size_t kReduce = kGroups > 1 ? (size_t)kWgThreads * 72 * 4 : 0;
+    static constexpr size_t kSmem = kStage > kReduce ? kStage : kReduce;
+    static_assert(kPlane * 8 % 128 == 16 && kPlane >= (kWgH + 2) * kWgRow && kGroups * kWorkers == kWgThreads, "");
+    static_assert(kGroups == 1 || kGroups == kWgW / 4, "a pixel group is one run of four columns");
+};
+
 template <int CIN, int COUT>
-__global__ void __launch_bounds__(256)
-conv_bwd_weight_kernel(const float* __restrict__ in, const float* __restrict__ dout, float* __restrict__ part, int nx,
-                       int ny) {
-    const int o = blockIdx.x / CIN, c = blockIdx.x % CIN, p = blockIdx.y;
+__global__ void __launch_bounds__(kWgThreads, 4)
+weight_grad_kernel(const float* __restrict__ in, const float* __restrict__ dout, float* __restrict__ part, int nx, int ny,
+                   int tiles_x, int tiles) {
+    typedef WgCfg<CIN, COUT> K;
+    extern __shared__ __align__(16) unsigned char wsm[];
+    float2* si = reinterpret_cast<float2*>(wsm);                                    // [CIN / 2][kPlane]
+    float* sg = reinterpret_cast<float*>(wsm + (size_t)(CIN / 2) * K::kPlane * 8);   // [COUT][kWgH][kWgW]
+    const int t = threadIdx.x;
+    const int work = t % K::kWorkers, group = t / K::kWorkers;
+    const int cp = work % (CIN / 2), oq = work / (CIN / 2);
     const size_t n = (size_t)nx * ny;
-    const size_t p0 = (size_t)p * kChunk, p1 = min(n, p0 + kChunk);
-    float s[10];
+    float2 acc[4][9];
 #pragma unroll
-    for (int k = 0; k < 10; ++k) s[k] = 0.0f;
-    const float* a = in + (size_t)c * n;
-    const float* g = dout + (size_t)o * n;
-    for (size_t q = p0 + threadIdx.x; q < p1; q += 256) {
-        const int y = (int)(q / nx), x = (int)(q % nx);
-        const float gv = g[q];
-        s[9] += gv;
+    for (int o = 0; o < 4; ++o)
 #pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            const int yy = y + k / 3 - 1;
-            const int xx = wrapx(x + k % 3 - 1, nx);
-            const float v = (yy >= 0 && yy < ny) ? a[(size_t)yy * nx + xx] : 0.0f;
-            s[k] = fmaf(gv, v, s[k]);
+        for (int k = 0; k < 9; ++k) acc[o][k] = splat(0.0f);
+    float bias = 0.0f;   // of channel t / 4, rows t % 4 of the tiles
+#pragma unroll 1
+    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        const int bx = tile % tiles_x * kWgW, by = tile / tiles_x * kWgH;
+        __syncthreads();
+        // staging: a thread's pixels are the same in every plane
+        static_assert(kWgH * kWgW == kWgThreads && (kWgH + 2) * kWgRow <= 2 * kWgThreads, "");
+        {
+            const int gy = by + t / kWgW, gx = bx + t % kWgW;
+            const bool real = gy < ny && gx < nx;
+            const float* p = dout + (size_t)gy * nx + gx;
+#pragma unroll 8
+            for (int o = 0; o < COUT; ++o) sg[o * kWgThreads + t] = real ? __ldg(p + (size_t)o * n) : 0.0f;
         }
-    }
-    __shared__ float red[8][10];
 #pragma unroll
-    for (int k = 0; k < 10; ++k) {
-        float v = s[k];
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][k] = v;
+        for (int q = 0; q < 2; ++q) {
+            const int r = t + q * kWgThreads;
+            if (r >= (kWgH + 2) * kWgRow) break;
+            const int yy = r / kWgRow, xx = r % kWgRow;
+            const int gy = by + yy - 1, gx = wrapx(bx + xx - 1, nx);
+            const bool real = gy >= 0 && gy < ny && gx < nx;
+            const float* p = in + (int64_t)gy * nx + gx;
+#pragma unroll 8
+            for (int c = 0; c < CIN / 2; ++c)
+                si[c * K::kPlane + r] = real ? make_float2(__ldg(p + (size_t)(2 * c) * n), __ldg(p + (size_t)(2 * c + 1) * n))
+                                             : splat(0.0f);
+        }
+        __syncthreads();
+        if (t < COUT * kWgH) {
+            const float4* g = reinterpret_cast<const float4*>(sg + t * kWgW);
+            float s = 0.0f;
+#pragma unroll
+            for (int q = 0; q < kWgW / 4; ++q) s += (g[q].x + g[q].y) + (g[q].z + g[q].w);
+            bias += s;
+        }
+#pragma unroll 1
+        for (int r = 0; r < kWgH; ++r)
+#pragma unroll 1
+            for (int q = group; q < kWgW / 4; q += K::kGroups) {
+                float4 g[4];
+#pragma unroll
+                for (int o = 0; o < 4; ++o) g[o] = *reinterpret_cast<const float4*>(sg + ((4 * oq + o) * kWgH + r) * kWgW + 4 * q);
+#pragma unroll
+                for (int ky = 0; ky < 3; ++ky) {
+                    const float4* p = reinterpret_cast<const float4*>(si + cp * K::kPlane + (r + ky) * kWgRow + 4 * q);
+                    const float4 a = p[0], b = p[1], c = p[2];
+                    const float2 v[6] = {make_float2(a.x, a.y), make_float2(a.z, a.w), make_float2(b.x, b.y),
+                                         make_float2(b.z, b.w), make_float2(c.x, c.y), make_float2(c.z, c.w)};
+#pragma unroll
+                    for (int o = 0; o < 4; ++o) {
+                        const float go[4] = {g[o].x, g[o].y, g[o].z, g[o].w};
+#pragma unroll
+                        for (int px = 0; px < 4; ++px)
+#pragma unroll
+                            for (int kx = 0; kx < 3; ++kx)
+                                acc[o][3 * ky + kx] = fma2(splat(go[px]), v[px + kx], acc[o][3 * ky + kx]);
+                    }
+                }
+            }
     }
-    __syncthreads();
-    if (threadIdx.x < 10) {
-        float v = 0.0f;
-        for (int wdx = 0; wdx < 8; ++wdx) v += red[wdx][threadIdx.x];
-        part[(((size_t)p * COUT + o) * CIN + c) * 10 + threadIdx.x] = v;
+    float* out = part + (size_t)blockIdx.x * K::kOut;
+    if (t < COUT * kWgH) {   // whole groups of four lanes
+        const unsigned mask = __activemask();
+        bias += __shfl_down_sync(mask, bias, 2, 4);
+        bias += __shfl_down_sync(mask, bias, 1, 4);
+        if (t % 4 == 0) out[COUT * CIN * 9 + t / 4] = bias;
+    }
+    if constexpr (K::kGroups == 1) {
+#pragma unroll
+        for (int o = 0; o < 4; ++o)
+#pragma unroll
+            for (int k = 0; k < 9; ++k) {
+                out[((4 * oq + o) * CIN + 2 * cp) * 9 + k] = acc[o][k].x;
+                out[((4 * oq + o) * CIN + 2 * cp + 1) * 9 + k] = acc[o][k].y;
+            }
+    } else {   // the groups' sums added in order
+        float* red = reinterpret_cast<float*>(wsm);   // [72][kWgThreads]
+        __syncthreads();
+#pragma unroll
+        for (int o = 0; o < 4; ++o)
+#pragma unroll
+            for (int k = 0; k < 9; ++k) {
+                red[(o * 18 + 2 * k) * kWgThreads + t] = acc[o][k].x;
+                red[(o * 18 + 2 * k + 1) * kWgThreads + t] = acc[o][k].y;
+            }
+        __syncthreads();
+        for (int i = t; i < 72 * K::kWorkers; i += kWgThreads) {
+            const int wk = i % K::kWorkers, e = i / K::kWorkers;
+            float v = 0.0f;
+            for (int g = 0; g < K::kGroups; ++g) v += red[e * kWgThreads + g * K::kWorkers + wk];
+            const int o = 4 * (wk / (CIN / 2)) + e / 18, c = 2 * (wk % (CIN / 2)) + (e & 1), k = e % 18 / 2;
+            out[(o * CIN + c) * 9 + k] = v;
+        }
     }
 }
 
-// Sum the chunk partials into the gradient vector (fixed order).
-template <int CIN, int COUT>
-__global__ void reduce_weight_kernel(const float* __restrict__ part, int P, float* __restrict__ gw, float* __restrict__ gb) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < COUT * CIN * 9) {
-        const int o = i / (CIN * 9), c = (i / 9) % CIN, k = i % 9;
-        float v = 0.0f;
-        for (int p = 0; p < P; ++p) v += part[(((size_t)p * COUT + o) * CIN + c) * 10 + k];
-        gw[i] = v;
-    } else if (i < COUT * CIN * 9 + COUT) {
-        const int o = i - COUT * CIN * 9;
-        float v = 0.0f;
-        for (int p = 0; p < P; ++p) v += part[(((size_t)p * COUT + o) * CIN + 0) * 10 + 9];
-        gb[o] = v;
+// The blocks' partials added in a fixed order: 32 values to a block, kReduceWays threads
+// to a value.  A thread's sum keeps its rounding errors (TwoSum) instead of running in FP64,
+// which is a small fraction of the FP32 rate here (41 us for the 32 -> 32 layer's 1024
+// partials, 10 now).
+constexpr int kReduceWays = 32;
+__global__ void __launch_bounds__(32 * kReduceWays) reduce_grad_kernel(const float* __restrict__ part, int P, int nw, int nb,
+                                                                       float* __restrict__ gw, float* __restrict__ gb) {
+    __shared__ double red[kReduceWays][32];
+    const int lane = threadIdx.x & 31, g = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
+    float s = 0.0f, e = 0.0f;
+    if (i < nw + nb) {
+#pragma unroll 8
+        for (int p = g; p < P; p += kReduceWays) {
+            const float v = __ldg(part + (size_t)p * (nw + nb) + i);
+            const float t = s + v, b = t - s;
+            e += (s - (t - b)) + (v - b);
+            s = t;
+        }
     }
+    red[g][lane] = (double)s + (double)e;
+    __syncthreads();
+    if (g == 0 && i < nw + nb) {
+        double v = 0.0;
+        for (int k = 0; k < kReduceWays; ++k) v += red[k][lane];
+        (i < nw ? gw[i] : gb[i - nw]) = (float)v;
+    }
+}
+
+template <int CIN, int COUT>
+cudaError_t launch_weight_grad(const float* in, const float* dout, float* part, int P, float* gw, float* gb, int nx, int ny,
+                               cudaStream_t st) {
+    typedef WgCfg<CIN, COUT> K;
+    cudaError_t e = cudaFuncSetAttribute(weight_grad_kernel<CIN, COUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)K::kSmem);
+    if (e != cudaSuccess) return e;
+    const int tiles_x = (nx + kWgW - 1) / kWgW, tiles = tiles_x * ((ny + kWgH - 1) / kWgH);
+    const int blocks = std::min(P, tiles);
+    weight_grad_kernel<CIN, COUT><<<blocks, kWgThreads, K::kSmem, st>>>(in, dout, part, nx, ny, tiles_x, tiles);
+    constexpr int nw = COUT * CIN * 9;
+    reduce_grad_kernel<<<(nw + COUT + 31) / 32, 32 * kReduceWays, 0, st>>>(part, blocks, nw, COUT, gw, gb);
+    return cudaGetLastError();
 }
 
 // d = 2 (y - t) / m and per-block partial sums of (y - t)^2 (double)
@@ -204,11 +378,6 @@ __global__ void loss_grad_kernel(const float* __restrict__ y, const float* __res
     }
 }
 
-__global__ void to_bf16_kernel(const float* __restrict__ p, __nv_bfloat16* __restrict__ q, int n) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) q[i] = __float2bfloat16_rn(p[i]);
-}
-
 __global__ void adam_kernel(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
                             float* __restrict__ v, int n, float lr, float b1t, float b2t) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -226,8 +395,7 @@ __global__ void adam_kernel(float* __restrict__ p, const float* __restrict__ g, 
 struct Net {
     int nx, ny;
     size_t n;
-    __nv_bfloat16* wb;
-    float *a1, *a2, *y, *dy, *dz2, *dz1, *part;
+    float *w, *a1, *a2, *y, *dy, *dz2, *dz1, *part;
     double* lpart;
     int P;
     cnn_tc::Bufs tc;   // tensor-core inference
@@ -235,13 +403,17 @@ struct Net {
 
 size_t align256(size_t v) { return (v + 255) / 256 * 256; }
 
+// Weight-gradient partials of an image: one per kPartPixels pixels, no more than
+// kMaxParts (92 MB of them).
+constexpr size_t kMaxParts = 2432, kPartFloats = kHid * kHid * 9 + kHid;
+size_t grad_parts(size_t n) { return std::min((n + kPartPixels - 1) / kPartPixels, kMaxParts); }
+
 // FP32 forward/backward buffers, then the tensor-core inference planes
 size_t training_bytes(int nx, int ny) {
     const size_t n = (size_t)nx * ny;
-    const size_t P = (n + kChunk - 1) / kChunk;
-    size_t b = align256(kParams * sizeof(__nv_bfloat16));
+    size_t b = align256(kConvWeights * sizeof(float));
     b += align256(kHid * n * 4) * 2 + align256(kOut * n * 4) * 2 + align256(kHid * n * 4) * 2;
-    b += align256(P * kHid * kHid * 10 * 4);
+    b += align256(grad_parts(n) * kPartFloats * 4);
     b += align256(1024 * sizeof(double));
     return b;
 }
@@ -253,27 +425,26 @@ Net carve(void* ws, int nx, int ny) {
     N.nx = nx;
     N.ny = ny;
     N.n = (size_t)nx * ny;
-    N.P = (int)((N.n + kChunk - 1) / kChunk);
+    N.P = (int)grad_parts(N.n);
     char* p = (char*)ws;
-    N.wb = (__nv_bfloat16*)p; p += align256(kParams * sizeof(__nv_bfloat16));
+    N.w = (float*)p; p += align256(kConvWeights * sizeof(float));
     N.a1 = (float*)p; p += align256(kHid * N.n * 4);
     N.a2 = (float*)p; p += align256(kHid * N.n * 4);
     N.y = (float*)p; p += align256(kOut * N.n * 4);
     N.dy = (float*)p; p += align256(kOut * N.n * 4);
     N.dz2 = (float*)p; p += align256(kHid * N.n * 4);
     N.dz1 = (float*)p; p += align256(kHid * N.n * 4);
-    N.part = (float*)p; p += align256((size_t)N.P * kHid * kHid * 10 * 4);
+    N.part = (float*)p; p += align256((size_t)N.P * kPartFloats * 4);
     N.lpart = (double*)p;
     N.tc = cnn_tc::carve((char*)ws + training_bytes(nx, ny), nx, ny);
     return N;
 }
 
 cudaError_t forward(const Net& N, const float* params, const float* x, float* y, cudaStream_t st) {
-    to_bf16_kernel<<<(kParams + 255) / 256, 256, 0, st>>>(params, N.wb, kParams);
-    dim3 grid((N.nx + kTile - 1) / kTile, (N.ny + kTile - 1) / kTile), blk(kTile, kTile);
-    conv_fwd_kernel<kIn, kHid, true><<<grid, blk, 0, st>>>(x, N.wb + kW1, params + kB1, N.a1, N.nx, N.ny);
-    conv_fwd_kernel<kHid, kHid, true><<<grid, blk, 0, st>>>(N.a1, N.wb + kW2, params + kB2, N.a2, N.nx, N.ny);
-    conv_fwd_kernel<kHid, kOut, false><<<grid, blk, 0, st>>>(N.a2, N.wb + kW3, params + kB3, y, N.nx, N.ny);
+    conv_weights_kernel<<<(kConvWeights + 255) / 256, 256, 0, st>>>(params, N.w);
+    launch_conv<kIn, kHid, kBiasRelu>(x, N.w + kF1, params + kB1, nullptr, N.a1, N.nx, N.ny, st);
+    launch_conv<kHid, kHid, kBiasRelu>(N.a1, N.w + kF2, params + kB2, nullptr, N.a2, N.nx, N.ny, st);
+    launch_conv<kHid, kOut, kBias>(N.a2, N.w + kF3, params + kB3, nullptr, y, N.nx, N.ny, st);
     return cudaGetLastError();
 }
 
@@ -286,19 +457,13 @@ cudaError_t loss_grad(const Net& N, const float* params, const float* x, const f
     const int nb = (int)std::min<size_t>(1024, (m + 255) / 256);
     loss_grad_kernel<<<nb, 256, 0, st>>>(N.y, t, N.dy, N.lpart, m);
     *nb_out = nb;
-    dim3 grid((N.nx + kTile - 1) / kTile, (N.ny + kTile - 1) / kTile), blk(kTile, kTile);
-    // layer 3
-    conv_bwd_weight_kernel<kHid, kOut><<<dim3(kOut * kHid, N.P), 256, 0, st>>>(N.a2, N.dy, N.part, N.nx, N.ny);
-    reduce_weight_kernel<kHid, kOut><<<(kOut * kHid * 9 + kOut + 255) / 256, 256, 0, st>>>(N.part, N.P, grad + kW3, grad + kB3);
-    conv_bwd_data_kernel<kHid, kOut, true><<<grid, blk, 0, st>>>(N.dy, N.wb + kW3, N.a2, N.dz2, N.nx, N.ny);
-    // layer 2
-    conv_bwd_weight_kernel<kHid, kHid><<<dim3(kHid * kHid, N.P), 256, 0, st>>>(N.a1, N.dz2, N.part, N.nx, N.ny);
-    reduce_weight_kernel<kHid, kHid><<<(kHid * kHid * 9 + kHid + 255) / 256, 256, 0, st>>>(N.part, N.P, grad + kW2, grad + kB2);
-    conv_bwd_data_kernel<kHid, kHid, true><<<grid, blk, 0, st>>>(N.dz2, N.wb + kW2, N.a1, N.dz1, N.nx, N.ny);
-    // layer 1
-    conv_bwd_weight_kernel<kIn, kHid><<<dim3(kHid * kIn, N.P), 256, 0, st>>>(x, N.dz1, N.part, N.nx, N.ny);
-    reduce_weight_kernel<kIn, kHid><<<(kHid * kIn * 9 + kHid + 255) / 256, 256, 0, st>>>(N.part, N.P, grad + kW1, grad + kB1);
-    return cudaGetLastError();
+    e = launch_weight_grad<kHid, kOut>(N.a2, N.dy, N.part, N.P, grad + kW3, grad + kB3, N.nx, N.ny, st);
+    if (e != cudaSuccess) return e;
+    launch_conv<kOut, kHid, kMask>(N.dy, N.w + kT3, nullptr, N.a2, N.dz2, N.nx, N.ny, st);
+    e = launch_weight_grad<kHid, kHid>(N.a1, N.dz2, N.part, N.P, grad + kW2, grad + kB2, N.nx, N.ny, st);
+    if (e != cudaSuccess) return e;
+    launch_conv<kHid, kHid, kMask>(N.dz2, N.w + kT2, nullptr, N.a1, N.dz1, N.nx, N.ny, st);
+    return launch_weight_grad<kIn, kHid>(x, N.dz1, N.part, N.P, grad + kW1, grad + kB1, N.nx, N.ny, st);
 }
 
 }  // namespace cnn
