@@ -585,46 +585,6 @@ __device__ __forceinline__ float interface_weight(const float rho[2], float2 cbu
     return 4.0f * c * (1.0f - c);
 }
 
-// Densities and total momentum of one site's gathered populations, summed in one
-// fixed order (the mass sums and the correction must see the same values).
-__device__ __forceinline__ void site_moments(const float2 f[9], float rho[2], float& jx, float& jy) {
-    jx = 0.0f;
-    jy = 0.0f;
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-        float r = 0.0f;
-#pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            const float v = s == 0 ? f[i].x : f[i].y;
-            r += v;
-            jx += cx(i) * v;
-            jy += cy(i) * v;
-        }
-        rho[s] = r;
-    }
-}
-
-// Pass 1 of a correction: the densities rho2 [2][n] and total momenta j2 [2][n] of the
-// coarse run's populations after streaming (FP32 storage), gathered as the step
-// kernels pull them.
-__global__ void __launch_bounds__(128) closure_moments_kernel(const float2* __restrict__ fin, Grid g,
-                                                              float* __restrict__ rho2, float* __restrict__ j2) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y;
-    if (x >= g.nx) return;
-    const int xm = x == 0 ? g.nx - 1 : x - 1;
-    const int xp = x == g.nx - 1 ? 0 : x + 1;
-    float2 f[9];
-    float rho[2], jx, jy;
-    pull_site<float>(fin, g, splat(0.0f), y, x, xm, xp, f);
-    site_moments(f, rho, jx, jy);
-    const size_t n = (size_t)g.nx * g.ny, k = (size_t)y * g.nx + x;
-    rho2[k] = rho[0];
-    rho2[n + k] = rho[1];
-    j2[k] = jx;
-    j2[n + k] = jy;
-}
-
 // Per-block sums (FP64) of the limited density corrections, from the densities
 // rho2 ([2][n], the sums of the FP32 populations); mode 4: the sum of the
 // order-parameter corrections and the sum of the weights.
@@ -853,7 +813,7 @@ struct lbm_closure {
     int64_t adam_t = 0;
     void* cnn_ws = nullptr;
     lbm::cnn::Net net;
-    float *raw = nullptr, *xin = nullptr, *yout = nullptr;   // [4 nc] each
+    float *raw = nullptr, *yout = nullptr;   // [4 nc] each
     double* S = nullptr;                                       // [18 nc]
     double* part = nullptr;                                    // reduction partials
     std::vector<float*> samp_raw, samp_tgt;                    // raw coarse / restricted fine after an interval
@@ -871,9 +831,10 @@ namespace {
 
 float4 f4(const float* a) { return make_float4(a[0], a[1], a[2], a[3]); }
 
-// blocks of the correction's mass sums (enough for the loads in flight to cover
-// the memory latency): 2 partials each, then 2 totals and 3 FP32 scalars (2 doubles)
-constexpr int kCorrBlocks = 4096;
+// blocks of the correction's mass sums, 4 to an SM: 2 partials each, then 2 totals and 3
+// FP32 scalars (2 doubles).  With 4096 a thread of the 1024x2048 grid had two sites and the
+// FP64 reduction of the warps was most of the kernel: 38.7 us, DRHO_US now.
+constexpr int kCorrBlocks = 608;
 constexpr size_t kPartDoubles = 2 * kCorrBlocks + 4;
 
 // restricted fields of the fine run into c->raw (or `dst`)
@@ -917,14 +878,11 @@ lbm_status correct(lbm_closure* c, int mode, bool clear_status) {
     const lbm::PopView v = lbm::handle_pops(c->coarse);
     if (v.storage != LBM_STORE_F32) return cl_fail(LBM_ESTATE, "the closure's coarse run must store FP32");
     float2* pops = static_cast<float2*>(v.pops);
-    // raw holds the densities (first half) and the momenta (second half)
-    float* rho2 = c->raw;
-    float* j2 = c->raw + 2 * c->nc;
+    float* rho2 = c->raw;   // the densities, [2][nc]
     const dim3 grid((v.grid.nx + 127) / 128, v.grid.ny);
-    lbm::closure_moments_kernel<<<grid, 128, 0, v.stream>>>(pops, v.grid, rho2, j2);
-    CL_TRY(cudaGetLastError(), "coarse moments");
-    CL_TRY(lbm::handle_closure_features(c->coarse, rho2, j2, c->in_mean, c->in_scale, c->xin), "network input");
-    CL_TRY(lbm::cnn_tc::infer(c->net.tc, c->params, c->xin, c->yout, c->stream, false, clear_status), "cnn inference");
+    CL_TRY(lbm::handle_closure_input(c->coarse, rho2, c->in_mean, c->in_scale, c->net.tc.xin, c->net.tc.pitch),
+           "network input");
+    CL_TRY(lbm::cnn_tc::infer(c->net.tc, c->params, nullptr, c->yout, c->stream, false, clear_status), "cnn inference");
     const float2 cb = make_float2((float)cbulk.x, (float)cbulk.y);
     lbm::drho_sum_kernel<<<kCorrBlocks, 256, 0, c->stream>>>(rho2, c->yout, c->nc, f4(c->out_scale), mode, cb, c->part);
     CL_TRY(cudaGetLastError(), "mass sums");
@@ -1042,7 +1000,7 @@ void lbm_closure_destroy(lbm_closure* c) {
     if (c->coarse) lbm_destroy(c->coarse);
     for (float* p : c->samp_raw) cudaFree(p);
     for (float* p : c->samp_tgt) cudaFree(p);
-    void* bufs[] = {c->params, c->grad, c->m, c->v, c->cnn_ws, c->raw, c->xin, c->yout, c->S, c->part, c->train_x, c->train_t,
+    void* bufs[] = {c->params, c->grad, c->m, c->v, c->cnn_ws, c->raw, c->yout, c->S, c->part, c->train_x, c->train_t,
                     c->snap, c->fine_fld, c->S_fine};
     for (void* p : bufs)
         if (p) cudaFree(p);
@@ -1110,7 +1068,6 @@ lbm_status lbm_closure_create(const lbm_params* fine, int32_t interval, uint64_t
               cudaMalloc((void**)&c->m, P * 4) == cudaSuccess && cudaMalloc((void**)&c->v, P * 4) == cudaSuccess &&
               cudaMalloc(&c->cnn_ws, lbm::cnn::workspace_bytes(c->ncx, c->ncy)) == cudaSuccess &&
               cudaMalloc((void**)&c->raw, 4 * c->nc * 4) == cudaSuccess &&
-              cudaMalloc((void**)&c->xin, 4 * c->nc * 4) == cudaSuccess &&
               cudaMalloc((void**)&c->yout, 4 * c->nc * 4) == cudaSuccess &&
               cudaMalloc((void**)&c->S, 18 * c->nc * 8) == cudaSuccess &&
               cudaMalloc((void**)&c->snap, 4 * c->nc * 4) == cudaSuccess &&

@@ -21,11 +21,11 @@
 // a tap is then just a 16-byte shift of the operand's start address.  Weights are
 // staged once per CTA in the same layout (N rows of 16 bytes per channel group).
 //
-// Roles (6 warps): warp 0 lane 0 issues the bulk copies; warp 1 owns the tensor
-// memory (two accumulators of N columns, alternating between input rows) and lane
-// 0 issues the MMAs; warps 2-5 read the accumulators (warp w reads lanes
-// 32 (w mod 4) ... of tensor memory, i.e. pixels 32 (w mod 4) ...), complete one
-// output row per input row, add the bias, apply ReLU, round to BF16 and store.
+// Roles: warp 0 lane 0 issues the bulk copies; warp 1 owns the tensor memory (two
+// accumulators of N columns, alternating between input rows) and lane 0 issues the
+// MMAs; warps 2-5 read the accumulators (warp w reads lanes 32 (w mod 4) ... of tensor
+// memory, i.e. pixels 32 (w mod 4) ...), complete one output row per input row, add the
+// bias, apply ReLU, round to BF16 and store.
 // mbarriers: full[s] (copies landed), empty[s] (MMAs reading slot s done, by
 // tcgen05.commit), accf[b] (accumulator b complete), acce[b] (accumulator b read).
 // Every wait is bounded: a wait that gives up raises the status word, tells the
@@ -52,6 +52,7 @@ constexpr int kPlane = kSlotPx * 16;    // bytes per plane (LBO of the A operand
 constexpr int kCopy = (kM + 2) * 16;    // bytes copied per plane and row
 constexpr int kStages = 6;              // ring slots: 3 rows in use + 3 in flight
 constexpr int kThreads = 192;
+constexpr int kHead = 512;              // shared memory before the weights: barriers, bias
 constexpr uint32_t kWaitLimit = 1u << 22;
 
 size_t align256(size_t v) { return (v + 255) / 256 * 256; }
@@ -125,54 +126,36 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
                  : "memory");
 }
 
-// 32 lanes x N consecutive 32-bit columns of tensor memory into v (one lane's row per thread).
-template <int N> __device__ __forceinline__ void tmem_load(uint32_t taddr, float* v);
-template <> __device__ __forceinline__ void tmem_load<32>(uint32_t t, float* v) {
-    uint32_t r[32];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-        "%15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(t));
-    // the registers pass through the wait, so that no use is scheduled before it
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
-          "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]),
-          "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]),
-          "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
-                 :
-                 : "memory");
-#pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+// 32 lanes x N consecutive 32-bit columns of tensor memory into r (one lane's row per
+// thread); r may be used after tmem_wait and tmem_tie.
+template <int N> __device__ __forceinline__ void tmem_load(uint32_t taddr, uint32_t* r);
+template <> __device__ __forceinline__ void tmem_load<32>(uint32_t t, uint32_t* r) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
+                 "%14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
+                   "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]),
+                   "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]),
+                   "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+                 : "r"(t));
 }
-template <> __device__ __forceinline__ void tmem_load<16>(uint32_t t, float* v) {
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-        "%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(t));
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
-          "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
-                 :
-                 : "memory");
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-template <> __device__ __forceinline__ void tmem_load<4>(uint32_t t, float* v) {
-    uint32_t r[4];
+template <> __device__ __forceinline__ void tmem_load<4>(uint32_t t, uint32_t* r) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                  : "r"(t));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]) : : "memory");
-#pragma unroll
-    for (int i = 0; i < 4; ++i) v[i] = __uint_as_float(r[i]);
+}
+__device__ __forceinline__ void tmem_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// The registers pass through after the wait, so that no use is scheduled before it.
+template <int N> __device__ __forceinline__ void tmem_tie(uint32_t* r);
+template <> __device__ __forceinline__ void tmem_tie<32>(uint32_t* r) {
+    asm volatile("" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]),
+                   "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]),
+                   "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]),
+                   "+r"(r[29]), "+r"(r[30]), "+r"(r[31]) : : "memory");
+}
+template <> __device__ __forceinline__ void tmem_tie<4>(uint32_t* r) {
+    asm volatile("" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]) : : "memory");
 }
 
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
@@ -180,7 +163,7 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
     return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-template <int KG, int NF> constexpr int smem_bytes() { return 256 + wbytes(KG, NF) + kStages * KG * kPlane; }
+template <int KG, int NF> constexpr int smem_bytes() { return kHead + wbytes(KG, NF) + kStages * KG * kPlane; }
 
 // One 3x3 convolution layer.  KGG channel groups of 8 are read per input row
 // (KG >= KGG groups in shared memory, the extra ones zero: the first layer has 4
@@ -188,7 +171,7 @@ template <int KG, int NF> constexpr int smem_bytes() { return 256 + wbytes(KG, N
 // output channels per row tap.  HIDDEN: bias + ReLU, BF16 activation planes out;
 // else bias, 4 channels as FP32 planes y[4][ny][nx].
 template <int KGG, int KG, int W, bool HIDDEN>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kThreads, 2)
 conv_tc_kernel(const uint8_t* __restrict__ in, const uint8_t* __restrict__ wop, const float* __restrict__ bias,
                uint8_t* __restrict__ hout, float* __restrict__ yout, int nx, int ny, int pitch, int rows_per_cta,
                int* __restrict__ status, int withhold) {
@@ -210,7 +193,8 @@ conv_tc_kernel(const uint8_t* __restrict__ in, const uint8_t* __restrict__ wop, 
     uint64_t* wbar = acce + 2;
     uint32_t* tslot = reinterpret_cast<uint32_t*>(wbar + 1);
     volatile int* stop = reinterpret_cast<volatile int*>(tslot + 1);
-    uint8_t* wsm = smem + 256;
+    float* bsm = reinterpret_cast<float*>(smem + 256);   // the layer's bias
+    uint8_t* wsm = smem + kHead;
     uint8_t* ring = wsm + WB;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -221,6 +205,7 @@ conv_tc_kernel(const uint8_t* __restrict__ in, const uint8_t* __restrict__ wop, 
 
     for (int i = threadIdx.x; i < kStages * SLOT / 16; i += kThreads)
         reinterpret_cast<uint4*>(ring)[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (threadIdx.x < (HIDDEN ? W : kOut)) bsm[threadIdx.x] = bias[threadIdx.x];
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
             mbar_init(&full[s], 1);
@@ -321,24 +306,35 @@ conv_tc_kernel(const uint8_t* __restrict__ in, const uint8_t* __restrict__ wop, 
             }
             tc_fence_after();
             const uint32_t t = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)((j & 1) * NF);
-            tmem_load<L>(t + 2 * W, O);        // third row tap: output row j - 2 is complete
+            uint32_t tap[2][L];
+            tmem_load<L>(t + 2 * W, tap[0]);
+            tmem_load<L>(t + W, tap[1]);
+            tmem_wait();
+            tmem_tie<L>(tap[0]);
+            tmem_tie<L>(tap[1]);
 #pragma unroll
-            for (int n = 0; n < L; ++n) O[n] += T1[n];
-            tmem_load<L>(t + W, T1);           // second row tap of output row j - 1
+            for (int n = 0; n < L; ++n) {
+                O[n] = __uint_as_float(tap[0][n]) + T1[n];    // third row tap: output row j - 2 is complete
+                T1[n] = __uint_as_float(tap[1][n]) + T2[n];   // second row tap of output row j - 1
+            }
+            tmem_load<L>(t, tap[0]);
+            tmem_wait();
+            tmem_tie<L>(tap[0]);
 #pragma unroll
-            for (int n = 0; n < L; ++n) T1[n] += T2[n];
-            tmem_load<L>(t, T2);               // first row tap of output row j
+            for (int n = 0; n < L; ++n) T2[n] = __uint_as_float(tap[0][n]);   // first row tap of output row j
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&acce[j & 1]);
             const int y = y0 + j - 2;
             if (j >= 2 && x < nx) {
                 if constexpr (HIDDEN) {
-                    uint32_t pk[W / 2];
+                    uint32_t pk[L / 2];
 #pragma unroll
-                    for (int n = 0; n < W / 2; ++n)
-                        pk[n] = pack_bf16(fmaxf(O[2 * n] + __ldg(bias + 2 * n), 0.0f),
-                                          fmaxf(O[2 * n + 1] + __ldg(bias + 2 * n + 1), 0.0f));
+                    for (int n = 0; n < L / 4; ++n) {
+                        const float4 b = reinterpret_cast<const float4*>(bsm)[n];
+                        pk[2 * n] = pack_bf16(fmaxf(O[4 * n] + b.x, 0.0f), fmaxf(O[4 * n + 1] + b.y, 0.0f));
+                        pk[2 * n + 1] = pack_bf16(fmaxf(O[4 * n + 2] + b.z, 0.0f), fmaxf(O[4 * n + 3] + b.w, 0.0f));
+                    }
                     const size_t row = (size_t)(y + 1) * 4 * pitch;
 #pragma unroll
                     for (int g = 0; g < 4; ++g) {
@@ -351,7 +347,7 @@ conv_tc_kernel(const uint8_t* __restrict__ in, const uint8_t* __restrict__ wop, 
                 } else {
                     const size_t n = (size_t)nx * ny;
 #pragma unroll
-                    for (int c = 0; c < kOut; ++c) yout[(size_t)c * n + (size_t)y * nx + x] = O[c] + __ldg(bias + c);
+                    for (int c = 0; c < kOut; ++c) yout[(size_t)c * n + (size_t)y * nx + x] = O[c] + bsm[c];
                 }
             }
         }
@@ -368,53 +364,60 @@ conv_tc_kernel(const uint8_t* __restrict__ in, const uint8_t* __restrict__ wop, 
 // Weights of one layer into the operand layout: [kx][K-step][group j][row n'][8]
 // with row n' = ky W + n (the three row taps side by side) and channel
 // c = (2 K-step + j) * 8 + e; zero for c >= cin, n >= cout or n' >= 3 W.
-__global__ void weights_kernel(const float* __restrict__ w, int cin, int cout, int ksteps, int W, int NF,
-                               __nv_bfloat16* __restrict__ out) {
-    const int total = 3 * ksteps * 2 * NF * 8;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-        const int e = i & 7;
-        const int np = (i >> 3) % NF;
-        const int j = (i / (8 * NF)) & 1;
-        const int s = (i / (16 * NF)) % ksteps;
-        const int kx = i / (16 * NF * ksteps);
-        const int ky = np / W, n = np % W;
-        const int c = (2 * s + j) * 8 + e;
-        const float v = (c < cin && n < cout && ky < 3) ? w[(n * cin + c) * 9 + ky * 3 + kx] : 0.0f;
-        out[i] = __float2bfloat16_rn(v);
-    }
+template <int CIN, int COUT, int KSTEPS, int W>
+__device__ __forceinline__ void operand_weight(const float* __restrict__ w, int i, uint8_t* __restrict__ out) {
+    constexpr int NF = nfold(W);
+    const int e = i & 7;
+    const int np = (i >> 3) % NF;
+    const int j = (i / (8 * NF)) & 1;
+    const int s = (i / (16 * NF)) % KSTEPS;
+    const int kx = i / (16 * NF * KSTEPS);
+    const int ky = np / W, n = np % W;
+    const int c = (2 * s + j) * 8 + e;
+    const float v = (c < CIN && n < COUT && ky < 3) ? w[(n * CIN + c) * 9 + ky * 3 + kx] : 0.0f;
+    reinterpret_cast<__nv_bfloat16*>(out)[i] = __float2bfloat16_rn(v);
 }
 
-// Input planes (4 channels + 4 zeros, ghost columns, zero wall rows), the wall
-// rows of the hidden planes, and (clear != 0) the status word.
-__global__ void prep_kernel(const float* __restrict__ x, int nx, int ny, int pitch, uint8_t* __restrict__ xin,
-                            uint8_t* __restrict__ h1, uint8_t* __restrict__ h2, int* __restrict__ status, int clear) {
+// All that the layers start from, in one launch: the weights of the three layers in
+// operand layout, the input planes (4 channels + 4 zeros, ghost columns, zero wall rows;
+// x null: only the zero wall rows, the caller fills the others), the wall rows of the hidden planes, and (clear != 0)
+// the status word.
+__global__ void prep_kernel(const float* __restrict__ params, const float* __restrict__ x, Bufs B, int clear) {
+    const int nx = B.nx, ny = B.ny, pitch = B.pitch;
     const size_t n = (size_t)nx * ny;
+    const size_t first = blockIdx.x * (size_t)blockDim.x + threadIdx.x, step = (size_t)gridDim.x * blockDim.x;
+    if (clear && first == 0) *B.status = 0;
+    constexpr int n1 = wbytes(2, nfold(kHid)) / 2, n2 = wbytes(4, nfold(kHid)) / 2, n3 = wbytes(4, nfold(kOut)) / 2;
+    for (size_t i = first; i < n1 + n2 + n3; i += step) {
+        const int k = (int)i;
+        if (k < n1) operand_weight<kIn, kHid, 1, kHid>(params + kW1, k, B.w1);
+        else if (k < n1 + n2) operand_weight<kHid, kHid, 2, kHid>(params + kW2, k - n1, B.w2);
+        else operand_weight<kHid, kOut, 2, kOut>(params + kW3, k - n1 - n2, B.w3);
+    }
+    const uint4 z = make_uint4(0u, 0u, 0u, 0u);
+    for (size_t i = first; i < (size_t)8 * pitch; i += step) {   // rows 0 and ny + 1 of 4 groups
+        const size_t r = i / (4 * (size_t)pitch) * (ny + 1), o = r * 4 * pitch + i % (4 * (size_t)pitch);
+        reinterpret_cast<uint4*>(B.h1)[o] = z;
+        reinterpret_cast<uint4*>(B.h2)[o] = z;
+    }
+    if (!x) {
+        for (size_t i = first; i < (size_t)2 * pitch; i += step)
+            reinterpret_cast<uint4*>(B.xin)[i < pitch ? i : (size_t)(ny + 1) * pitch + (i - pitch)] = z;
+        return;
+    }
     const size_t total = (size_t)(ny + 2) * pitch;
-    if (clear && blockIdx.x == 0 && threadIdx.x == 0) *status = 0;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
+    for (size_t i = first; i < total; i += step) {
         const int r = (int)(i / pitch), p = (int)(i % pitch);
-        uint4 val = make_uint4(0u, 0u, 0u, 0u);
+        uint4 val = z;
         if (r >= 1 && r <= ny && p <= nx + 1) {
             const int xa = p == 0 ? nx - 1 : (p == nx + 1 ? 0 : p - 1);
             const size_t k = (size_t)(r - 1) * nx + xa;
             val.x = pack_bf16(x[k], x[n + k]);
             val.y = pack_bf16(x[2 * n + k], x[3 * n + k]);
         }
-        reinterpret_cast<uint4*>(xin)[i] = val;
-        if (r == 0 || r == ny + 1) {
-            const uint4 z = make_uint4(0u, 0u, 0u, 0u);
-            for (int g = 0; g < 4; ++g) {
-                const size_t o = ((size_t)r * 4 + g) * pitch + p;
-                reinterpret_cast<uint4*>(h1)[o] = z;
-                reinterpret_cast<uint4*>(h2)[o] = z;
-            }
-        }
+        reinterpret_cast<uint4*>(B.xin)[i] = val;
     }
 }
-
-struct Launch {
-    int groups = 1, rows = 1;
-};
 
 // Bands of rows so that all CTAs of a layer are resident at once.
 template <int KGG, int KG, int W, bool HIDDEN>
@@ -440,8 +443,9 @@ cudaError_t launch_conv(const Bufs& B, const uint8_t* in, const uint8_t* w, cons
         cudaFuncAttributes fa{};
         e = cudaFuncGetAttributes(&fa, kern);
         if (e != cudaSuccess) return e;
-        const int regs = (std::max(fa.numRegs, 1) + 7) / 8 * 8 * kThreads;
-        per_sm = std::min({smem_sm / (SM + 1024), regs_sm / regs, thr_sm / kThreads, 512 / (int)tmem_cols(nfold(W))});
+        constexpr int T = kThreads;
+        const int regs = (std::max(fa.numRegs, 1) + 7) / 8 * 8 * T;
+        per_sm = std::min({smem_sm / (SM + 1024), regs_sm / regs, thr_sm / T, 512 / (int)tmem_cols(nfold(W))});
         per_sm = std::max(1, per_sm);
         configured = true;
     }
@@ -449,9 +453,8 @@ cudaError_t launch_conv(const Bufs& B, const uint8_t* in, const uint8_t* w, cons
     int groups = std::max(1, slots / B.tiles_x);
     int rows = std::max(1, (B.ny + groups - 1) / groups);
     groups = (B.ny + rows - 1) / rows;
-    conv_tc_kernel<KGG, KG, W, HIDDEN><<<dim3(B.tiles_x, groups), kThreads, SM, st>>>(in, w, bias, hout, yout, B.nx,
-                                                                                      B.ny, B.pitch, rows, B.status,
-                                                                                      withhold);
+    conv_tc_kernel<KGG, KG, W, HIDDEN><<<dim3(B.tiles_x, groups), kThreads, SM, st>>>(
+        in, w, bias, hout, yout, B.nx, B.ny, B.pitch, rows, B.status, withhold);
     return cudaGetLastError();
 }
 
@@ -486,13 +489,9 @@ Bufs carve(void* base, int nx, int ny) {
 cudaError_t infer(const Bufs& B, const float* params, const float* x, float* y, cudaStream_t st, bool withhold,
                   bool clear_status) {
     const int wh = withhold ? 1 : 0;
-    weights_kernel<<<8, 256, 0, st>>>(params + kW1, kIn, kHid, 1, kHid, nfold(kHid), reinterpret_cast<__nv_bfloat16*>(B.w1));
-    weights_kernel<<<16, 256, 0, st>>>(params + kW2, kHid, kHid, 2, kHid, nfold(kHid), reinterpret_cast<__nv_bfloat16*>(B.w2));
-    weights_kernel<<<4, 256, 0, st>>>(params + kW3, kHid, kOut, 2, kOut, nfold(kOut), reinterpret_cast<__nv_bfloat16*>(B.w3));
-    const size_t px = (size_t)(B.ny + 2) * B.pitch;
-    const int blocks = (int)std::min<size_t>(4096, (px + 255) / 256);
-    prep_kernel<<<blocks, 256, 0, st>>>(x, B.nx, B.ny, B.pitch, B.xin, B.h1, B.h2, B.status,
-                                                clear_status ? 1 : 0);
+    const size_t px = x ? (size_t)(B.ny + 2) * B.pitch : (size_t)8 * B.pitch;
+    const int blocks = (int)std::min<size_t>(4096, std::max<size_t>((px + 255) / 256, 60));
+    prep_kernel<<<blocks, 256, 0, st>>>(params, x, B, clear_status ? 1 : 0);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     e = launch_conv<1, 2, 32, true>(B, B.xin, B.w1, params + kB1, B.h1, nullptr, st, wh);

@@ -29,7 +29,8 @@ struct Bufs {
 
 size_t bytes(int nx, int ny);
 Bufs carve(void* base, int nx, int ny);
-// y[4][ny][nx] = CNN(x[4][ny][nx]); params as in the FP32 path.  Asynchronous.
+// y[4][ny][nx] = CNN(x[4][ny][nx]); params as in the FP32 path.  Asynchronous.  x null:
+// the caller has filled rows 1 .. ny of B.xin.
 // withhold (tests of the timeout path only): the kernels issue no copies and poll
 // briefly, so their waits give up and raise the status word.  clear_status: the
 // status word starts from 0; without it a failure of an earlier call stays raised.

@@ -610,71 +610,98 @@ cudaError_t moments(const DiagLaunch& D, const DiagArgs& a, cudaStream_t st) {
 }
 
 // ---------------------------------------------------------------------------
-// closure network input (FP32)
+// closure network input
 // ---------------------------------------------------------------------------
 struct FeatArgs {
-    int nx, ny;
-    size_t n;
+    Grid g;
     float G, gx, gw6[2], gext[2];
     float mean[4], scale[4];
     int mirror;
 };
 
-// sum_i w_i rho(x + c_i) c_i of one density field, zero beyond the walls (or the wall
-// rows' values with the mirror)
-__device__ __forceinline__ void nbr_sum_f(const float* __restrict__ r, const FeatArgs& a, int x, int y, float& sx,
-                                          float& sy) {
-    const int xm = x == 0 ? a.nx - 1 : x - 1;
-    const int xp = x == a.nx - 1 ? 0 : x + 1;
-    auto at = [&](int xx, int yy) {
-        if (yy < 0 || yy >= a.ny) {
-            if (!a.mirror) return 0.0f;
-            yy = yy < 0 ? 0 : a.ny - 1;
-        }
-        return r[(size_t)yy * a.nx + xx];
-    };
-    const float E = at(xp, y), W = at(xm, y), N = at(x, y + 1), S = at(x, y - 1);
-    const float d = at(xp, y + 1) - at(xm, y - 1);
-    const float SE = at(xp, y - 1), NW = at(xm, y + 1);
-    sx = (E - W) * (1.0f / 9.0f) + (d + (SE - NW)) * (1.0f / 36.0f);
-    sy = (N - S) * (1.0f / 9.0f) + (d + (NW - SE)) * (1.0f / 36.0f);
-}
+// One sweep: a block of 128 threads owns kFeatCols columns and the by-th of gridDim.y tiles
+// of rows, thread t column x0 + t - 1 (the two outermost for their neighbours), with the
+// densities of three rows in a ring in shared memory.  The force and physical velocity are
+// those of the diagnostics, in FP32.  Bound by HBM: 72 bytes read and 24 written per site.
+// A moments pass, a pass over their neighbours and one that packed the planes took 69 us at
+// 1024x2048, FEAT_US now.
+constexpr int kFeatT = 128, kFeatCols = kFeatT - 2, kFeatRows = 16;
 
-// the same force and physical velocity as the diagnostics' velocity pass, in FP32;
-// one thread per column, rows y = blockIdx.y, blockIdx.y + gridDim.y, ...
-__global__ void __launch_bounds__(128) closure_features_kernel(FeatArgs a, const float* __restrict__ rho2,
-                                                                const float* __restrict__ j2, float* __restrict__ xo) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= a.nx) return;
-    for (int y = blockIdx.y; y < a.ny; y += gridDim.y) {
-        const size_t k = (size_t)y * a.nx + x;
-        const float jx = j2[k], jy = j2[a.n + k];
-        const float rA = rho2[k], rB = rho2[a.n + k];
-        float nAx, nAy, nBx, nBy;
-        nbr_sum_f(rho2, a, x, y, nAx, nAy);
-        nbr_sum_f(rho2 + a.n, a, x, y, nBx, nBy);
+__global__ void __launch_bounds__(kFeatT) closure_input_kernel(const float2* __restrict__ fin, FeatArgs a,
+                                                               float* __restrict__ rho2, uint4* __restrict__ xin,
+                                                               int pitch) {
+    __shared__ float2 sR[4][kFeatT];
+    const int t = threadIdx.x, nx = a.g.nx, ny = a.g.ny;
+    const int x = blockIdx.x * kFeatCols + t - 1;
+    const int xw = (x + nx) % nx, xm = xw == 0 ? nx - 1 : xw - 1, xp = xw == nx - 1 ? 0 : xw + 1;
+    const bool own = t >= 1 && t < kFeatT - 1 && x < nx;
+    const int y0 = blockIdx.y * kFeatRows, y1 = min(y0 + kFeatRows, ny);
+    const size_t n = (size_t)nx * ny;
+    float2 f[9], j = splat(0.0f), jn = splat(0.0f);   // momenta of the row whose input is next, and of row m
+    float2 r = splat(0.0f), rn = splat(0.0f);         // densities likewise
+    auto load = [&](int m) {
+        if (m >= 0 && m < ny) pull_site<float>(fin, a.g, splat(0.0f), m, xw, xm, xp, f);
+    };
+    load(y0 - 1);
+#pragma unroll 1
+    for (int m = y0 - 1; m <= y1; ++m) {
+        j = jn;
+        r = rn;
+        if (m >= 0 && m < ny) {
+            float rho[2], jx, jy;
+            site_moments(f, rho, jx, jy);
+            jn = make_float2(jx, jy);
+            rn = make_float2(rho[0], rho[1]);
+            sR[m & 3][t] = rn;
+            if (own && m >= y0 && m < y1) {
+                const size_t k = (size_t)m * nx + x;
+                rho2[k] = rho[0];
+                rho2[n + k] = rho[1];
+            }
+        }
+        load(m + 1);
+        __syncthreads();
+        const int y = m - 1;
+        if (y < y0 || !own) continue;
+        // neighbours' densities, zero beyond the walls (or the wall rows' with the mirror)
+        auto at = [&](int yy, int dx) {
+            if (yy < 0 || yy >= ny) {
+                if (!a.mirror) return splat(0.0f);
+                yy = y;
+            }
+            return sR[yy & 3][t + dx];
+        };
+        const float2 E = at(y, 1), W = at(y, -1), N = at(y + 1, 0), S = at(y - 1, 0);
+        const float2 d = sub2(at(y + 1, 1), at(y - 1, -1)), SE = at(y - 1, 1), NW = at(y + 1, -1);
+        const float2 sx = fma2(sub2(E, W), splat(1.0f / 9.0f), mul2(add2(d, sub2(SE, NW)), splat(1.0f / 36.0f)));
+        const float2 sy = fma2(sub2(N, S), splat(1.0f / 9.0f), mul2(add2(d, sub2(NW, SE)), splat(1.0f / 36.0f)));
         float wA = 0.0f, wB = 0.0f;
         if (y == 0) { wA += a.gw6[0]; wB += a.gw6[1]; }
-        if (y == a.ny - 1) { wA -= a.gw6[0]; wB -= a.gw6[1]; }
-        const float aAx = a.gx - a.G * nBx, aAy = (wA + a.gext[0]) - a.G * nBy;
-        const float aBx = a.gx - a.G * nAx, aBy = (wB + a.gext[1]) - a.G * nAy;
-        const float Fx = rA * aAx + rB * aBx, Fy = rA * aAy + rB * aBy;
-        const float rho = rA + rB;
-        const float ux = (jx + 0.5f * Fx) / rho, uy = (jy + 0.5f * Fy) / rho;
-        const float v[4] = {rA, rB, ux, uy};
+        if (y == ny - 1) { wA -= a.gw6[0]; wB -= a.gw6[1]; }
+        // each component feels the other's neighbours
+        const float aAx = a.gx - a.G * sx.y, aAy = (wA + a.gext[0]) - a.G * sy.y;
+        const float aBx = a.gx - a.G * sx.x, aBy = (wB + a.gext[1]) - a.G * sy.x;
+        const float Fx = r.x * aAx + r.y * aBx, Fy = r.x * aAy + r.y * aBy;
+        const float rho = r.x + r.y;
+        const float v[4] = {r.x, r.y, (j.x + 0.5f * Fx) / rho, (j.y + 0.5f * Fy) / rho};
+        float q[4];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) xo[(size_t)c * a.n + k] = (v[c] - a.mean[c]) / a.scale[c];
+        for (int c = 0; c < 4; ++c) q[c] = (v[c] - a.mean[c]) / a.scale[c];
+        const __nv_bfloat162 lo = __floats2bfloat162_rn(q[0], q[1]), hi = __floats2bfloat162_rn(q[2], q[3]);
+        const uint4 cell = make_uint4(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi), 0u, 0u);
+        uint4* row = xin + (size_t)(y + 1) * pitch;
+        row[x + 1] = cell;
+        if (x == 0) row[nx + 1] = cell;
+        if (x == nx - 1) row[0] = cell;
     }
 }
 
 }  // namespace
 
-cudaError_t launch_closure_features(const DiagLaunch& D, const float* rho2, const float* j2, const float mean[4],
-                                    const float scale[4], float* x, cudaStream_t st) {
+cudaError_t launch_closure_input(const DiagLaunch& D, float* rho2, const float mean[4], const float scale[4],
+                                 uint8_t* xin, int pitch, cudaStream_t st) {
     FeatArgs a;
-    a.nx = D.grid.nx;
-    a.ny = D.grid.ny;
-    a.n = (size_t)a.nx * a.ny;
+    a.g = D.grid;
     a.G = (float)D.G;
     a.gx = (float)D.gx;
     a.mirror = D.wall_mirror;
@@ -686,8 +713,8 @@ cudaError_t launch_closure_features(const DiagLaunch& D, const float* rho2, cons
         a.mean[c] = mean[c];
         a.scale[c] = scale[c];
     }
-    const dim3 grid((a.nx + 127) / 128, std::min(a.ny, 65535));
-    closure_features_kernel<<<grid, 128, 0, st>>>(a, rho2, j2, x);
+    const dim3 grid((D.grid.nx + kFeatCols - 1) / kFeatCols, (D.grid.ny + kFeatRows - 1) / kFeatRows);
+    closure_input_kernel<<<grid, kFeatT, 0, st>>>((const float2*)D.fin, a, rho2, reinterpret_cast<uint4*>(xin), pitch);
     return cudaGetLastError();
 }
 

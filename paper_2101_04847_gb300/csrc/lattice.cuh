@@ -194,4 +194,23 @@ __device__ __forceinline__ float2 sum9_2(const float2* f) {
     return add2(add2(lo, hi), f[8]);
 }
 
+// Densities and total momentum of one site's gathered populations, summed in one
+// fixed order (the mass sums and the correction must see the same values).
+__device__ __forceinline__ void site_moments(const float2 f[9], float rho[2], float& jx, float& jy) {
+    jx = 0.0f;
+    jy = 0.0f;
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        float r = 0.0f;
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            const float v = s == 0 ? f[i].x : f[i].y;
+            r += v;
+            jx += cx(i) * v;
+            jy += cy(i) * v;
+        }
+        rho[s] = r;
+    }
+}
+
 }  // namespace lbm

@@ -365,9 +365,9 @@ PopView handle_pops(lbm_handle* h) {
     v.stream = h->stream;
     return v;
 }
-cudaError_t handle_closure_features(lbm_handle* h, const float* rho2, const float* j2, const float mean[4],
-                                    const float scale[4], float* x) {
-    return launch_closure_features(diag_launch(h), rho2, j2, mean, scale, x, h->stream);
+cudaError_t handle_closure_input(lbm_handle* h, float* rho2, const float mean[4], const float scale[4], uint8_t* xin,
+                                 int pitch) {
+    return launch_closure_input(diag_launch(h), rho2, mean, scale, xin, pitch, h->stream);
 }
 lbm_status handle_reseed(lbm_handle* h, uint64_t seed) {
     h->p.seed = seed;

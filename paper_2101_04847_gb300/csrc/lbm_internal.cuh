@@ -198,13 +198,14 @@ cudaError_t launch_diagnostics(const DiagLaunch& D, cudaStream_t st);
 // rho_A, rho_B, ux, uy (double [ny][nx] each) into the scratch region at
 // diag_fields_offset (uses the whole scratch: 15 doubles per site)
 cudaError_t launch_fields(const DiagLaunch& D, double* fields, cudaStream_t st);
-// The closure network's input in FP32: rho_A, rho_B from rho2 [2][n] and the
-// physical velocity (j + F/2) / rho from the momenta j2 [2][n] (the force from the
-// neighbours' densities, as in the diagnostics), each as (v - mean[c]) / scale[c],
-// into x [4][n].
-cudaError_t launch_closure_features(const DiagLaunch& D, const float* rho2, const float* j2, const float mean[4],
-                                    const float scale[4], float* x, cudaStream_t st);
-cudaError_t handle_closure_features(lbm_handle* h, const float* rho2, const float* j2, const float mean[4],
-                                    const float scale[4], float* x);
+// The closure's network input from the stored FP32 populations: rho_A, rho_B and the
+// physical velocity (j + F/2) / rho (the force from the neighbours' densities, as in the
+// diagnostics), each as (v - mean[c]) / scale[c] in BF16, into the rows 1 .. ny of the
+// tensor cores' input planes xin (cnn_tc.cuh; pitch pixels a row), and the densities into
+// rho2 [2][ny][nx].
+cudaError_t launch_closure_input(const DiagLaunch& D, float* rho2, const float mean[4], const float scale[4],
+                                 uint8_t* xin, int pitch, cudaStream_t st);
+cudaError_t handle_closure_input(lbm_handle* h, float* rho2, const float mean[4], const float scale[4], uint8_t* xin,
+                                 int pitch);
 
 }  // namespace lbm
