@@ -193,7 +193,7 @@ def run_ours(args):
     with torch.cuda.stream(stream):
         solver = lbm.Solver(storage=args.storage, kernel=args.kernel, tile_y=args.tile_y, **params)
     sites = args.nx * args.ny
-    launches_per_step = LB_STEPS_PER_STEP * (2 if args.kernel == "two_pass" else 1) + 5
+    launches_per_step = LB_STEPS_PER_STEP * (2 if args.kernel == "two_pass" else 1) + 2   # the diagnostics: a sweep and a reduction
 
     def one_step(ev_pair=None):
         if ev_pair is not None:

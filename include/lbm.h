@@ -76,7 +76,7 @@ typedef enum {
                               * keeps its own density ring, stages are handed back through per-stage barriers */
     LBM_KERNEL_PAIRED = 6    /* 16-bit storage only: as STAGED with 256-column tiles, each thread owning two
                               * neighbouring columns (per-row work shared by two sites, paired 32-bit stores);
-                              * what STAGED runs for 16-bit storage when tile_x is 0 */
+                              * what STAGED runs for 16-bit storage when tile_x is 0 and nx > 128 */
 } lbm_kernel;
 
 /* Parameters (lattice units, dx = dt = 1).  lbm_params_default() fills them. */
@@ -101,13 +101,15 @@ typedef struct {
     int32_t kernel;          /* lbm_kernel */
     int32_t tile_y;          /* at most this many rows per block tile of the step kernel (the
                               * rows are split evenly over the tiles); 0 = the kernel's default
-                              * (block-staged: one wave of tiles filling every SM) */
+                              * (block-staged: as short as one wave of tiles filling every SM
+                              * allows, or several waves of about 32 rows) */
     double shift_A, shift_B; /* rho0_s of the shifted storage; <= 0 means (mass_s (1 + minority)) / 2 */
     int32_t tile_x;          /* columns per block tile of the block-staged kernel: 128 or 256
                               * (one column per thread); 0 = chosen per grid: for 16-bit storage
                               * the paired-column tile (256 columns, two per thread, the
-                              * LBM_KERNEL_PAIRED kernel), for FP32 256 when the 256-column tiles
-                              * are at least 64 rows tall, else 128.  Other kernels ignore it.
+                              * LBM_KERNEL_PAIRED kernel) unless nx <= 128, for FP32 256 when one
+                              * wave of 256-column tiles is at least 64 rows tall, else 128.  Other
+                              * kernels ignore it.
                               * Ensembles (the first member's value): 128 or 256 columns, one
                               * per thread, for every member; 0 = 16-bit members in paired
                               * 256-column tiles, FP32 members in 128-column ones, or 256
