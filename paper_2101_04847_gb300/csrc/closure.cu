@@ -69,26 +69,31 @@ __global__ void conv_weights_kernel(const float* __restrict__ p, float* __restri
 // against 36 weight loads (16 bytes, broadcast), 6 input loads and 18 moves, so the FMA
 // pipe is what bounds it.  One pixel and all 32 channels per thread with scalar weight loads
 // took as many loads as FMAs: 506 us for the 32 -> 32 layer at 512x1024, 188 now.
+// kSmall: tiles of 32 x 4 pixels and 4 output channels per thread, for images that make few
+// blocks: a thread's own chain of FMAs sets the time there (loss and
+// gradient of a 24 x 24 image 198 -> 162 us); one tile per weight-gradient
+// block brings it to 126.
 enum Epi { kBias, kBiasRelu, kMask };
-constexpr int kConvW = 32, kConvH = 16, kConvPitch = 36;   // tile; floats per staged row (34 used)
+constexpr int kConvW = 32, kConvPitch = 36;   // tile width; floats per staged row (34 used)
 
-template <int CIN, int COUT, Epi EPI>
+template <int CIN, int COUT, bool kSmall>
 struct ConvCfg {
-    static constexpr int TO = COUT < 16 ? COUT : 16;               // output channels per thread
-    static constexpr int CH = CIN < 8 ? CIN : 8;                   // input channels staged at a time
-    static constexpr int kThreads = (kConvW / 4) * kConvH * (COUT / TO);
+    static constexpr int H = kSmall ? 4 : 16;                                       // tile height
+    static constexpr int TO = kSmall || COUT < 16 ? 4 : 16;                         // output channels per thread
+    static constexpr int CH = CIN < 8 ? CIN : 8;                                    // input channels staged at a time
+    static constexpr int kThreads = (kConvW / 4) * H * (COUT / TO);
 };
 
-template <int CIN, int COUT, Epi EPI>
-__global__ void __launch_bounds__((ConvCfg<CIN, COUT, EPI>::kThreads), 2)
+template <int CIN, int COUT, Epi EPI, bool kSmall>
+__global__ void __launch_bounds__((ConvCfg<CIN, COUT, kSmall>::kThreads), 2)
 conv_kernel(const float* __restrict__ in, const float* __restrict__ w, const float* __restrict__ b,
             const float* __restrict__ act, float* __restrict__ out, int nx, int ny) {
-    typedef ConvCfg<CIN, COUT, EPI> K;
-    constexpr int TO = K::TO, CH = K::CH, T = K::kThreads;
+    typedef ConvCfg<CIN, COUT, kSmall> K;
+    constexpr int TO = K::TO, CH = K::CH, T = K::kThreads, kConvH = K::H;
     __shared__ __align__(16) float si[CH][kConvH + 2][kConvPitch];
     __shared__ __align__(16) float sw[CH * 9 * COUT];
     const int tid = threadIdx.x;
-    const int tx = tid & 7, ty = (tid >> 3) & 15, half = tid >> 7;
+    const int tx = tid & 7, ty = (tid >> 3) % kConvH, half = tid / (8 * kConvH);   // half: which TO channels
     const int bx = blockIdx.x * kConvW, by = blockIdx.y * kConvH;
     const size_t n = (size_t)nx * ny;
     float2 acc[4][TO / 2];
@@ -168,11 +173,19 @@ conv_kernel(const float* __restrict__ in, const float* __restrict__ w, const flo
     }
 }
 
+constexpr int kTallTiles = 304;
+
 template <int CIN, int COUT, Epi EPI>
 void launch_conv(const float* in, const float* w, const float* b, const float* act, float* out, int nx, int ny,
                  cudaStream_t st) {
-    const dim3 grid((nx + kConvW - 1) / kConvW, (ny + kConvH - 1) / kConvH);
-    conv_kernel<CIN, COUT, EPI><<<grid, ConvCfg<CIN, COUT, EPI>::kThreads, 0, st>>>(in, w, b, act, out, nx, ny);
+    // fewer tall tiles than two to an SM: the short ones
+    typedef ConvCfg<CIN, COUT, false> Tall;
+    typedef ConvCfg<CIN, COUT, true> Short;
+    const int gx = (nx + kConvW - 1) / kConvW, tall = (ny + Tall::H - 1) / Tall::H, low = (ny + Short::H - 1) / Short::H;
+    if ((long long)gx * tall < kTallTiles)
+        conv_kernel<CIN, COUT, EPI, true><<<dim3(gx, low), Short::kThreads, 0, st>>>(in, w, b, act, out, nx, ny);
+    else
+        conv_kernel<CIN, COUT, EPI, false><<<dim3(gx, tall), Tall::kThreads, 0, st>>>(in, w, b, act, out, nx, ny);
 }
 
 // Partial weight and bias gradients, part[block][COUT * CIN * 9 + COUT] in the parameters'
@@ -404,16 +417,20 @@ struct Net {
 size_t align256(size_t v) { return (v + 255) / 256 * 256; }
 
 // Weight-gradient partials of an image: one per kPartPixels pixels, no more than
-// kMaxParts (92 MB of them).
-constexpr size_t kMaxParts = 2432, kPartFloats = kHid * kHid * 9 + kHid;
-size_t grad_parts(size_t n) { return std::min((n + kPartPixels - 1) / kPartPixels, kMaxParts); }
+// kMaxParts (92 MB of them); on small images one per tile, so that a block has one tile.
+constexpr size_t kMaxParts = 2432, kTileParts = 304, kPartFloats = kHid * kHid * 9 + kHid;
+size_t grad_parts(int nx, int ny) {
+    const size_t n = (size_t)nx * ny;
+    const size_t tiles = ((size_t)(nx + kWgW - 1) / kWgW) * ((size_t)(ny + kWgH - 1) / kWgH);
+    return std::min(std::max((n + kPartPixels - 1) / kPartPixels, std::min(tiles, kTileParts)), kMaxParts);
+}
 
 // FP32 forward/backward buffers, then the tensor-core inference planes
 size_t training_bytes(int nx, int ny) {
     const size_t n = (size_t)nx * ny;
     size_t b = align256(kConvWeights * sizeof(float));
     b += align256(kHid * n * 4) * 2 + align256(kOut * n * 4) * 2 + align256(kHid * n * 4) * 2;
-    b += align256(grad_parts(n) * kPartFloats * 4);
+    b += align256(grad_parts(nx, ny) * kPartFloats * 4);
     b += align256(1024 * sizeof(double));
     return b;
 }
@@ -425,7 +442,7 @@ Net carve(void* ws, int nx, int ny) {
     N.nx = nx;
     N.ny = ny;
     N.n = (size_t)nx * ny;
-    N.P = (int)grad_parts(N.n);
+    N.P = (int)grad_parts(nx, ny);
     char* p = (char*)ws;
     N.w = (float*)p; p += align256(kConvWeights * sizeof(float));
     N.a1 = (float*)p; p += align256(kHid * N.n * 4);
