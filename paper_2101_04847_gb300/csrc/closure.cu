@@ -70,9 +70,8 @@ __global__ void conv_weights_kernel(const float* __restrict__ p, float* __restri
 // pipe is what bounds it.  One pixel and all 32 channels per thread with scalar weight loads
 // took as many loads as FMAs: 506 us for the 32 -> 32 layer at 512x1024, 188 now.
 // kSmall: tiles of 32 x 4 pixels and 4 output channels per thread, for images that make few
-// blocks: a thread's own chain of FMAs sets the time there (loss and
-// gradient of a 24 x 24 image 198 -> 162 us); one tile per weight-gradient
-// block brings it to 126.
+// blocks: a thread's own chain of FMAs sets the time there (loss and gradient of a
+// 24 x 24 image 198 -> 162 us; one tile per weight-gradient block brings it to 126).
 enum Epi { kBias, kBiasRelu, kMask };
 constexpr int kConvW = 32, kConvPitch = 36;   // tile width; floats per staged row (34 used)
 
@@ -850,7 +849,7 @@ float4 f4(const float* a) { return make_float4(a[0], a[1], a[2], a[3]); }
 
 // blocks of the correction's mass sums, 4 to an SM: 2 partials each, then 2 totals and 3
 // FP32 scalars (2 doubles).  With 4096 a thread of the 1024x2048 grid had two sites and the
-// FP64 reduction of the warps was most of the kernel: 38.7 us, DRHO_US now.
+// FP64 reduction of the warps was most of the kernel: 38.7 us, 22 now.
 constexpr int kCorrBlocks = 608;
 constexpr size_t kPartDoubles = 2 * kCorrBlocks + 4;
 

@@ -624,7 +624,7 @@ struct FeatArgs {
 // densities of three rows in a ring in shared memory.  The force and physical velocity are
 // those of the diagnostics, in FP32.  Bound by HBM: 72 bytes read and 24 written per site.
 // A moments pass, a pass over their neighbours and one that packed the planes took 69 us at
-// 1024x2048, FEAT_US now.
+// 1024x2048, 39 now.
 constexpr int kFeatT = 128, kFeatCols = kFeatT - 2, kFeatRows = 16;
 
 __global__ void __launch_bounds__(kFeatT) closure_input_kernel(const float2* __restrict__ fin, FeatArgs a,

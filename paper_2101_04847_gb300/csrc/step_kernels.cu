@@ -489,9 +489,9 @@ step_pipe_kernel(const Cell<T>* __restrict__ fin, Cell<T>* __restrict__ fout, Gr
 //
 // What bounds it: FP32 is limited by HBM (0.97 of the copy rate at 10000x5000, 0.87 at
 // 1024x2048, where the ramp of each 51 us launch shows); 16-bit storage by instruction issue
-// (361 per site with the paired tile below).  Cells of both components halve the loads,
-// stores and address arithmetic (FP32 492 -> 323 instructions per site, paired FP16 500 ->
-// 361), a window of TW + 4 FP32 cells needs no alignment slack (34 sectors read per 32
+// (360 per site with the paired tile below).  Cells of both components halve the loads,
+// stores and address arithmetic (FP32 492 -> 361 instructions per site although its tiles
+// went from 20 rows to 14, paired FP16 500 -> 360 at 16), a window of TW + 4 FP32 cells needs no alignment slack (34 sectors read per 32
 // owned at 128 columns, 36 before), and a tile whose sweep meets no wall row runs code without the wall
 // checks.  us per step before and after: FP32 54.0 -> 51.4 (1024x2048), 1232 -> 1094
 // (10000x5000); FP16 47.3 -> 36.2, 1024 -> 684; BF16 36.9 -> 27.1 (1501x999).
