@@ -21,7 +21,8 @@
 // a tap is then just a 16-byte shift of the operand's start address.  Weights are
 // staged once per CTA in the same layout (N rows of 16 bytes per channel group).
 //
-// Roles: warp 0 lane 0 issues the bulk copies; warp 1 owns the tensor memory (two
+// Roles: warp 0 lane 0 issues the bulk copies (the first layer of a plain inference: warp 0
+// itself reads the FP32 image and writes the rows, stage_image); warp 1 owns the tensor memory (two
 // accumulators of N columns, alternating between input rows) and lane 0 issues the
 // MMAs; warps 2-5 read the accumulators (warp w reads lanes 32 (w mod 4) ... of tensor
 // memory, i.e. pixels 32 (w mod 4) ...), complete one output row per input row, add the
@@ -163,16 +164,82 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
     return *reinterpret_cast<const uint32_t*>(&h);
 }
 
+// The rows of a band from the FP32 image x[4][ny][nx], one warp: pixels rounded to BF16 as
+// they enter the slots (4 channels + 4 zeros, the ghost columns and zero wall rows made
+// here), kAhead rows of loads in flight per lane.  The image is read by plain loads, so
+// its width needs no alignment.  A pass that first wrote the BF16 planes moved 32 more bytes
+// per pixel: the whole inference 695.6 -> 656.5 us at 5000x2500, 134.6 -> 128.4 at 1024x2048,
+// 24.9 at 200x100 both ways.  The warp's loads set the layer's time: 670 us with 3 rows in
+// flight, 664 with 4, 656 with 5 (162 registers, the most for 2 CTAs per SM is 168); 4-byte
+// asynchronous copies through a ring of 8 FP32 rows took 731.  False if a wait gave up.
+constexpr int kAhead = 5;
+constexpr int kLanePx = (kM + 2 + 31) / 32;
+
+// col: the image column of each of the lane's pixels, -1 outside; row: x + (r - 1) nx
+__device__ __forceinline__ void load_image_row(const float* __restrict__ row, bool inside, size_t n,
+                                               const int (&col)[kLanePx], float4 (&v)[kLanePx]) {
+#pragma unroll
+    for (int k = 0; k < kLanePx; ++k) {
+        v[k] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (inside && col[k] >= 0) {
+            const float* q = row + col[k];
+            v[k] = make_float4(__ldg(q), __ldg(q + n), __ldg(q + 2 * n), __ldg(q + 3 * n));
+        }
+    }
+}
+
+__device__ __forceinline__ bool stage_image(const float* __restrict__ x, int nx, int ny, int x0, int y0, int rows_in,
+                                            uint8_t* ring, int slot_bytes, uint64_t* full, uint64_t* empty,
+                                            volatile int* stop, int lane) {
+    const size_t n = (size_t)nx * ny;
+    int col[kLanePx];
+#pragma unroll
+    for (int k = 0; k < kLanePx; ++k) {
+        const int i = lane + 32 * k, p = x0 + i;   // padded column
+        col[k] = i >= kM + 2 || p > nx + 1 ? -1 : (p == 0 ? nx - 1 : (p == nx + 1 ? 0 : p - 1));
+    }
+    float4 v[kAhead][kLanePx];
+    int r = y0 - 1;   // image row of the next loads
+    const float* row = x + (ptrdiff_t)r * nx;
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u, ++r, row += nx) load_image_row(row, r >= 0 && r < ny && u < rows_in, n, col, v[u]);
+    int s = 0;
+    uint32_t parity = 1;   // of the wait for slot s: passes at once in the first trip
+    for (int j0 = 0; j0 < rows_in; j0 += kAhead)
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) {
+            const int j = j0 + u;
+            if (j >= rows_in) break;
+            const bool free = mbar_wait(&empty[s], parity);
+            if (!__all_sync(0xffffffffu, free)) return false;
+            if (__any_sync(0xffffffffu, *stop != 0)) return true;
+            uint8_t* slot = ring + s * slot_bytes + lane * 16;
+#pragma unroll
+            for (int k = 0; k < kLanePx; ++k)
+                if (lane + 32 * k < kM + 2)
+                    *reinterpret_cast<uint4*>(slot + 512 * k) =
+                        make_uint4(pack_bf16(v[u][k].x, v[u][k].y), pack_bf16(v[u][k].z, v[u][k].w), 0u, 0u);
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the row visible to the tensor cores
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&full[s]);
+            load_image_row(row, r >= 0 && r < ny && j + kAhead < rows_in, n, col, v[u]);
+            ++r, row += nx;
+            if (++s == kStages) s = 0, parity ^= 1;
+        }
+    return true;
+}
+
 template <int KG, int NF> constexpr int smem_bytes() { return kHead + wbytes(KG, NF) + kStages * KG * kPlane; }
 
 // One 3x3 convolution layer.  KGG channel groups of 8 are read per input row
 // (KG >= KGG groups in shared memory, the extra ones zero: the first layer has 4
 // channels, padded to one group of 8 in memory and to K = 16 in the MMA).  W
 // output channels per row tap.  HIDDEN: bias + ReLU, BF16 activation planes out;
-// else bias, 4 channels as FP32 planes y[4][ny][nx].
-template <int KGG, int KG, int W, bool HIDDEN>
+// else bias, 4 channels as FP32 planes y[4][ny][nx].  IMAGE: the input is the FP32
+// image x[4][ny][nx] itself (in unused), else BF16 planes (x unused).
+template <int KGG, int KG, int W, bool HIDDEN, bool IMAGE>
 __global__ void __launch_bounds__(kThreads, 2)
-conv_tc_kernel(const uint8_t* __restrict__ in, const uint8_t* __restrict__ wop, const float* __restrict__ bias,
+conv_tc_kernel(const uint8_t* __restrict__ in, const float* __restrict__ x, const uint8_t* __restrict__ wop, const float* __restrict__ bias,
                uint8_t* __restrict__ hout, float* __restrict__ yout, int nx, int ny, int pitch, int rows_per_cta,
                int* __restrict__ status, int withhold) {
     // withhold != 0 (tests of the timeout path only): no copies are issued and every
@@ -231,7 +298,19 @@ conv_tc_kernel(const uint8_t* __restrict__ in, const uint8_t* __restrict__ wop, 
     tc_fence_after();
     const uint32_t tmem = *tslot;
 
-    if (warp == 0 && lane == 0 && R > 0 && !withhold) {
+    static_assert(!IMAGE || KGG == 1, "an image has one channel group");
+    if (IMAGE && warp == 0 && R > 0 && !withhold) {
+        // ---- producer: weights once, then the rows of the band from the image
+        if (lane == 0) {
+            mbar_expect_tx(wbar, WB);
+            bulk_g2s(wsm, wop, WB, wbar);
+        }
+        if (!stage_image(x, nx, ny, x0, y0, rows_in, ring, SLOT, full, empty, stop, lane) && lane == 0) {
+            *stop = 1;
+            atomicOr(status, 1);
+        }
+        if (lane == 0) mbar_wait(wbar, 0);
+    } else if (!IMAGE && warp == 0 && lane == 0 && R > 0 && !withhold) {
         // ---- producer: weights once, then the input rows of the band
         mbar_expect_tx(wbar, WB);
         bulk_g2s(wsm, wop, WB, wbar);
@@ -290,7 +369,7 @@ conv_tc_kernel(const uint8_t* __restrict__ in, const uint8_t* __restrict__ wop, 
         constexpr int L = HIDDEN ? W : kOut;   // channels read back per row tap
         const int q = warp & 3;
         const int m = q * 32 + lane;
-        const int x = x0 + m;
+        const int px = x0 + m;
         float T1[L], T2[L], O[L];
 #pragma unroll
         for (int n = 0; n < L; ++n) T1[n] = T2[n] = 0.0f;
@@ -326,7 +405,7 @@ conv_tc_kernel(const uint8_t* __restrict__ in, const uint8_t* __restrict__ wop, 
             __syncwarp();
             if (lane == 0) mbar_arrive(&acce[j & 1]);
             const int y = y0 + j - 2;
-            if (j >= 2 && x < nx) {
+            if (j >= 2 && px < nx) {
                 if constexpr (HIDDEN) {
                     uint32_t pk[L / 2];
 #pragma unroll
@@ -340,14 +419,14 @@ conv_tc_kernel(const uint8_t* __restrict__ in, const uint8_t* __restrict__ wop, 
                     for (int g = 0; g < 4; ++g) {
                         const uint4 val = make_uint4(pk[4 * g], pk[4 * g + 1], pk[4 * g + 2], pk[4 * g + 3]);
                         uint8_t* plane = hout + (row + (size_t)g * pitch) * 16;
-                        *reinterpret_cast<uint4*>(plane + (size_t)(x + 1) * 16) = val;
-                        if (x == 0) *reinterpret_cast<uint4*>(plane + (size_t)(nx + 1) * 16) = val;
-                        if (x == nx - 1) *reinterpret_cast<uint4*>(plane) = val;
+                        *reinterpret_cast<uint4*>(plane + (size_t)(px + 1) * 16) = val;
+                        if (px == 0) *reinterpret_cast<uint4*>(plane + (size_t)(nx + 1) * 16) = val;
+                        if (px == nx - 1) *reinterpret_cast<uint4*>(plane) = val;
                     }
                 } else {
                     const size_t n = (size_t)nx * ny;
 #pragma unroll
-                    for (int c = 0; c < kOut; ++c) yout[(size_t)c * n + (size_t)y * nx + x] = O[c] + bsm[c];
+                    for (int c = 0; c < kOut; ++c) yout[(size_t)c * n + (size_t)y * nx + px] = O[c] + bsm[c];
                 }
             }
         }
@@ -379,12 +458,10 @@ __device__ __forceinline__ void operand_weight(const float* __restrict__ w, int 
 }
 
 // All that the layers start from, in one launch: the weights of the three layers in
-// operand layout, the input planes (4 channels + 4 zeros, ghost columns, zero wall rows;
-// x null: only the zero wall rows, the caller fills the others), the wall rows of the hidden planes, and (clear != 0)
-// the status word.
-__global__ void prep_kernel(const float* __restrict__ params, const float* __restrict__ x, Bufs B, int clear) {
-    const int nx = B.nx, ny = B.ny, pitch = B.pitch;
-    const size_t n = (size_t)nx * ny;
+// operand layout, the zero wall rows of the input and hidden planes, and (clear != 0) the
+// status word.
+__global__ void prep_kernel(const float* __restrict__ params, Bufs B, int clear) {
+    const int ny = B.ny, pitch = B.pitch;
     const size_t first = blockIdx.x * (size_t)blockDim.x + threadIdx.x, step = (size_t)gridDim.x * blockDim.x;
     if (clear && first == 0) *B.status = 0;
     constexpr int n1 = wbytes(2, nfold(kHid)) / 2, n2 = wbytes(4, nfold(kHid)) / 2, n3 = wbytes(4, nfold(kOut)) / 2;
@@ -400,31 +477,16 @@ __global__ void prep_kernel(const float* __restrict__ params, const float* __res
         reinterpret_cast<uint4*>(B.h1)[o] = z;
         reinterpret_cast<uint4*>(B.h2)[o] = z;
     }
-    if (!x) {
-        for (size_t i = first; i < (size_t)2 * pitch; i += step)
-            reinterpret_cast<uint4*>(B.xin)[i < pitch ? i : (size_t)(ny + 1) * pitch + (i - pitch)] = z;
-        return;
-    }
-    const size_t total = (size_t)(ny + 2) * pitch;
-    for (size_t i = first; i < total; i += step) {
-        const int r = (int)(i / pitch), p = (int)(i % pitch);
-        uint4 val = z;
-        if (r >= 1 && r <= ny && p <= nx + 1) {
-            const int xa = p == 0 ? nx - 1 : (p == nx + 1 ? 0 : p - 1);
-            const size_t k = (size_t)(r - 1) * nx + xa;
-            val.x = pack_bf16(x[k], x[n + k]);
-            val.y = pack_bf16(x[2 * n + k], x[3 * n + k]);
-        }
-        reinterpret_cast<uint4*>(B.xin)[i] = val;
-    }
+    for (size_t i = first; i < (size_t)2 * pitch; i += step)
+        reinterpret_cast<uint4*>(B.xin)[i < pitch ? i : (size_t)(ny + 1) * pitch + (i - pitch)] = z;
 }
 
 // Bands of rows so that all CTAs of a layer are resident at once.
-template <int KGG, int KG, int W, bool HIDDEN>
-cudaError_t launch_conv(const Bufs& B, const uint8_t* in, const uint8_t* w, const float* bias, uint8_t* hout,
+template <int KGG, int KG, int W, bool HIDDEN, bool IMAGE = false>
+cudaError_t launch_conv(const Bufs& B, const uint8_t* in, const float* x, const uint8_t* w, const float* bias, uint8_t* hout,
                         float* yout, cudaStream_t st, int withhold) {
     constexpr int SM = smem_bytes<KG, nfold(W)>();
-    auto kern = conv_tc_kernel<KGG, KG, W, HIDDEN>;
+    auto kern = conv_tc_kernel<KGG, KG, W, HIDDEN, IMAGE>;
     static bool configured = false;
     static int per_sm = 1, sms = 1;
     if (!configured) {
@@ -453,8 +515,8 @@ cudaError_t launch_conv(const Bufs& B, const uint8_t* in, const uint8_t* w, cons
     int groups = std::max(1, slots / B.tiles_x);
     int rows = std::max(1, (B.ny + groups - 1) / groups);
     groups = (B.ny + rows - 1) / rows;
-    conv_tc_kernel<KGG, KG, W, HIDDEN><<<dim3(B.tiles_x, groups), kThreads, SM, st>>>(
-        in, w, bias, hout, yout, B.nx, B.ny, B.pitch, rows, B.status, withhold);
+    conv_tc_kernel<KGG, KG, W, HIDDEN, IMAGE><<<dim3(B.tiles_x, groups), kThreads, SM, st>>>(
+        in, x, w, bias, hout, yout, B.nx, B.ny, B.pitch, rows, B.status, withhold);
     return cudaGetLastError();
 }
 
@@ -489,16 +551,16 @@ Bufs carve(void* base, int nx, int ny) {
 cudaError_t infer(const Bufs& B, const float* params, const float* x, float* y, cudaStream_t st, bool withhold,
                   bool clear_status) {
     const int wh = withhold ? 1 : 0;
-    const size_t px = x ? (size_t)(B.ny + 2) * B.pitch : (size_t)8 * B.pitch;
-    const int blocks = (int)std::min<size_t>(4096, std::max<size_t>((px + 255) / 256, 60));
-    prep_kernel<<<blocks, 256, 0, st>>>(params, x, B, clear_status ? 1 : 0);
+    const int blocks = (int)std::min<size_t>(4096, std::max<size_t>(((size_t)8 * B.pitch + 255) / 256, 60));
+    prep_kernel<<<blocks, 256, 0, st>>>(params, B, clear_status ? 1 : 0);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    e = launch_conv<1, 2, 32, true>(B, B.xin, B.w1, params + kB1, B.h1, nullptr, st, wh);
+    e = x ? launch_conv<1, 2, 32, true, true>(B, nullptr, x, B.w1, params + kB1, B.h1, nullptr, st, wh)
+          : launch_conv<1, 2, 32, true>(B, B.xin, nullptr, B.w1, params + kB1, B.h1, nullptr, st, wh);
     if (e != cudaSuccess) return e;
-    e = launch_conv<4, 4, 32, true>(B, B.h1, B.w2, params + kB2, B.h2, nullptr, st, wh);
+    e = launch_conv<4, 4, 32, true>(B, B.h1, nullptr, B.w2, params + kB2, B.h2, nullptr, st, wh);
     if (e != cudaSuccess) return e;
-    return launch_conv<4, 4, kOut, false>(B, B.h2, B.w3, params + kB3, nullptr, y, st, wh);
+    return launch_conv<4, 4, kOut, false>(B, B.h2, nullptr, B.w3, params + kB3, nullptr, y, st, wh);
 }
 
 cudaError_t status(const Bufs& B, cudaStream_t st, int* out) {

@@ -18,7 +18,7 @@ namespace cnn_tc {
 //   byte offset of (padded row r, group g, padded column p) = ((r * G + g) * pitch + p) * 16.
 struct Bufs {
     int nx = 0, ny = 0, tiles_x = 0, pitch = 0;
-    uint8_t* xin = nullptr;   // G = 1: the 4 input channels + 4 zero channels
+    uint8_t* xin = nullptr;   // G = 1: the 4 input channels + 4 zero channels (x null only)
     uint8_t* h1 = nullptr;    // G = 4: 32 hidden channels after the first ReLU
     uint8_t* h2 = nullptr;    // G = 4: after the second ReLU
     uint8_t* w1 = nullptr;    // weights in the tensor cores' shared-memory operand layout
