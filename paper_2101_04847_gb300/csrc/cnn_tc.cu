@@ -481,7 +481,28 @@ __global__ void prep_kernel(const float* __restrict__ params, Bufs B, int clear)
         reinterpret_cast<uint4*>(B.xin)[i < pitch ? i : (size_t)(ny + 1) * pitch + (i - pitch)] = z;
 }
 
-// Bands of rows so that all CTAs of a layer are resident at once.
+// Bands of rows for 1 to 4 waves of resident CTAs, by the rows that a slot sweeps: a band
+// reads two rows beside its own and costs about kBandRows more to start (weights, zeroed
+// ring, tensor memory).  One wave of 40 strips leaves 24 of 304 slots empty, two waves 8 of 608:
+// inference at 5000x2500 652.5 -> 645.2 us with two waves; at 1024x2048 one wave fills
+// the slots, 128.4 us, and two take 138.8.
+constexpr int kBandRows = 8;
+int band_rows(int ny, int tiles_x, int slots) {
+    int best = ny;
+    long long best_cost = -1;
+    for (int w = 1; w <= 4; ++w) {
+        const int groups = std::max(1, (int)((long long)w * slots / tiles_x));
+        const int rows = std::max(1, (ny + groups - 1) / groups);
+        const long long tiles = (long long)((ny + rows - 1) / rows) * tiles_x;
+        const long long cost = (tiles + slots - 1) / slots * (rows + 2 + kBandRows);
+        if (best_cost < 0 || cost < best_cost) {
+            best_cost = cost;
+            best = rows;
+        }
+    }
+    return best;
+}
+
 template <int KGG, int KG, int W, bool HIDDEN, bool IMAGE = false>
 cudaError_t launch_conv(const Bufs& B, const uint8_t* in, const float* x, const uint8_t* w, const float* bias, uint8_t* hout,
                         float* yout, cudaStream_t st, int withhold) {
@@ -511,10 +532,8 @@ cudaError_t launch_conv(const Bufs& B, const uint8_t* in, const float* x, const 
         per_sm = std::max(1, per_sm);
         configured = true;
     }
-    const int slots = sms * per_sm;
-    int groups = std::max(1, slots / B.tiles_x);
-    int rows = std::max(1, (B.ny + groups - 1) / groups);
-    groups = (B.ny + rows - 1) / rows;
+    const int rows = band_rows(B.ny, B.tiles_x, sms * per_sm);
+    const int groups = (B.ny + rows - 1) / rows;
     conv_tc_kernel<KGG, KG, W, HIDDEN, IMAGE><<<dim3(B.tiles_x, groups), kThreads, SM, st>>>(
         in, x, w, bias, hout, yout, B.nx, B.ny, B.pitch, rows, B.status, withhold);
     return cudaGetLastError();
