@@ -335,7 +335,8 @@ void lbm_ens_destroy(lbm_ensemble* e);
  * w2[32][32][3][3], b2[32], w3[4][32][3][3], b3[4]. ---- */
 #define LBM_CNN_PARAMS 11588
 
-/* Device workspace for the CNN calls on an nx x ny image. */
+/* Device workspace for the CNN calls on an nx x ny image: so many bytes at any address
+ * (the calls align their buffers within it). */
 lbm_status lbm_cnn_workspace_bytes(int32_t nx, int32_t ny, size_t* bytes);
 
 /* y = CNN(x); all pointers device (x, y: 4*ny*nx floats). Asynchronous. */

@@ -434,7 +434,11 @@ size_t training_bytes(int nx, int ny) {
     return b;
 }
 
-size_t workspace_bytes(int nx, int ny) { return training_bytes(nx, ny) + cnn_tc::bytes(nx, ny); }
+// The kernels read the workspace in accesses of up to 16 bytes and by bulk copies; the
+// caller's pointer may have any alignment, so the buffers start at its next multiple of
+// 256 bytes.
+constexpr size_t kWorkspaceSlack = 255;
+size_t workspace_bytes(int nx, int ny) { return training_bytes(nx, ny) + cnn_tc::bytes(nx, ny) + kWorkspaceSlack; }
 
 Net carve(void* ws, int nx, int ny) {
     Net N;
@@ -442,7 +446,8 @@ Net carve(void* ws, int nx, int ny) {
     N.ny = ny;
     N.n = (size_t)nx * ny;
     N.P = (int)grad_parts(nx, ny);
-    char* p = (char*)ws;
+    char* const base = (char*)align256((size_t)ws);
+    char* p = base;
     N.w = (float*)p; p += align256(kConvWeights * sizeof(float));
     N.a1 = (float*)p; p += align256(kHid * N.n * 4);
     N.a2 = (float*)p; p += align256(kHid * N.n * 4);
@@ -452,7 +457,7 @@ Net carve(void* ws, int nx, int ny) {
     N.dz1 = (float*)p; p += align256(kHid * N.n * 4);
     N.part = (float*)p; p += align256((size_t)N.P * kPartFloats * 4);
     N.lpart = (double*)p;
-    N.tc = cnn_tc::carve((char*)ws + training_bytes(nx, ny), nx, ny);
+    N.tc = cnn_tc::carve(base + training_bytes(nx, ny), nx, ny);
     return N;
 }
 
