@@ -287,7 +287,7 @@ struct Acc2 {
 // takes the moments of row m (from the stored populations), the velocity of row m - 1 and
 // the terms of row m - 2; densities and velocities are exchanged through rings in shared
 // memory.  Row sums of phi and the mass fraction are taken kRowBatch rows at a time, 16
-// threads to a row.
+// threads to a row: 8 columns each in double-float, then FP64.
 //
 // Bound by issue: about 1.7 k mostly packed FP32 instructions per site against 72 bytes
 // read.  The four passes it replaces stored 15 dfl per site, read them again with their
@@ -346,16 +346,16 @@ diag_sweep_kernel(const Cell<T>* __restrict__ fin, DiagArgs a, float2 shift) {
 #pragma unroll 1
             for (int k = 1; k < kSweepT / 16; ++k) v = v + dfl2_of(sm.rows[r][l + 16 * k]);
             const unsigned mask = (t & 16) ? 0xffff0000u : 0x0000ffffu;
+            double phi = to_d(first(v)), c = to_d(second(v));   // 8 columns' sums; FP64 from here on
 #pragma unroll
             for (int o = 8; o > 0; o >>= 1) {
-                const dfl2 w = {make_float2(__shfl_down_sync(mask, v.hi.x, o, 16), __shfl_down_sync(mask, v.hi.y, o, 16)),
-                                make_float2(__shfl_down_sync(mask, v.lo.x, o, 16), __shfl_down_sync(mask, v.lo.y, o, 16))};
-                v = v + w;
+                phi += __shfl_down_sync(mask, phi, o, 16);
+                c += __shfl_down_sync(mask, c, o, 16);
             }
             if (l == 0) {
                 const size_t k = (size_t)(last - batched + 1 + r) * a.nbx + blockIdx.x;
-                a.rowpart[k] = to_d(first(v));
-                a.rowpart_c[k] = to_d(second(v));
+                a.rowpart[k] = phi;
+                a.rowpart_c[k] = c;
             }
         }
         batched = 0;

@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 GRIDS = [(97, 60), (124, 48), (64, 90), (130, 71), (33, 120), (200, 40), (77, 77), (150, 33)]
 
 
-def seeded_flow(seed, nx, ny):
+def seeded_flow(seed, nx, ny, minority=0.08):
     """FP32 equilibrium populations of a tanh interface in a field of vortices with speeds up
     to 0.02."""
     rng = np.random.default_rng(seed)
@@ -22,7 +22,7 @@ def seeded_flow(seed, nx, ny):
     for kx, ky, a, p in zip(rng.integers(1, 4, 4), rng.integers(1, 4, 4), rng.uniform(-0.01, 0.01, 4), rng.uniform(0, 6, 4)):
         ux += a * np.cos(2 * np.pi * kx * x / nx + p) * np.cos(np.pi * ky * y / ny)
         uy += a * np.sin(2 * np.pi * kx * x / nx + p) * np.sin(np.pi * ky * y / ny)
-    rho = (1.0 * (0.08 + 0.92 * H), 0.9 * (0.08 + 0.92 * (1 - H)))
+    rho = (1.0 * (minority + (1 - minority) * H), 0.9 * (minority + (1 - minority) * (1 - H)))
     return np.stack([O.equilibrium(r, ux, uy) for r in rho]).astype(np.float32)
 
 
@@ -72,3 +72,28 @@ def test_terms_are_as_accurate_as_the_fields(samples, term):
         return float(np.sqrt(np.mean([((s[k][term] - s[2][term]) / s[2][term]) ** 2 for s in samples])))
 
     assert rms(0) <= rms(3) + 2.0 ** -50, (rms(0), rms(3))
+
+
+# A row's phi are added in double-float by 16 threads, 8 columns each, and in FP64 from
+# there on.  The low part of a double-float sum S lies evenly within 2^-25 |S|, so its two
+# roundings in an addition have a standard deviation of about 0.15 * 2^-48 |S|; over
+# partial sums of 2 .. 8 values of size 1 that makes 2.2 * 2^-48 per thread, 8.8 * 2^-48
+# over 16 threads and 2^-51.8 in the mean of a block's 124 columns.  With double-float
+# partial sums of up to 124 values it is 2^-50.4.  Allowed: 2^-51 beside the error of the
+# densities, which the extracted fields carry too.
+def test_row_means_are_as_accurate_as_the_fields(gpu):
+    errors = []
+    for k in range(24):
+        d = inputs.params(inputs.C0, nx=124, ny=64, g=1e-4, crop_rows=5, G=0.0, minority=0.0)
+        f = seeded_flow(100 + k, 124, 64, minority=0.0)
+        p = O.Params(**{q: v for q, v in d.items() if q in O.Params.__dataclass_fields__})
+        with lbm.Solver(**d) as s:
+            s.set_populations(f)
+            s.diagnostics()
+            rows, fld = s.profile(), s.fields()
+        A, B = extended_fields(f, p)[:2]
+        means = [np.mean((a - b)[5:-5], axis=1, dtype=np.longdouble)
+                 for a, b in ((A, B), (fld["rhoA"].astype(np.longdouble), fld["rhoB"].astype(np.longdouble)))]
+        errors.append((rows - means[0], means[1] - means[0]))
+    sweep, fields = (float(np.sqrt(np.mean(np.square([e[q] for e in errors])))) for q in range(2))
+    assert sweep <= fields + 2.0 ** -51, (sweep, fields)
