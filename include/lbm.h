@@ -316,9 +316,12 @@ lbm_status lbm_ens_diagnostics(lbm_ensemble* e, lbm_diag* out);
 
 /* Pick the tile shape for the whole ensemble by timing candidates: the three tile
  * widths of lbm_params.tile_x (128, 256, 0 = paired 16-bit tiles) times tile heights
- * (0, the default but at least 12 rows, among them); states are kept.  tile_y receives the
- * rows per tile in use.  The initial width is the first member's tile_x when it is
- * 128 or 256, else 0. */
+ * from 12 rows on (0, the default, among them where it has that many); states are kept.
+ * The shape that the ensemble had stays where no candidate is faster (the default of small
+ * grids has fewer rows).  tile_y receives the rows per tile in use, or where these are
+ * fewer than 12 those of the fastest candidate; ms_per_step the time of a step with the
+ * shape in use.  The initial width is the first member's tile_x when it is 128 or 256,
+ * else 0. */
 lbm_status lbm_ens_tune(lbm_ensemble* e, int32_t* tile_y, double* ms_per_step);
 
 /* Tile width of the ensemble's launch: 128, 256 or 0 (see lbm_params.tile_x). */

@@ -18,7 +18,7 @@ namespace {
 
 constexpr int kEnsGraphChunk = 50;
 constexpr int kEnsMaxMembers = 256;
-constexpr int kTuneMinRows = 12;   // shortest tile that lbm_ens_tune picks
+constexpr int kTuneMinRows = 12;   // shortest tile that lbm_ens_tune tries itself
 
 lbm_status ens_fail(lbm_status st, const std::string& msg) {
     lbm::set_last_error(msg);
@@ -52,7 +52,6 @@ struct lbm_ensemble {
     int tile_x = lbm::kEnsAuto;      // 128 or 256 columns per tile (one per thread), or kEnsAuto
     int tile_y = 0;       // requested rows per tile; 0: chosen from the device's block slots
     int rows = 0;         // rows per tile in use
-    int min_rows = 1;     // at least so many rows when chosen (the tuner's shapes: kTuneMinRows)
     int parity = 0;
     int64_t step = 0;
     cudaStream_t stream = nullptr;
@@ -85,10 +84,9 @@ int tiles_of(const lbm::Grid& g, int tile_x, int rows, int* tx, int* ty) {
 // beyond that two rows are the least that pay (eight 128x256 members 14.5 with 1, 10.2).
 constexpr int kMaxAutoRows = 48;
 constexpr int kWideRows = 16;     // FP32 tiles of so many rows are 256 columns wide
-int auto_rows(double waves_of_one_row, int min_rows) {
-    if (waves_of_one_row <= 1.0) return min_rows;
-    const int rows = (int)std::ceil(std::min(waves_of_one_row / 2.0, (double)kMaxAutoRows));
-    return std::max({2, rows, min_rows});
+int auto_rows(double waves_of_one_row) {
+    if (waves_of_one_row <= 1.0) return 1;
+    return std::max(2, (int)std::ceil(std::min(waves_of_one_row / 2.0, (double)kMaxAutoRows)));
 }
 
 // The chains of an ensemble: its members by storage type, each type's in up to
@@ -141,7 +139,7 @@ lbm_status ens_build_table(lbm_ensemble* e) {
         ENS_TRY(lbm::ensemble_slots(c.kernel, &slots), "ensemble occupancy");
         for (lbm_handle* h : c.members) waves += (double)tiles_of(lbm::handle_grid(h), c.kernel.cols, 1, &tx, &ty) / slots;
     }
-    e->rows = e->tile_y > 0 ? e->tile_y : auto_rows(waves, e->min_rows);
+    e->rows = e->tile_y > 0 ? e->tile_y : auto_rows(waves);
     for (EnsChain& c : e->chains) {
         // tall FP32 tiles: 256 columns, as on one grid (ten 1024x2048 members 486 -> 461 us a
         // step, sixteen 512x1024 209 -> 192; short ones lose, eight 128x256 10 -> 13)
@@ -202,23 +200,56 @@ lbm_status ens_launch(lbm_ensemble* e, int64_t n) {
     return LBM_OK;
 }
 
+// n steps from the given parity as a graph.
+lbm_status ens_capture(lbm_ensemble* e, int parity, int n, cudaGraphExec_t* out) {
+    cudaGraph_t g = nullptr;
+    ENS_TRY(cudaStreamBeginCapture(e->stream, cudaStreamCaptureModeThreadLocal), "begin capture");
+    cudaError_t err = ens_launch_steps(e, parity, n);
+    const cudaError_t end = cudaStreamEndCapture(e->stream, &g);
+    if (err == cudaSuccess) err = end;
+    if (err != cudaSuccess) {
+        if (g) cudaGraphDestroy(g);
+        return ens_fail(LBM_ECUDA, std::string("capture ensemble step: ") + cudaGetErrorString(err));
+    }
+    err = cudaGraphInstantiate(out, g, 0);
+    cudaGraphDestroy(g);
+    if (err != cudaSuccess) return ens_fail(LBM_ECUDA, std::string("instantiate: ") + cudaGetErrorString(err));
+    return LBM_OK;
+}
+
 lbm_status ens_graph(lbm_ensemble* e, cudaGraphExec_t* out) {
     const int par = e->parity;
     if (!e->graph[par]) {
-        cudaGraph_t g = nullptr;
-        ENS_TRY(cudaStreamBeginCapture(e->stream, cudaStreamCaptureModeThreadLocal), "begin capture");
-        cudaError_t err = ens_launch_steps(e, par, kEnsGraphChunk);
-        const cudaError_t end = cudaStreamEndCapture(e->stream, &g);
-        if (err == cudaSuccess) err = end;
-        if (err != cudaSuccess) {
-            if (g) cudaGraphDestroy(g);
-            return ens_fail(LBM_ECUDA, std::string("capture ensemble step: ") + cudaGetErrorString(err));
-        }
-        err = cudaGraphInstantiate(&e->graph[par], g, 0);
-        cudaGraphDestroy(g);
-        if (err != cudaSuccess) return ens_fail(LBM_ECUDA, std::string("instantiate: ") + cudaGetErrorString(err));
+        const lbm_status st = ens_capture(e, par, kEnsGraphChunk, &e->graph[par]);
+        if (st != LBM_OK) return st;
     }
     *out = e->graph[par];
+    return LBM_OK;
+}
+
+// ms per step with the tile shape in use, by events a and b around replays of a graph of
+// kTuneSteps steps (single launches would time the host where a step takes a few us); more
+// replays where they are short, 32 steps in all at most.  The parity, an even number of
+// steps on, is the same; the members' states have to be restored.
+constexpr int kTuneSteps = 4;
+lbm_status ens_time(lbm_ensemble* e, cudaEvent_t a, cudaEvent_t b, double* ms_per_step) {
+    cudaGraphExec_t g = nullptr;
+    const lbm_status st = ens_capture(e, e->parity, kTuneSteps, &g);
+    if (st != LBM_OK) return st;
+    cudaError_t err = cudaGraphLaunch(g, e->stream);
+    float ms = 0.0f;
+    for (int replays : {1, 6}) {
+        if (err == cudaSuccess) err = cudaEventRecord(a, e->stream);
+        for (int k = 0; k < replays && err == cudaSuccess; ++k) err = cudaGraphLaunch(g, e->stream);
+        if (err == cudaSuccess) err = cudaEventRecord(b, e->stream);
+        if (err == cudaSuccess) err = cudaEventSynchronize(b);
+        if (err == cudaSuccess) err = cudaEventElapsedTime(&ms, a, b);
+        if (err != cudaSuccess) break;
+        *ms_per_step = ms / (replays * kTuneSteps);
+        if (ms > 1.0f) break;
+    }
+    cudaGraphExecDestroy(g);
+    if (err != cudaSuccess) return ens_fail(LBM_ECUDA, std::string("timing: ") + cudaGetErrorString(err));
     return LBM_OK;
 }
 
@@ -340,53 +371,64 @@ lbm_status lbm_ens_diagnostics(lbm_ensemble* e, lbm_diag* out) {
 
 lbm_status lbm_ens_tune(lbm_ensemble* e, int32_t* tile_y_out, double* ms_out) {
     if (!e) return ens_fail(LBM_EINVAL, "ensemble is NULL");
-    e->min_rows = kTuneMinRows;
-    const int cand[] = {0, 12, 16, 20, 24, 32, 48, 64, 96};   // 0: the default
+    const int cand[] = {0, 12, 16, 20, 24, 32, 48, 64, 96};   // 0: the default where it is no shorter
     const int widths[] = {lbm::kEnsAuto, lbm::kBlockTileW, lbm::kWideTileW};
+    static_assert(kTuneMinRows == 12, "the shortest candidate");
     cudaEvent_t a, b;
     ENS_TRY(cudaEventCreate(&a), "event");
     ENS_TRY(cudaEventCreate(&b), "event");
-    for (lbm_handle* h : e->members) ENS_TRY(lbm::handle_save_state(h), "save state");
-    const int par0 = e->parity;
-    double best_ms = 1e30;
-    int best_ty = e->tile_y, best_tx = e->tile_x;
-    for (int tx : widths)
-    for (int ty : cand) {
+    // the shape found: it stays where no candidate is faster, and after an error (eight
+    // 128x256 members keep their 2 rows and 9.9 us a step; 15.9 with 12 rows)
+    const int found_tx = e->tile_x, found_ty = e->tile_y;
+    auto shape = [&](int tx, int ty) {
         e->tile_x = tx;
         e->tile_y = ty;
-        lbm_status st = ens_build_table(e);
-        const int reps = 6;
-        if (st == LBM_OK) st = ens_launch(e, 2);
-        if (st == LBM_OK) {
-            cudaEventRecord(a, e->stream);
-            st = ens_launch(e, reps);
-            cudaEventRecord(b, e->stream);
-        }
-        if (st != LBM_OK) {
-            cudaEventDestroy(a);
-            cudaEventDestroy(b);
-            return st;
-        }
-        ENS_TRY(cudaEventSynchronize(b), "sync");
-        float ms = 0.0f;
-        cudaEventElapsedTime(&ms, a, b);
-        e->parity = par0;   // 8 steps: back on the same buffer; restore its contents
+        return ens_build_table(e);
+    };
+    auto timed = [&](double* ms) {
+        const lbm_status st = ens_time(e, a, b, ms);
         for (lbm_handle* h : e->members) ENS_TRY(lbm::handle_restore_state(h), "restore state");
-        if (ms / reps < best_ms) {
-            best_ms = ms / reps;
-            best_ty = ty;
-            best_tx = tx;
-        }
+        return st;
+    };
+    auto tune = [&]() -> lbm_status {
+        for (lbm_handle* h : e->members) ENS_TRY(lbm::handle_save_state(h), "save state");
+        double found_ms = 0.0, best_ms = 1e30;
+        lbm_status st = timed(&found_ms);
+        if (st != LBM_OK) return st;
+        int best_tx = found_tx, best_ty = found_ty, best_rows = 0;
+        for (int tx : widths)
+            for (int ty : cand) {
+                if ((st = shape(tx, ty)) != LBM_OK) return st;
+                if (e->rows < kTuneMinRows) continue;
+                double ms = 0.0;
+                if ((st = timed(&ms)) != LBM_OK) return st;
+                if (ms < best_ms) {
+                    best_ms = ms;
+                    best_tx = tx;
+                    best_ty = ty;
+                    best_rows = e->rows;
+                }
+            }
+        // the least of many noisy timings is below what it stands for: both once more
+        double again_ms = 0.0;
+        if ((st = shape(found_tx, found_ty)) != LBM_OK || (st = timed(&again_ms)) != LBM_OK) return st;
+        found_ms = std::min(found_ms, again_ms);
+        if ((st = shape(best_tx, best_ty)) != LBM_OK || (st = timed(&best_ms)) != LBM_OK) return st;
+        const bool faster = best_ms < found_ms;
+        if (!faster && (st = shape(found_tx, found_ty)) != LBM_OK) return st;
+        if (tile_y_out) *tile_y_out = e->rows >= kTuneMinRows ? e->rows : best_rows;
+        if (ms_out) *ms_out = faster ? best_ms : found_ms;
+        return LBM_OK;
+    };
+    lbm_status st = tune();
+    if (st != LBM_OK) {
+        const std::string msg = lbm_last_error();
+        shape(found_tx, found_ty);
+        lbm::set_last_error(msg);
     }
     cudaEventDestroy(a);
     cudaEventDestroy(b);
-    e->tile_x = best_tx;
-    e->tile_y = best_ty;
-    lbm_status st = ens_build_table(e);
-    if (st != LBM_OK) return st;
-    if (tile_y_out) *tile_y_out = e->rows;
-    if (ms_out) *ms_out = best_ms;
-    return LBM_OK;
+    return st;
 }
 
 lbm_status lbm_ens_tile_width(lbm_ensemble* e, int32_t* tile_x) {
