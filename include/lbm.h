@@ -280,9 +280,9 @@ void lbm_destroy(lbm_handle* h);
  * values (0 = the default among them) on the handle's own grid, then use the
  * fastest; lbm_get_params reports both.  The state and the step counter are left as
  * they were.  cache_path: NULL, or a text file of
- * "<gpu>|<kernel>|<storage>|<nx>x<ny> <tile_x> <tile_y> <ms>" lines; a matching line
- * is used without timing, a new result is appended (lines of another form are
- * skipped).  Outputs may be NULL. */
+ * "<gpu>|<kernel>|<storage>|<nx>x<ny>|r<revision> <tile_x> <tile_y> <ms>" lines; a
+ * matching line is used without timing, a new result is appended (lines of another form,
+ * or written for another revision of the kernels, are skipped).  Outputs may be NULL. */
 lbm_status lbm_tune(lbm_handle* h, const char* cache_path, int32_t* tile_y, double* ms_per_step);
 
 /* The handle's parameters as in use (tile_x / tile_y after lbm_tune). */

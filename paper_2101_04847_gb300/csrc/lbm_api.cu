@@ -383,13 +383,18 @@ cudaError_t handle_clear_guard(lbm_handle* h) {
 
 namespace {
 
+// Revision of the step kernels' tiles, part of the key: a tile height cached for other
+// kernels would be kept unmeasured, and can be far from the best of these (128x256 FP32
+// takes 3.6 us a step with its default of one row, 12.9 with 12).
+constexpr int kTileRevision = 2;
+
 std::string tune_key(const lbm_handle* h) {
     cudaDeviceProp prop;
     std::string dev = cudaGetDeviceProperties(&prop, h->device) == cudaSuccess ? prop.name : "unknown";
     for (char& c : dev)
         if (c == ' ') c = '_';
     return dev + "|" + std::to_string(h->p.kernel) + "|" + std::to_string(h->p.storage) + "|" +
-           std::to_string(h->p.nx) + "x" + std::to_string(h->p.ny);
+           std::to_string(h->p.nx) + "x" + std::to_string(h->p.ny) + "|r" + std::to_string(kTileRevision);
 }
 
 // "<key> <tile_x> <tile_y> <ms>" lines; the last match wins, lines of another form
