@@ -346,7 +346,8 @@ __global__ void __launch_bounds__(32 * kReduceWays) reduce_grad_kernel(const flo
             s = t;
         }
     }
-    red[g][lane] = (double)s + (double)e;
+    // an infinite sum (e is not a number then) stays what it is
+    red[g][lane] = isfinite(s) ? (double)s + (double)e : (double)s;
     __syncthreads();
     if (g == 0 && i < nw + nb) {
         double v = 0.0;
