@@ -713,20 +713,21 @@ __device__ __forceinline__ void correct_site(float2 f[9], float4 p, int mode, fl
         d[1] -= mB;
     }
     const float du2 = 1.5f * ((vx * vx + vy * vy) - (ux * ux + uy * uy));
-    // an absent component keeps its populations: q = 1, r1 = 0
     float q[2], r1[2];
 #pragma unroll
     for (int s = 0; s < 2; ++s) {
-        const bool present = rho[s] > 0.0f;
-        r1[s] = present ? fmaxf(rho[s] + d[s], 0.0f) : 0.0f;
-        q[s] = present ? r1[s] / rho[s] : 1.0f;
+        r1[s] = fmaxf(rho[s] + d[s], 0.0f);
+        q[s] = r1[s] / rho[s];
     }
+    // an absent component keeps its populations, whatever the network says of the velocity
+    const bool present[2] = {rho[0] > 0.0f, rho[1] > 0.0f};
     const float2 q2 = make_float2(q[0], q[1]), r2 = make_float2(r1[0], r1[1]);
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
         const float c0 = cx(i) * ux + cy(i) * uy, c1 = cx(i) * vx + cy(i) * vy;
         const float dc = c1 - c0;
-        f[i] = fma2(q2, f[i], mul2(r2, splat(wf(i) * (3.0f * dc + 4.5f * dc * (c1 + c0) - du2))));
+        const float2 v = fma2(q2, f[i], mul2(r2, splat(wf(i) * (3.0f * dc + 4.5f * dc * (c1 + c0) - du2))));
+        f[i] = make_float2(present[0] ? v.x : f[i].x, present[1] ? v.y : f[i].y);
     }
 }
 
