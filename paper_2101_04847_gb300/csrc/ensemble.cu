@@ -246,7 +246,7 @@ lbm_status ens_time(lbm_ensemble* e, cudaEvent_t a, cudaEvent_t b, double* ms_pe
         if (err == cudaSuccess) err = cudaEventElapsedTime(&ms, a, b);
         if (err != cudaSuccess) break;
         *ms_per_step = ms / (replays * kTuneSteps);
-        if (ms > 1.0f) break;
+        if (ms > 0.2f) break;
     }
     cudaGraphExecDestroy(g);
     if (err != cudaSuccess) return ens_fail(LBM_ECUDA, std::string("timing: ") + cudaGetErrorString(err));
