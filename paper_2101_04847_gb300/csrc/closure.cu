@@ -292,12 +292,9 @@ weight_grad_kernel(const float* __restrict__ in, const float* __restrict__ dout,
             }
     }
     float* out = part + (size_t)blockIdx.x * K::kOut;
-    if (t < COUT * kWgH) {   // whole groups of four lanes
-        const unsigned mask = __activemask();
-        bias += __shfl_down_sync(mask, bias, 2, 4);
-        bias += __shfl_down_sync(mask, bias, 1, 4);
-        if (t % 4 == 0) out[COUT * CIN * 9 + t / 4] = bias;
-    }
+    bias += __shfl_down_sync(0xffffffffu, bias, 2, 4);
+    bias += __shfl_down_sync(0xffffffffu, bias, 1, 4);
+    if (t < COUT * kWgH && t % 4 == 0) out[COUT * CIN * 9 + t / 4] = bias;
     if constexpr (K::kGroups == 1) {
 #pragma unroll
         for (int o = 0; o < 4; ++o)
