@@ -75,7 +75,7 @@ typedef enum {
     LBM_KERNEL_DECOUPLED = 5,/* as STAGED (same tiles and row stages), but no block barrier per row: each warp
                               * keeps its own density ring, stages are handed back through per-stage barriers */
     LBM_KERNEL_PAIRED = 6    /* 16-bit storage only: as STAGED with 256-column tiles, each thread owning two
-                              * neighbouring columns (per-row work shared by two sites, paired 32-bit stores);
+                              * neighbouring columns (per-row work shared by two sites, paired 64-bit stores);
                               * what STAGED runs for 16-bit storage when tile_x is 0 and nx > 128 */
 } lbm_kernel;
 

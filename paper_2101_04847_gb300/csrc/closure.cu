@@ -28,7 +28,7 @@ constexpr int kW1 = 0, kB1 = kW1 + kHid * kIn * 9;
 constexpr int kW2 = kB1 + kHid, kB2 = kW2 + kHid * kHid * 9;
 constexpr int kW3 = kB2 + kHid, kB3 = kW3 + kOut * kHid * 9;
 constexpr int kParams = kB3 + kOut;   // 11588
-constexpr int kPartPixels = 512;      // pixels per weight-gradient partial, at least
+constexpr int kPartPixels = 512;      // pixels per weight-gradient partial (see grad_parts)
 
 static_assert(kParams == 11588, "parameter count");
 
@@ -195,9 +195,11 @@ void launch_conv(const float* in, const float* w, const float* b, const float* a
 // loads of 16 bytes.  Layers with 4 channels on one side split a row's pixels over 8
 // groups of threads.  The (o, c) pair per block it replaces read every input plane 32
 // times and loaded ten values for ten FMAs: 3460 us for the 32 -> 32 layer at 512x1024,
-// 226 now.  A partial covers at most a few hundred pixels and reduce_grad_kernel
-// adds them without rounding errors of its own: the gradient is 6e-8 off 64 bits at 512x1024,
-// 2.4e-7 before.
+// 226 now.  A partial covers 128 to a few hundred pixels, and more where kMaxParts limits
+// their number (about 5100 at 5000x2500), summed in FP32 by one thread or by 8 groups of
+// them; reduce_grad_kernel adds the partials without rounding errors of its own.  The last
+// layer's weight gradient is 3e-8 to 5e-8 of its largest value off 64 bits from 512x1024 to
+// 5000x2500; 6e-7 to 4e-6 before, with partials of 2048 pixels added in FP32.
 constexpr int kWgThreads = 128, kWgW = 32, kWgH = 4;
 constexpr int kWgRow = kWgW + 2;                               // staged columns of a row
 template <int CIN, int COUT> struct WgCfg {
@@ -414,7 +416,7 @@ struct Net {
 size_t align256(size_t v) { return (v + 255) / 256 * 256; }
 
 // Weight-gradient partials of an image: one per kPartPixels pixels, no more than
-// kMaxParts (92 MB of them); on small images one per tile, so that a block has one tile.
+// kMaxParts (90 MB of them); on small images one per tile, so that a block has one tile.
 constexpr size_t kMaxParts = 2432, kTileParts = 304, kPartFloats = kHid * kHid * 9 + kHid;
 size_t grad_parts(int nx, int ny) {
     const size_t n = (size_t)nx * ny;

@@ -726,7 +726,7 @@ cudaError_t launch_closure_input(const DiagLaunch& D, float* rho2, const float m
     return cudaGetLastError();
 }
 
-size_t diag_scratch_doubles(int nx, int ny) { return (size_t)15 * nx * ny; }
+size_t diag_scratch_doubles(int nx, int ny) { return diag_fields_offset(nx, ny) + (size_t)4 * nx * ny; }
 
 size_t diag_partials_doubles(int nx, int ny) {
     const size_t gx = sweep_tiles_x(nx), gy = sweep_tiles_y(nx, ny);

@@ -185,9 +185,6 @@ __device__ __forceinline__ void store_step(Cell<T>* __restrict__ fout, const Gri
 }
 
 // sum of nine values, associated as ((0+1)+(2+3)) + ((4+5)+(6+7)) + 8
-__device__ __forceinline__ float sum9(const float* f) {
-    return ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])) + f[8];
-}
 __device__ __forceinline__ float2 sum9_2(const float2* f) {
     const float2 lo = add2(add2(f[0], f[1]), add2(f[2], f[3]));
     const float2 hi = add2(add2(f[4], f[5]), add2(f[6], f[7]));

@@ -98,9 +98,9 @@ int row_columns(int nx) {
 Layout make_layout(const lbm_params& p) {
     Layout L;
     // column 0 sits 128 bytes into each row; the row leaves room for the staged
-    // kernels' windows (up to 144 columns from x0 - 10, x0 < nx; the 256-column tile's
-    // up to 8 columns past nx rounded up to 256) and the ghost copies.  No wider: wider
-    // rows measured slower.
+    // kernels' windows (at most 136 columns from at most 4 before x0, x0 < nx; the
+    // 256-column tile's up to 4 columns past nx rounded up to 256) and the ghost copies.
+    // No wider: wider rows measured slower.
     const size_t cell = 2 * elem_size(p.storage);
     L.origin = (int)(128 / cell);
     L.pitch = (L.origin + row_columns(p.nx) + 63) / 64 * 64;

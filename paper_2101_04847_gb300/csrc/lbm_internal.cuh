@@ -185,7 +185,7 @@ struct DiagLaunch {
     double G, G_wall[2], g_ext[2], gx, tau_bar;
     int crop;
     int wall_mirror;     // pseudopotential beyond the walls: 0 none, 1 the wall rows' (wall_mode)
-    double* scratch;     // 15 doubles per site
+    double* scratch;     // diag_scratch_doubles (fields only)
     double* partials;    // kDiagTerms * nblocks + 2 * ny * nbx
     double* out;         // kDiagTerms + 2 * ny doubles (terms, row sums of phi, of the mass fraction)
 };
@@ -196,7 +196,7 @@ size_t diag_partials_doubles(int nx, int ny);
 size_t diag_fields_offset(int nx, int ny);
 cudaError_t launch_diagnostics(const DiagLaunch& D, cudaStream_t st);
 // rho_A, rho_B, ux, uy (double [ny][nx] each) into the scratch region at
-// diag_fields_offset (uses the whole scratch: 15 doubles per site)
+// diag_fields_offset
 cudaError_t launch_fields(const DiagLaunch& D, double* fields, cudaStream_t st);
 // The closure's network input from the stored FP32 populations: rho_A, rho_B and the
 // physical velocity (j + F/2) / rho (the force from the neighbours' densities, as in the

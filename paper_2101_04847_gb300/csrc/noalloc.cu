@@ -36,10 +36,12 @@ __device__ __forceinline__ void load_pops(const float* __restrict__ S, size_t n,
 // holds post-streaming populations, so a row's densities are local sums and the next row's
 // loads are issued before row y collides.
 //
-// Bound by HBM (144 bytes per site) on large grids and by latency on small ones.  The two
-// launches it replaces, a density pass and one that collided, read the populations twice:
-// 25.1 us at 512x1024, 16.3 now (4.6 TB/s of the 144 bytes).  Loading row y + 2 ahead in a
-// third set of registers measured 15.1 there and 36.2 against 34.7 at 1024x1024.
+// Bound by latency: one launch and one wave of tiles of a few rows.  The two launches it
+// replaces, a density pass and one that collided, read the populations twice.  512x1024,
+// whose arrays (75 MB) fit in the L2: 25.1 us before and 16.3 now where they lie in it, 26.4
+// and 22.6 where they come from HBM (11.1 us for the 144 bytes per site at the copy rate).
+// Loading row y + 2 ahead in a third set of registers measured 15.1 against 16.3, and 36.2
+// against 34.7 at 1024x1024.
 __global__ void __launch_bounds__(kCols, 5)
 noalloc_step_kernel(const float* __restrict__ S, float* __restrict__ out, Physics ph, int nx, int ny) {
     __shared__ float2 sR[4][kCols + 2];

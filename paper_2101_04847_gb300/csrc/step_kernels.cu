@@ -488,8 +488,9 @@ step_pipe_kernel(const Cell<T>* __restrict__ fin, Cell<T>* __restrict__ fout, Gr
 // (one block barrier per row).
 //
 // What bounds it: FP32 is limited by HBM (0.97 of the copy rate at 10000x5000, 0.87 at
-// 1024x2048, where the ramp of each 51 us launch shows); 16-bit storage by instruction issue
-// (360 per site with the paired tile below).  Cells of both components halve the loads,
+// 1024x2048, where the ramp of each 51 us launch shows); 16-bit storage by its instructions
+// (360 per site with the paired tile below, 57 % of the issue slots: the pipes they share,
+// their latency and the row barriers with 16 warps per SM).  Cells of both components halve the loads,
 // stores and address arithmetic (FP32 492 -> 361 instructions per site although its tiles
 // went from 20 rows to 14, paired FP16 500 -> 360 at 16), a window of TW + 4 FP32 cells needs no alignment slack (34 sectors read per 32
 // owned at 128 columns, 36 before), and a tile whose sweep meets no wall row runs code without the wall
@@ -1398,11 +1399,14 @@ static cudaError_t block_slots(int* slots) {
 }
 
 // A launch that may start while the kernel before it on the stream drains (the kernels
-// call wait_previous_step), where that pays: for launches that leave room for the next
-// one's blocks (128x256 FP32 4.0 -> 3.5 us a step) and for those that fill the slots of
-// 128-thread blocks (512x1024 12.65 -> 12.26, 1024x2048 51.8 -> 51.0).  In between, blocks
-// that start early take the free slots of some SMs and leave the wave uneven (512x512, 684
-// blocks in 912 slots, 7.8 -> 8.2; 10000x5000, 280 in 304, 1103 -> 1131).
+// call wait_previous_step), where that pays.  us per step with plain and with early launches:
+// launches that leave room for the next one's blocks, 128x256 FP32 3.92 and 3.49; those
+// that fill the slots of 128-thread blocks, 512x1024 FP32 12.37 and 12.26, 1024x2048 FP32
+// 51.3 and 50.9, 1501x999 BF16 27.7 and 27.5, and in several waves 2048x4096 FP16 126.5 and
+// 126.0, 10000x5000 FP16 679 both ways.  In between, blocks that start early take the free
+// slots of some SMs and leave the wave uneven (512x512 FP32, 684 blocks in 912 slots, 7.82
+// and 8.24).  The 256-thread tile runs in several waves and measures the same either way
+// (6000x3000 407.8 and 407.3, 10000x5000 1093.3 and 1093.0): plain.
 template <typename... P, typename... A>
 static cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, int threads, size_t smem, int slots, cudaStream_t st,
                                     A... args) {

@@ -364,7 +364,8 @@ class _Member(Solver):
 
 
 class Ensemble:
-    """Independent realisations advanced together by one launch per time step."""
+    """Independent realisations advanced together: one launch per time step and chain, up to two
+    chains of members per storage type."""
 
     def __init__(self, members: list[LbmParams], stream=None):
         import torch
