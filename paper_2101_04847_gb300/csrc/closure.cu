@@ -18,6 +18,7 @@
 #include <algorithm>
 #include <cmath>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 namespace lbm {
@@ -268,29 +269,40 @@ weight_grad_kernel(const float* __restrict__ in, const float* __restrict__ dout,
             for (int q = 0; q < kWgW / 4; ++q) s += (g[q].x + g[q].y) + (g[q].z + g[q].w);
             bias += s;
         }
-#pragma unroll 1
-        for (int r = 0; r < kWgH; ++r)
-#pragma unroll 1
-            for (int q = group; q < kWgW / 4; q += K::kGroups) {
-                float4 g[4];
+        // four pixels of a row; kRagged: only those before column w of the tile
+        auto four = [&](auto ragged, int r, int q, int w) {
+            constexpr bool kRagged = decltype(ragged)::value;
+            float4 g[4];
 #pragma unroll
-                for (int o = 0; o < 4; ++o) g[o] = *reinterpret_cast<const float4*>(sg + ((4 * oq + o) * kWgH + r) * kWgW + 4 * q);
+            for (int o = 0; o < 4; ++o) g[o] = *reinterpret_cast<const float4*>(sg + ((4 * oq + o) * kWgH + r) * kWgW + 4 * q);
 #pragma unroll
-                for (int ky = 0; ky < 3; ++ky) {
-                    const float4* p = reinterpret_cast<const float4*>(si + cp * K::kPlane + (r + ky) * kWgRow + 4 * q);
-                    const float4 a = p[0], b = p[1], c = p[2];
-                    const float2 v[6] = {make_float2(a.x, a.y), make_float2(a.z, a.w), make_float2(b.x, b.y),
-                                         make_float2(b.z, b.w), make_float2(c.x, c.y), make_float2(c.z, c.w)};
+            for (int ky = 0; ky < 3; ++ky) {
+                const float4* p = reinterpret_cast<const float4*>(si + cp * K::kPlane + (r + ky) * kWgRow + 4 * q);
+                const float4 a = p[0], b = p[1], c = p[2];
+                const float2 v[6] = {make_float2(a.x, a.y), make_float2(a.z, a.w), make_float2(b.x, b.y),
+                                     make_float2(b.z, b.w), make_float2(c.x, c.y), make_float2(c.z, c.w)};
+#pragma unroll
+                for (int px = 0; px < 4; ++px) {
+                    if (kRagged && 4 * q + px >= w) break;
 #pragma unroll
                     for (int o = 0; o < 4; ++o) {
-                        const float go[4] = {g[o].x, g[o].y, g[o].z, g[o].w};
+                        const float go = px == 0 ? g[o].x : (px == 1 ? g[o].y : (px == 2 ? g[o].z : g[o].w));
 #pragma unroll
-                        for (int px = 0; px < 4; ++px)
-#pragma unroll
-                            for (int kx = 0; kx < 3; ++kx)
-                                acc[o][3 * ky + kx] = fma2(splat(go[px]), v[px + kx], acc[o][3 * ky + kx]);
+                        for (int kx = 0; kx < 3; ++kx)
+                            acc[o][3 * ky + kx] = fma2(splat(go), v[px + kx], acc[o][3 * ky + kx]);
                     }
                 }
+            }
+        };
+        // real pixels only: a zero gradient beyond the image times an input that is not
+        // finite would be no zero
+        const int w = min(kWgW, nx - bx), h = min(kWgH, ny - by);
+#pragma unroll 1
+        for (int r = 0; r < h; ++r)
+#pragma unroll 1
+            for (int q = group; 4 * q < w; q += K::kGroups) {
+                if (4 * q + 4 <= w) four(std::false_type(), r, q, w);
+                else four(std::true_type(), r, q, w);
             }
     }
     float* out = part + (size_t)blockIdx.x * K::kOut;
