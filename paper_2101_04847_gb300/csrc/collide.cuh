@@ -32,9 +32,12 @@ __device__ __forceinline__ bool velocity_and_accel(float2 rho, float2 jx, float2
                                                    const Physics& ph, int y, int ny, float& ux, float& uy, float2& ax,
                                                    float2& ay) {
     const bool ok = rho.x >= ph.rho_floor[0] && rho.y >= ph.rho_floor[1] && rho.x < 1e30f && rho.y < 1e30f;
-    const float inv = 1.0f / (rho.x * ph.om[0] + rho.y * ph.om[1]);
-    ux = (jx.x * ph.om[0] + jx.y * ph.om[1]) * inv;
-    uy = (jy.x * ph.om[0] + jy.y * ph.om[1]) * inv;
+    // one product rounded, the other one not: spelled out, because the compiler may take either
+    // and the results are not to depend on the kernel or the tile that a row falls into
+    auto weighted = [&](float2 v) { return fmaf(v.x, ph.om[0], __fmul_rn(v.y, ph.om[1])); };
+    const float inv = 1.0f / weighted(rho);
+    ux = weighted(jx) * inv;
+    uy = weighted(jy) * inv;
     float2 sx, sy;
     nbr_sum2(psi, sx, sy);
     ax = fma2(splat(-ph.G), sx, splat(ph.ax_ext));
